@@ -169,13 +169,13 @@ struct LaunchShape {
 // assembles Q/FLL into `out`. Precision: 0 = FP32 trace, 1 = FP64 trace.
 // ev (optional): two events recorded around the tracer kernel. index
 // (optional, device): launch seed j traces seed index[j] (FP64 retrace lists).
-// scratch (optional, device): 256 + end_record_bytes(precision) * 2 * n_seeds
-// bytes of caller memory; allocated per call when null.
+// scratch (optional, device): scratch_bytes(precision, 2 * n_seeds) bytes of
+// caller memory; allocated per call when null.
 int trace_and_assemble(const qsl_field* f, const SeedSource& src, int64_t n_seeds, const int64_t* n_seeds_dev,
                        const TraceConfig& cfg, int precision, const LaunchShape& shape, const LineOutputs& out,
                        cudaStream_t stream, DeviceStats* stats_dev, cudaEvent_t* ev, const int64_t* index = nullptr,
                        void* scratch = nullptr);
-size_t end_record_bytes(int precision);
+size_t scratch_bytes(int precision, size_t n_units);
 
 // Selects seeds whose chosen Q exceeds `threshold` (or is not finite while
 // L is) into `index` (device), count into count_dev (device).

@@ -468,6 +468,17 @@ struct Item {
   int64_t seed_start;          // global id of the item's first seed (outputs are concatenated in item order)
 };
 
+// State of an unfinished line direction handed from cell_kernel_f64 to
+// cell_wide_kernel, beside its end record (which holds the position offset in
+// x, the deviations in cell units, mu and the step count).
+struct Cont {
+  double muc;
+  int64_t unit;
+  int ic[3];
+  float h;
+  int zc, pad;
+};
+
 template <class R>
 struct TraceParams {
   Item<R> item0;               // the problem of a single-problem launch
@@ -485,6 +496,10 @@ struct TraceParams {
   int refill_min;
   unsigned long long timeout_ns;  // per-warp watchdog, 0 = none
   int* timeout_flag;
+  Cont* cont;                      // FP64 cell-wise launches: handed-over lines
+  unsigned long long* cont_count;
+  int handoff;                     // cell_kernel_f64: hand over a warp's lines at or below this many, 0 = never
+  int cont_in;                     // cell_wide_kernel: trace the handed-over lines
 };
 
 // Problem and seed of launch seed j: global id, item, position.
@@ -567,6 +582,10 @@ __device__ __forceinline__ unsigned long long globaltimer() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
+}
+
+__device__ __forceinline__ void prefetch_l1(const void* p) {
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
 template <class R, int NC, bool LOC>
@@ -1011,6 +1030,99 @@ __device__ __forceinline__ R y_at(R t, R dy, R hk1, R hk7, R c4) {
   return t * (dy + s1 * (bspl + t * (c3 + s1 * c4)));
 }
 
+// First crossing of a plane on the continuous extension (FP64). The offset
+// along the axis is t P(t), P(t) = dya + (1 - t) (bspl + t (c3 + (1 - t) c4));
+// the root sought is the first sign change of t P(t) - r (of P itself when the
+// step starts on the plane, r = 0: the root t = 0 divided out) over t = 1/4,
+// 1/2, 3/4, 1, and the result meets |f| <= 4 eps (|r| + |dya|).
+// cross_bracket is the safeguarded Newton iteration in the arithmetic R.
+template <class R>
+__device__ __forceinline__ R cross_f(R t, R r, R dya, R bspl, R c3, R c4, bool defl, R* df) {
+  const R s1 = R(1) - t;
+  const R inner = fma(s1, c4, c3);
+  const R mid = fma(t, inner, bspl);
+  const R pv = fma(s1, mid, dya);
+  if (df) {
+    const R dmid = inner - t * c4;
+    const R dp = fma(s1, dmid, -mid);
+    *df = defl ? dp : fma(t, dp, pv);
+  }
+  return defl ? pv : fma(t, pv, -r);
+}
+
+template <class R>
+__device__ __forceinline__ R cross_bracket(R r, R dya, R bspl, R c3, R c4, bool defl, R sg, R* ta_out, R* tb_out) {
+  R ta = R(0), tb = R(1);
+#pragma unroll
+  for (int q = 1; q < 4; ++q) {
+    const R tq = R(0.25) * R(q);
+    const R f = cross_f<R>(tq, r, dya, bspl, c3, c4, defl, (R*)nullptr);
+    if (sg * f > R(0) && tb == R(1)) tb = tq;
+    else if (tb == R(1)) ta = tq;
+  }
+  *ta_out = ta;
+  *tb_out = tb;
+  R t = ta + (tb - ta) * R(0.5);
+  if (!defl) {
+    const R tl = qdiv(r, dya);
+    if (tl > ta && tl < tb) t = tl;
+  }
+#pragma unroll 1
+  for (int it = 0; it < 30; ++it) {
+    R df;
+    const R f = cross_f<R>(t, r, dya, bspl, c3, c4, defl, &df);
+    if (fabs(f) <= R(4) * eps_of<R>() * (fabs(r) + fabs(dya)) || !(tb - ta > R(2) * eps_of<R>())) break;
+    if (sg * f > R(0)) tb = t;
+    else ta = t;
+    const R tn = t - qdiv(f, df);
+    t = (tn > ta && tn < tb) ? tn : R(0.5) * (ta + tb);
+  }
+  return t;
+}
+
+// x > thr for thr >= 0 and no NaN, and |x|'s order, on the bit patterns: an
+// FP64 comparison is an FP64-pipe instruction (64 cycles of a warp on GB300),
+// the integer one is not.
+__device__ __forceinline__ bool gt_bits(double x, double thr) {
+  return __double_as_longlong(x) > __double_as_longlong(thr);
+}
+
+// The search runs in FP32 (an FP64 instruction takes 64 cycles of a warp on
+// GB300 whether or not it depends on the one before, an FP32 one about 1 to
+// 5), then Newton corrections with an FP64 residual and the FP32 derivative
+// (each reduces the error by about 1e-6) reach the FP64 criterion. A root that
+// leaves the FP32 bracket or does not converge takes the FP64 iteration.
+__device__ __forceinline__ double cross_root(double r, double dya, double bspl, double c3, double c4, int up) {
+  const bool defl = (r == 0.0);
+  const float sg = up ? 1.0f : -1.0f;
+  const float rf = (float)r, df0 = (float)dya, bf = (float)bspl, c3f = (float)c3, c4f = (float)c4;
+  float taf, tbf;
+  float tf = cross_bracket<float>(rf, df0, bf, c3f, c4f, defl, sg, &taf, &tbf);
+  const float tol = 4.0f * (float)eps_of<double>() * (fabsf(rf) + fabsf(df0));
+  double t = (double)tf;
+  float last = 0.0f;
+  bool ok = false;
+#pragma unroll 1
+  for (int it = 0; it < 4; ++it) {
+    const float f = (float)cross_f<double>(t, r, dya, bspl, c3, c4, defl, (double*)nullptr);
+    ok = fabsf(f) <= tol;
+    if (ok) break;
+    float dff;
+    cross_f<float>(tf, rf, df0, bf, c3f, c4f, defl, &dff);
+    const float cor = __fdividef(f, dff);
+    t -= (double)cor;
+    tf -= cor;
+    // the corrections shrink by the factor just seen: the next one, not taken,
+    // would be below 1e-17 of the step
+    ok = it > 0 && fabsf(cor) <= 1e-3f * fabsf(last) && cor * cor <= 1e-17f * fabsf(last);
+    if (ok) break;
+    last = cor;
+  }
+  if (ok && tf > 0.0f && tf <= 1.0f && tf >= taf - 1e-5f && tf <= tbf + 1e-5f) return t;
+  double ta, tb;
+  return cross_bracket<double>(r, dya, bspl, c3, c4, defl, (double)sg, &ta, &tb);
+}
+
 // Right-hand side inside one cell: the 24 corner values (3 components x 8
 // corners, corner c = x + 2y + 4z) sit in shared memory with a stride of one
 // block; (u, v, w) are the in-cell coordinates (may lie slightly outside
@@ -1077,6 +1189,14 @@ __device__ __forceinline__ void trilinear_coeffs(const R* cv, R ihc, R* a) {
   a[7] = (((cv[7] - cv[6]) - (cv[5] - cv[4])) - ((cv[3] - cv[2]) - (cv[1] - cv[0]))) * ihc;
 }
 
+// 1 / |B| from |B|^2, 0 for a null field (FP64 by rsqrt_fp64: half the FP64
+// instructions of the square root and division).
+__device__ __forceinline__ float rcp_norm(float m2) {
+  const float m = sqrt(m2);
+  return (m > 0.0f) ? 1.0f / m : 0.0f;
+}
+__device__ __forceinline__ double rcp_norm(double m2) { return rsqrt_fp64(m2); }
+
 // Right-hand side inside one cell from the coefficients of the cell's
 // trilinear polynomials (8 per component c, corner form turned into
 // a0 + a1 u + a2 v + a3 w + a4 uv + a5 uw + a6 vw + a7 uvw once per cell entry),
@@ -1124,8 +1244,7 @@ __device__ __forceinline__ void cell_rhs_poly(const typename C4<R>::type* __rest
           k[3 + 3 * v2 + i] = fma(d[i][0], y[3 + 3 * v2], fma(d[i][1], y[4 + 3 * v2], d[i][2] * y[5 + 3 * v2]));
     }
   } else {
-    const R m = sqrt(val[0] * val[0] + val[1] * val[1] + val[2] * val[2]);
-    const R rm = (m > R(0)) ? R(1) / m : R(0);
+    const R rm = rcp_norm(val[0] * val[0] + val[1] * val[1] + val[2] * val[2]);
     R b[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) b[c] = val[c] * rm;
@@ -1164,6 +1283,7 @@ __device__ __forceinline__ void dev_to_domain(R* y, const R* hh3) {
 
 template <class R, int NC>
 __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
+  constexpr bool F64 = sizeof(R) == 8;
   extern __shared__ __align__(32) unsigned char smem_raw[];
   typedef typename C4<R>::type CV;
   const int st = blockDim.x;
@@ -1197,6 +1317,11 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
   int ic[3] = {0, 0, 0};
   R mu = 0, muc = 0, h = 0, sgn = 1;
   int steps = 0, zc = 0;
+  // FP64: the step controller's FP32 copies of the line's scales, and the
+  // cells beyond which a domain bound comes before the cell's own face
+  float hcf[3] = {1.0f, 1.0f, 1.0f}, orgf[3] = {0.0f, 0.0f, 0.0f}, hF = 0.0f, tinyF = 0.0f, hmaxF = 0.0f;
+  const float tolaF = (float)P.tol_abs, tolrF = (float)P.tol_rel;
+  int ilo[3] = {0, 0, 0}, ihi[3] = {0, 0, 0};
   unsigned long long c_stage = 0, c_acc = 0, c_rej = 0, c_land = 0, c_lines = 0;
   int iter = 0;
   bool timed_out = false;
@@ -1228,6 +1353,18 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
               hh3[a] = R(1) / ih[a];
             }
             tiny = R(1e-4) * E->h_max;
+            if constexpr (F64) {
+#pragma unroll
+              for (int a = 0; a < 3; ++a) {
+                hcf[a] = (float)hh3[a];
+                orgf[a] = (float)E->F.org[a];
+                ilo[a] = (int)floor(E->lo[a]);
+                ihi[a] = (int)ceil(E->hi[a]) - 1;
+              }
+              tinyF = (float)tiny;
+              hmaxF = (float)E->h_max;
+              hF = (float)E->h_init;
+            }
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
               double fa = (xd[a] - E->org_d[a]) * E->inv_h_d[a];
@@ -1304,6 +1441,37 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
         }
       }
     }
+    if constexpr (F64 && NC == 9) {
+      // the queue is empty and few lanes of this warp still have a line: the
+      // rest of those lines goes to cell_wide_kernel, sixteen lanes each
+      if (exhausted && P.handoff > 0) {
+        const unsigned am = __ballot_sync(FULL, active);
+        const int na = __popc(am);
+        if (na > 0 && na <= P.handoff && !__any_sync(FULL, timed_out)) {
+          unsigned long long base = 0;
+          if (lane == __ffs(am) - 1) base = atomicAdd(P.cont_count, (unsigned long long)na);
+          base = __shfl_sync(FULL, base, __ffs(am) - 1);
+          if (active) {
+            Cont& k = P.cont[base + __popc(am & lt_mask)];
+            EndRec<R>& e = P.ends[unit];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+              e.x[a] = y[a];
+              e.d1[a] = y[3 + a];
+              e.d2[a] = y[6 + a];
+              k.ic[a] = ic[a];
+            }
+            e.mu = mu;
+            e.steps = steps;
+            k.muc = muc;
+            k.unit = unit;
+            k.h = hF;
+            k.zc = zc;
+            active = false;
+          }
+        }
+      }
+    }
     if (!__any_sync(FULL, active)) {
       if (exhausted) break;
       continue;
@@ -1317,7 +1485,7 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
     if (timed_out) status = QSL_LINE_TIMEOUT;
     if (status == ST_RUNNING && steps >= P.max_steps) status = QSL_LINE_MAXSTEPS;
     R room = E->max_len - mu;
-    if (status == ST_RUNNING && !(room > R(0))) status = QSL_LINE_MAXLEN;
+    if (status == ST_RUNNING && !(F64 ? gt_bits(room, 0.0) : room > R(0))) status = QSL_LINE_MAXLEN;
     if (status == ST_RUNNING) {
       if (!kvalid) {
         // gather the 8 vertices of the current cell once; every stage of the
@@ -1359,28 +1527,65 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
       // planes of this cell (cell faces, or domain faces where they come first)
       R lo_pl[3], hi_pl[3];
       bool lo_dom[3], hi_dom[3];
+      R hs;
+      bool capped;
+      float hsF = 0.0f;
+      if constexpr (F64) {
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        R lr = E->lo[a] - R(ic[a]), hr = E->hi[a] - R(ic[a]);
-        lo_dom[a] = lr >= R(0);
-        hi_dom[a] = hr <= R(1);
-        lo_pl[a] = lo_dom[a] ? lr : R(0);
-        hi_pl[a] = hi_dom[a] ? hr : R(1);
-      }
-      // step: controller size, capped a little beyond the first plane along k1
-      R tface = R(1e30);
+        for (int a = 0; a < 3; ++a) {
+          lo_dom[a] = ic[a] <= ilo[a];
+          hi_dom[a] = ic[a] >= ihi[a];
+          lo_pl[a] = R(0);
+          hi_pl[a] = R(1);
+          if (lo_dom[a]) lo_pl[a] = E->lo[a] - R(ic[a]);
+          if (hi_dom[a]) hi_pl[a] = E->hi[a] - R(ic[a]);
+        }
+        float tfc = 1e30f;
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        R vel = sgn * k1[a];
-        if (vel > R(0)) tface = fmin(tface, qdiv(hi_pl[a] - y[a], vel));
-        else if (vel < R(0)) tface = fmin(tface, qdiv(lo_pl[a] - y[a], vel));
-      }
-      R hs = fmin(fmin(h, E->h_max), room);
-      bool capped = room <= fmin(h, E->h_max);
-      R hf = R(1.25) * fmax(tface, R(0)) + tiny;
-      if (hf < hs) {
-        hs = hf;
-        capped = false;
+        for (int a = 0; a < 3; ++a) {
+          const float vel = (float)(sgn * k1[a]);
+          if (vel != 0.0f) tfc = fminf(tfc, __fdividef((float)((vel > 0.0f ? hi_pl[a] : lo_pl[a]) - y[a]), vel));
+        }
+        const float hcap = fminf(hF, hmaxF);
+        const float hfF = 1.25f * fmaxf(tfc, 0.0f) + tinyF;
+        if ((float)room > 1.001f * hcap) {
+          capped = false;
+          hs = (R)hcap;
+          hsF = hcap;
+        } else {  // near the maximum length: the cap in FP64
+          capped = room <= (R)hcap;
+          hs = capped ? room : (R)hcap;
+          hsF = (float)hs;
+        }
+        if (hfF < hsF) {
+          hsF = hfF;
+          hs = (R)hfF;
+          capped = false;
+        }
+      } else {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          R lr = E->lo[a] - R(ic[a]), hr = E->hi[a] - R(ic[a]);
+          lo_dom[a] = lr >= R(0);
+          hi_dom[a] = hr <= R(1);
+          lo_pl[a] = lo_dom[a] ? lr : R(0);
+          hi_pl[a] = hi_dom[a] ? hr : R(1);
+        }
+        // step: controller size, capped a little beyond the first plane along k1
+        R tface = R(1e30);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          R vel = sgn * k1[a];
+          if (vel > R(0)) tface = fmin(tface, qdiv(hi_pl[a] - y[a], vel));
+          else if (vel < R(0)) tface = fmin(tface, qdiv(lo_pl[a] - y[a], vel));
+        }
+        hs = fmin(fmin(h, E->h_max), room);
+        capped = room <= fmin(h, E->h_max);
+        R hf = R(1.25) * fmax(tface, R(0)) + tiny;
+        if (hf < hs) {
+          hs = hf;
+          capped = false;
+        }
       }
       R hh = sgn * hs;
       // stage combinations with the step folded into the coefficients; each
@@ -1421,34 +1626,59 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
       const R w1 = hh * R(DD1), w3 = hh * R(DD3), w4 = hh * R(DD4), w5 = hh * R(DD5), w6 = hh * R(DD6),
               w7 = hh * R(DD7);
       R err = 0;
+      float errf = 0.0f;
       bool finite = true;
+      if constexpr (F64) {
+        // the error estimate in FP64, its norm and the step controller in FP32:
+        // they only size the next step, and their divisions, comparisons and
+        // power were a third of a step's FP64 instructions
 #pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        R e = fabs(fma(e7, k7[i], fma(e6, k6[i], fma(e5, k5[i], fma(e4, k4[i], fma(e3, k3[i], e1 * k1[i]))))));
-        if (!isfinite(t[i])) finite = false;
-        R ya, yb;
-        if (i < 3) {
-          R base = R(E->F.org[i]) + R(ic[i]) * hh3[i];
-          e *= hh3[i];
-          ya = fabs(base + y[i] * hh3[i]);
-          yb = fabs(base + t[i] * hh3[i]);
-        } else {  // deviations, in domain units
-          const R hc = hh3[i % 3];
-          e *= hc;
-          ya = fabs(y[i]) * hc;
-          yb = fabs(t[i]) * hc;
+        for (int i = 0; i < NC; ++i) {
+          const float hc = hcf[i % 3];
+          const float e =
+              fabsf((float)fma(e7, k7[i], fma(e6, k6[i], fma(e5, k5[i], fma(e4, k4[i], fma(e3, k3[i], e1 * k1[i])))))) * hc;
+          if ((__double2hiint(t[i]) & 0x7ff00000) == 0x7ff00000) finite = false;
+          const float base = i < 3 ? fmaf((float)ic[i], hc, orgf[i]) : 0.0f;
+          const float m = fmaxf(fabsf(fmaf((float)y[i], hc, base)), fabsf(fmaf((float)t[i], hc, base)));
+          errf = fmaxf(errf, __fdividef(e, fmaf(tolrF, m, tolaF)));
         }
-        err = fmax(err, cdiv(e, P.tol_abs + P.tol_rel * fmax(ya, yb)));
+      } else {
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+          R e = fabs(fma(e7, k7[i], fma(e6, k6[i], fma(e5, k5[i], fma(e4, k4[i], fma(e3, k3[i], e1 * k1[i]))))));
+          if (!isfinite(t[i])) finite = false;
+          R ya, yb;
+          if (i < 3) {
+            R base = R(E->F.org[i]) + R(ic[i]) * hh3[i];
+            e *= hh3[i];
+            ya = fabs(base + y[i] * hh3[i]);
+            yb = fabs(base + t[i] * hh3[i]);
+          } else {  // deviations, in domain units
+            const R hc = hh3[i % 3];
+            e *= hc;
+            ya = fabs(y[i]) * hc;
+            yb = fabs(t[i]) * hc;
+          }
+          err = fmax(err, cdiv(e, P.tol_abs + P.tol_rel * fmax(ya, yb)));
+        }
       }
       if (!finite) {
         status = QSL_LINE_NONFINITE;
-      } else if (err > R(1)) {
+      } else if (F64 ? errf > 1.0f : err > R(1)) {
         c_rej += 1;
-        h = hs * fmax(R(0.2), R(0.9) * cpow(err, R(-0.25)));
-        if (h < E->h_min) status = QSL_LINE_STALL;
+        if constexpr (F64) {
+          hF = hsF * fmaxf(0.2f, 0.9f * __powf(errf, -0.25f));
+          if (hF < (float)E->h_min) status = QSL_LINE_STALL;
+        } else {
+          h = hs * fmax(R(0.2), R(0.9) * cpow(err, R(-0.25)));
+          if (h < E->h_min) status = QSL_LINE_STALL;
+        }
       } else {
         c_acc += 1;
-        R hnext = hs * ((err == R(0)) ? R(5) : fmin(R(5), R(0.9) * cpow(err, R(-0.2))));
+        R hnext = R(0);
+        float hnextF = 0.0f;
+        if constexpr (F64) hnextF = hsF * ((errf == 0.0f) ? 5.0f : fminf(5.0f, 0.9f * __powf(errf, -0.2f)));
+        else hnext = hs * ((err == R(0)) ? R(5) : fmin(R(5), R(0.9) * cpow(err, R(-0.2))));
         // First plane crossed within the step, on the dense output (4th-order
         // continuous extension): for every plane the step ends beyond, the
         // first sign change of dense(t) - plane over t = 1/4, 1/2, 3/4, 1
@@ -1460,8 +1690,13 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
         unsigned cmask = 0;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-          if ((lo_pl[a] - y[a]) - dy[a] > (lo_dom[a] ? R(0) : band)) cmask |= 1u << (2 * a);
-          if (dy[a] - (hi_pl[a] - y[a]) > (hi_dom[a] ? R(0) : band)) cmask |= 2u << (2 * a);
+          if constexpr (F64) {
+            if (gt_bits((lo_pl[a] - y[a]) - dy[a], lo_dom[a] ? R(0) : band)) cmask |= 1u << (2 * a);
+            if (gt_bits(dy[a] - (hi_pl[a] - y[a]), hi_dom[a] ? R(0) : band)) cmask |= 2u << (2 * a);
+          } else {
+            if ((lo_pl[a] - y[a]) - dy[a] > (lo_dom[a] ? R(0) : band)) cmask |= 1u << (2 * a);
+            if (dy[a] - (hi_pl[a] - y[a]) > (hi_dom[a] ? R(0) : band)) cmask |= 2u << (2 * a);
+          }
         }
 #pragma unroll 1
         while (cmask) {
@@ -1480,45 +1715,50 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
                  fma(w4, sel3(a, k4[0], k4[1], k4[2]), fma(w3, sel3(a, k3[0], k3[1], k3[2]), w1 * k1a)))));
           R bspl = hh * k1a - dya;
           R c3 = dya - hh * k7a - bspl;
-          // The offset along the axis is t * P(t) with the cubic
-          // P(t) = dya + (1 - t) (bspl + t (c3 + (1 - t) c4)). A step that
-          // starts on the plane (r = 0: a seed on a domain face, or the face
-          // just entered) has the trivial root t = 0; the crossing sought is
-          // the root of P, so P is solved instead (the root t = 0 divided out).
-          const bool defl = (r == R(0));
-          // bracket the first crossing
-          R ta = R(0), tb = R(1);
+          R t;
+          if constexpr (sizeof(R) == 8) {
+            t = cross_root(r, dya, bspl, c3, c4, up);
+          } else {
+            // The offset along the axis is t * P(t) with the cubic
+            // P(t) = dya + (1 - t) (bspl + t (c3 + (1 - t) c4)). A step that
+            // starts on the plane (r = 0: a seed on a domain face, or the face
+            // just entered) has the trivial root t = 0; the crossing sought is
+            // the root of P, so P is solved instead (the root t = 0 divided out).
+            const bool defl = (r == R(0));
+            // bracket the first crossing
+            R ta = R(0), tb = R(1);
 #pragma unroll
-          for (int q = 1; q < 4; ++q) {
-            R tq = R(0.25) * R(q);
-            R s1 = R(1) - tq;
-            R pq = dya + s1 * (bspl + tq * (c3 + s1 * c4));
-            R f = defl ? pq : tq * pq - r;
-            if (sg * f > R(0) && tb == R(1)) tb = tq;
-            else if (tb == R(1)) ta = tq;
+            for (int q = 1; q < 4; ++q) {
+              R tq = R(0.25) * R(q);
+              R s1 = R(1) - tq;
+              R pq = dya + s1 * (bspl + tq * (c3 + s1 * c4));
+              R f = defl ? pq : tq * pq - r;
+              if (sg * f > R(0) && tb == R(1)) tb = tq;
+              else if (tb == R(1)) ta = tq;
+            }
+            t = ta + (tb - ta) * R(0.5);
+            if (!defl) {
+              // chord estimate inside the bracket as the first iterate
+              R tl = qdiv(r, dya);
+              if (tl > ta && tl < tb) t = tl;
+            }
+            for (int it = 0; it < 30; ++it) {
+              R s1 = R(1) - t;
+              R inner = c3 + s1 * c4;
+              R mid = bspl + t * inner;
+              R pv = dya + s1 * mid;
+              R f = defl ? pv : t * pv - r;
+              if (fabs(f) <= R(4) * eps_of<R>() * (fabs(r) + fabs(dya)) || !(tb - ta > R(2) * eps_of<R>())) break;
+              if (sg * f > R(0)) tb = t;
+              else ta = t;
+              R dmid = inner - t * c4;
+              R dp = s1 * dmid - mid;
+              R df = defl ? dp : pv + t * dp;
+              R tn = t - qdiv(f, df);
+              t = (tn > ta && tn < tb) ? tn : R(0.5) * (ta + tb);
+            }
           }
-          R t = ta + (tb - ta) * R(0.5);
-          if (!defl) {
-            // chord estimate inside the bracket as the first iterate
-            R tl = qdiv(r, dya);
-            if (tl > ta && tl < tb) t = tl;
-          }
-          for (int it = 0; it < 30; ++it) {
-            R s1 = R(1) - t;
-            R inner = c3 + s1 * c4;
-            R mid = bspl + t * inner;
-            R pv = dya + s1 * mid;
-            R f = defl ? pv : t * pv - r;
-            if (fabs(f) <= R(4) * eps_of<R>() * (fabs(r) + fabs(dya)) || !(tb - ta > R(2) * eps_of<R>())) break;
-            if (sg * f > R(0)) tb = t;
-            else ta = t;
-            R dmid = inner - t * c4;
-            R dp = s1 * dmid - mid;
-            R df = defl ? dp : pv + t * dp;
-            R tn = t - qdiv(f, df);
-            t = (tn > ta && tn < tb) ? tn : R(0.5) * (ta + tb);
-          }
-          if (t < th) {
+          if (F64 ? gt_bits(th, t) : t < th) {
             th = t;
             ax_c = a;
             up_c = up;
@@ -1534,15 +1774,29 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
           R t1 = hs - muc, t2 = mu + t1;
           muc = (t2 - mu) - t1;
           mu = t2;
-          h = hnext;
+          if constexpr (F64) hF = hnextF;
+          else h = hnext;
           zc = 0;
           if (capped) status = QSL_LINE_MAXLEN;
         } else {
           // advance to the plane on the dense output and snap onto it
+          if constexpr (F64) {
+            // y_at's increment as one sum over the stages (its weights formed
+            // once, 7 FP64 instructions per component against 17)
+            const R s1 = R(1) - th, st_ = s1 * th;
+            const R ad = th * fma(R(2), st_, th), d4 = th * (s1 * st_);
+            const R g1 = fma(d4, w1, hh * (th * (s1 * s1))), g7 = fma(d4, w7, -(hh * (th * st_)));
+            const R g3 = d4 * w3, g4 = d4 * w4, g5 = d4 * w5, g6 = d4 * w6;
+#pragma unroll
+            for (int i = 0; i < NC; ++i)
+              y[i] = fma(ad, dy[i], fma(g7, k7[i], fma(g6, k6[i], fma(g5, k5[i], fma(g4, k4[i], fma(g3, k3[i],
+                     fma(g1, k1[i], y[i])))))));
+          } else {
 #pragma unroll
           for (int i = 0; i < NC; ++i)
             y[i] += y_at<R>(th, dy[i], hh * k1[i], hh * k7[i],
                             fma(w7, k7[i], fma(w6, k6[i], fma(w5, k5[i], fma(w4, k4[i], fma(w3, k3[i], w1 * k1[i]))))));
+          }
           bool dom = up_c ? sel3(ax_c, hi_dom[0], hi_dom[1], hi_dom[2]) : sel3(ax_c, lo_dom[0], lo_dom[1], lo_dom[2]);
           R target = up_c ? sel3(ax_c, hi_pl[0], hi_pl[1], hi_pl[2]) : sel3(ax_c, lo_pl[0], lo_pl[1], lo_pl[2]);
           if (ax_c == 0) y[0] = target;
@@ -1558,7 +1812,7 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
             lface = 2 * ax_c + up_c;
           } else {
             // enter the neighbouring cell
-            zc = (dl < tiny) ? zc + 1 : 0;
+            zc = (F64 ? (float)dl < tinyF : dl < tiny) ? zc + 1 : 0;
             int na = sel3(ax_c, ic[0], ic[1], ic[2]) + (up_c ? 1 : -1);
             if (zc > 3 || na < 0 || na > sel3(ax_c, E->F.n[0], E->F.n[1], E->F.n[2]) - 2) {
               // grazing a face back and forth: stay in this cell for one step
@@ -1573,7 +1827,8 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
               else y[2] = up_c ? R(0) : R(1);
               kvalid = false;
             }
-            h = fmax(hnext, hs);
+            if constexpr (F64) hF = fmaxf(hnextF, hsF);
+            else h = fmax(hnext, hs);
           }
         }
       }
@@ -1604,7 +1859,11 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
   if (lane == 0 && any_to && P.timeout_flag) atomicExch(P.timeout_flag, 1);
 }
 
-// The cell-wise kernel. FP32: at most 168 registers, so three blocks of 128
+// The cell-wise kernel. FP64 is bound by the FP64 pipe (19 cycles per SM and
+// warp instruction): with the controller, the plane tests and the crossing
+// search off it, about 1,000 FP64 instructions per warp step against 1,800
+// (FP64 map of 82,497 seeds on 128^3: 45.0 -> 29.6 ms, with the hand-over of
+// the last lines 20.6 ms). FP32: at most 168 registers, so three blocks of 128
 // threads stay resident per SM (the allocation granularity would make 170 a
 // two-block kernel); FP64 keeps the compiler's choice (a cap would spill).
 template <int NC>
@@ -2116,6 +2375,472 @@ __global__ void __launch_bounds__(256) cell_coop_kernel(const __grid_constant__ 
     if (any_to) atomicAdd(&P.stats->timeouts, 1ull);
   }
   if (lane == 0 && any_to && P.timeout_flag) atomicExch(P.timeout_flag, 1);
+}
+
+// ------------------------------------------------------------ FP64 tracer with a lane per component
+// The cell-wise Dormand-Prince tracer in FP64 for few to moderately many lines
+// (the retrace of lines above retrace_q, FP64 maps of ordinary size): such a
+// launch lasts about as long as its longest line, and on GB300 every FP64 warp
+// instruction (add, multiply, FMA, comparison, conversion alike) takes 64
+// cycles of its warp whatever the number of active lanes and whether or not it
+// depends on the one before (measured; 19 cycles per SM with all four
+// schedulers busy). A line's time is therefore its count of FP64 warp
+// instructions, so a line is spread over 16 lanes until each does the work of
+// one component. Lane 4c + j of a group: axis c; j = 0 the position x_c,
+// j = 1, 2 component c of deviation j, j = 3 no state. For a stage derivative
+// it evaluates, as one bilinear polynomial (3 FMAs), d b_c / d u_j for j < 3
+// and b_c on the cell's lower x face for j = 3; three more FMAs after shuffles
+// give value or gradient times deviation. Lanes 12..15 repeat lanes 8..11.
+// Comparisons use bit patterns; the step controller, the error norm and the
+// crossing search FP32 (cross_root), as in cell_trace. Deviations are carried
+// in cell units. One line per warp while there are warps (the first lines go
+// to one warp per SM, then to the other schedulers), else two; three lines of
+// ten lanes per warp, one more polynomial in the position lanes, measured no
+// faster (29.5 against 29.9 ms for 165 k line directions).
+// About 165 FP64 instructions per step against 865 of the three-lane kernel it
+// replaced: 7.0 against 25.6 us per step of a lone line; 64 seeds of a map on
+// 128^3 1.6 ms (6.8 ms on one lane per line).
+// End record of a group: lane (c, j) writes axis c of the end
+// point (j = 0) or of deviation j, the group's first lane the rest.
+__device__ __forceinline__ void write_end_wide(const TraceParams<double>& P, const Item<double>* E, int64_t unit,
+                                               int c, int j, bool writer, double y, const int* ic, double hhc,
+                                               double mu, int face, int status, int steps) {
+  EndRec<double>& e = P.ends[unit];
+  if (!writer) return;
+  if (j == 0) {
+    double xv = E->org_d[c] + ((double)sel3(c, ic[0], ic[1], ic[2]) + y) * E->h_d[c];
+    if (status == QSL_LINE_OK && face != NO_FACE && (face >> 1) == c)
+      xv = (face & 1) ? E->hi_d[c] : E->lo_d[c];  // exactly on the face
+    e.x[c] = xv;
+    if (c == 0) {
+      e.mu = mu;
+      e.face = (status == QSL_LINE_OK) ? face : NO_FACE;
+      e.status = status;
+      e.steps = steps;
+    }
+  } else if (j == 1) {
+    e.d1[c] = y * hhc;
+  } else {
+    e.d2[c] = y * hhc;
+  }
+}
+
+// Launch counters: one atomic per warp and counter.
+template <class R>
+__device__ __forceinline__ void write_stats(const TraceParams<R>& P, int lane, unsigned long long c_stage,
+                                            unsigned long long c_acc, unsigned long long c_rej,
+                                            unsigned long long c_land, unsigned long long c_lines, bool timed_out) {
+  const unsigned FULL = 0xffffffffu;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    c_stage += __shfl_down_sync(FULL, c_stage, o);
+    c_acc += __shfl_down_sync(FULL, c_acc, o);
+    c_rej += __shfl_down_sync(FULL, c_rej, o);
+    c_land += __shfl_down_sync(FULL, c_land, o);
+    c_lines += __shfl_down_sync(FULL, c_lines, o);
+  }
+  const unsigned any_to = __ballot_sync(FULL, timed_out);
+  if (lane == 0 && P.stats) {
+    atomicAdd(&P.stats->stage_evals, c_stage);
+    atomicAdd(&P.stats->accepted, c_acc);
+    atomicAdd(&P.stats->rejected, c_rej);
+    atomicAdd(&P.stats->landing, c_land);
+    atomicAdd(&P.stats->lines, c_lines);
+    if (any_to) atomicAdd(&P.stats->timeouts, 1ull);
+  }
+  if (lane == 0 && any_to && P.timeout_flag) atomicExch(P.timeout_flag, 1);
+}
+
+__device__ __forceinline__ double gsh(unsigned gm, double v, int src) { return __shfl_sync(gm, v, src); }
+
+struct WideLane {
+  unsigned gm;       // the group's lanes
+  int gb;            // its first lane
+  int c, j;          // axis and role of the lane
+  int s_src, t_src;  // lanes holding the lane's two bilinear coordinates
+  int p1_src;        // lane of the second factor of the product sum
+  __device__ __forceinline__ int pos(int a) const { return gb + 4 * a; }  // position lane of axis a
+};
+
+// Stage derivative of the lane's component at the stage state t (co: the
+// lane's bilinear coefficients).
+__device__ __forceinline__ double wide_rhs(const WideLane& W, const double* co, bool raw, double ihc, double t) {
+  const double s = gsh(W.gm, t, W.s_src), w = gsh(W.gm, t, W.t_src);
+  double z0 = gsh(W.gm, t, W.pos(0) + W.j), z1 = gsh(W.gm, t, W.pos(1) + W.j), z2 = gsh(W.gm, t, W.pos(2) + W.j);
+  const double q = fma(fma(co[3], s, co[2]), w, fma(co[1], s, co[0]));
+  const double p0 = gsh(W.gm, q, W.pos(W.c)), p1 = gsh(W.gm, q, W.p1_src), p2 = gsh(W.gm, q, W.pos(W.c) + 2);
+  if (W.j == 0) {  // value = u d0 + (value on the lower x face)
+    z1 = 1.0;
+    z2 = 0.0;
+  }
+  const double g = fma(p0, z0, fma(p1, z1, p2 * z2));
+  if (!raw) return g;
+  // raw fields: b = B / |B|, grad b = (I - b b^T) grad B / |B|
+  const double val = gsh(W.gm, g, W.pos(W.c));
+  const double v0 = gsh(W.gm, val, W.pos(0)), v1 = gsh(W.gm, val, W.pos(1)), v2 = gsh(W.gm, val, W.pos(2));
+  const double rm = rcp_norm(fma(v0, v0, fma(v1, v1, v2 * v2)));
+  const double b = val * rm;
+  const double bg = b * g;
+  const double bs = gsh(W.gm, bg, W.pos(0) + W.j) + gsh(W.gm, bg, W.pos(1) + W.j) + gsh(W.gm, bg, W.pos(2) + W.j);
+  return W.j == 0 ? b * ihc : (ihc * rm) * fma(-b, bs, g);
+}
+
+__global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ TraceParams<double> P, int sms) {
+  typedef double R;
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int l = lane & 15;
+  WideLane W;
+  W.gb = lane & 16;
+  W.gm = 0xffffu << W.gb;
+  W.c = min(l >> 2, 2);
+  W.j = l & 3;
+  W.s_src = (W.j == 0 || W.j == 3) ? W.pos(1) : W.pos(0);
+  W.t_src = W.j == 2 ? W.pos(1) : W.pos(2);
+  W.p1_src = W.pos(W.c) + (W.j == 0 ? 3 : 1);
+  const int c = W.c, j = W.j;
+  const bool lead = l == 0, writer = l < 12 && j < 3;
+  int64_t total = P.n_units;
+  if (P.n_seeds_dev) {
+    int64_t cnt = 2 * (*P.n_seeds_dev);
+    total = cnt < total ? cnt : total;
+  }
+  if (P.cont_in) total = (int64_t)*P.cont_count;
+  const int wpb = blockDim.x >> 5;
+  const int64_t warps_total = (int64_t)gridDim.x * wpb;
+  // rank of this warp: first warps of the first `sms` blocks, their second warps, ...
+  const int64_t wave = blockIdx.x / sms, in_wave = blockIdx.x % sms;
+  const int64_t nb = min((int64_t)sms, (int64_t)gridDim.x - wave * sms);
+  const int64_t rank = wave * sms * wpb + (int64_t)(threadIdx.x >> 5) * nb + in_wave;
+  if (rank >= total) return;
+  const bool usable = total > warps_total || W.gb == 0;
+  const Item<R>* E = &P.item0;
+
+  bool active = false, exhausted = false, kvalid = false;
+  int64_t unit = 0;
+  R y = 0, k1 = 0, co[4] = {0, 0, 0, 0};
+  R lo_pl = 0, hi_pl = 0, ihc = 1, hhc = 1;
+  bool lo_dom = false, hi_dom = false, raw = false;
+  int ic[3] = {0, 0, 0};
+  R mu = 0, muc = 0, sgn = 1, max_len = 0;
+  float h = 0, h_max = 0, h_min = 0, tiny = 0, hcf = 0, orgf = 0;
+  const float tola = (float)P.tol_abs, tolr = (float)P.tol_rel;
+  int ilo = 0, ihi = 0;
+  int steps = 0, zc = 0;
+  unsigned long long c_stage = 0, c_acc = 0, c_rej = 0, c_land = 0, c_lines = 0;
+  int iter = 0;
+  bool timed_out = false;
+  const unsigned long long t_start = P.timeout_ns ? globaltimer() : 0ull;
+
+  for (;;) {
+    if (!exhausted) {
+      const unsigned need = __ballot_sync(FULL, usable && lead && !active);
+      const int nneed = __popc(need);
+      if (nneed > 0) {
+        const int leader = __ffs(need) - 1;
+        unsigned long long base = 0;
+        if (lane == leader) base = atomicAdd(P.head, (unsigned long long)nneed);
+        base = __shfl_sync(FULL, base, leader);
+        if ((int64_t)(base + nneed) >= total) exhausted = true;
+        if (usable && ((need >> W.gb) & 1u)) {
+          const int64_t myu = (int64_t)base + __popc(need & ((1u << W.gb) - 1u));
+          if (myu < total) {
+            const Cont* k = P.cont_in ? P.cont + myu : nullptr;
+            unit = k ? k->unit : myu;
+            active = true;
+            if (lead && !k) c_lines += (myu & 1) == 0;
+            int64_t g;
+            double xd[3];
+            E = resolve_seed(P, unit >> 1, &g, xd);
+            sgn = (unit & 1) ? R(-1) : R(1);
+            raw = E->F.raw != 0;
+            R ih[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) ih[a] = E->F.inv_h[a];
+            ihc = sel3(c, ih[0], ih[1], ih[2]);
+            hhc = R(1) / ihc;
+            hcf = (float)hhc;
+            orgf = (float)sel3(c, E->F.org[0], E->F.org[1], E->F.org[2]);
+            max_len = E->max_len;
+            h_max = (float)E->h_max;
+            h_min = (float)E->h_min;
+            tiny = 1e-4f * h_max;
+            ilo = (int)floor(sel3(c, E->lo[0], E->lo[1], E->lo[2]));
+            ihi = (int)ceil(sel3(c, E->hi[0], E->hi[1], E->hi[2])) - 1;
+            kvalid = false;
+            if (k) {
+              // a line that cell_kernel_f64 handed over: its state from the
+              // continuation and end records
+              const EndRec<R>& e = P.ends[unit];
+              y = j == 0 ? e.x[c] : (j == 1 ? e.d1[c] : (j == 2 ? e.d2[c] : R(0)));
+              mu = e.mu;
+              muc = k->muc;
+              steps = e.steps;
+              zc = k->zc;
+              h = k->h;
+#pragma unroll
+              for (int a = 0; a < 3; ++a) ic[a] = k->ic[a];
+            } else {
+            R yf[9];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+              double fa = (xd[a] - E->org_d[a]) * E->inv_h_d[a];
+              double fl = floor(fmin(fmax(fa, 0.0), (double)(E->F.n[a] - 2)));
+              ic[a] = (int)fl;
+              yf[a] = fa - fl;
+            }
+#pragma unroll
+            for (int i = 3; i < 9; ++i) yf[i] = R(0);
+            mu = 0;
+            muc = 0;
+            steps = 0;
+            zc = 0;
+            int lface = NO_FACE;
+            int status = ST_RUNNING;
+            bool outside = false;
+#pragma unroll
+            for (int f = 0; f < 6; ++f)
+              if (face_g<R, true>(E->lo, E->hi, ic, f, yf, (const R*)nullptr) > R(0)) outside = true;
+            if (outside || !isfinite(xd[0]) || !isfinite(xd[1]) || !isfinite(xd[2])) {
+              status = QSL_LINE_OUTSIDE;
+            } else {
+              Interp<R> I0;
+              interp<R, R, false, false, true, false>(E->F, yf[0], yf[1], yf[2], I0, ic);
+              R m0 = sqrt(I0.b[0] * I0.b[0] + I0.b[1] * I0.b[1] + I0.b[2] * I0.b[2]);
+              if (!(m0 > R(0))) {
+                status = QSL_LINE_NULL;
+              } else {
+                // Eq. ic (same construction as the other tracers)
+                R u0[3] = {I0.b[0] / m0, I0.b[1] / m0, I0.b[2] / m0};
+                int ax = 0;
+                if (fabs(u0[1]) < fabs(u0[ax])) ax = 1;
+                if (fabs(u0[2]) < fabs(u0[ax])) ax = 2;
+                R av[3];
+                if (ax == 0) { av[0] = 0; av[1] = -u0[2]; av[2] = u0[1]; }
+                else if (ax == 1) { av[0] = u0[2]; av[1] = 0; av[2] = -u0[0]; }
+                else { av[0] = -u0[1]; av[1] = u0[0]; av[2] = 0; }
+                R an = sqrt(av[0] * av[0] + av[1] * av[1] + av[2] * av[2]);
+                av[0] /= an;
+                av[1] /= an;
+                av[2] /= an;
+                yf[3] = av[0];
+                yf[4] = av[1];
+                yf[5] = av[2];
+                yf[6] = u0[1] * av[2] - u0[2] * av[1];
+                yf[7] = u0[2] * av[0] - u0[0] * av[2];
+                yf[8] = u0[0] * av[1] - u0[1] * av[0];
+#pragma unroll
+                for (int f = 0; f < 6; ++f) {
+                  if (status == ST_RUNNING && face_g<R, true>(E->lo, E->hi, ic, f, yf, (const R*)nullptr) == R(0)) {
+                    R bn = I0.b[f >> 1] * sgn;
+                    R outw = (f & 1) ? bn : -bn;
+                    if (outw > R(0)) {
+                      status = QSL_LINE_OK;
+                      lface = f;
+                    }
+                  }
+                }
+              }
+            }
+            const R x_c = sel3(c, yf[0], yf[1], yf[2]), d1_c = sel3(c, yf[3], yf[4], yf[5]),
+                    d2_c = sel3(c, yf[6], yf[7], yf[8]);
+            y = j == 0 ? x_c : (j == 1 ? d1_c * ihc : (j == 2 ? d2_c * ihc : R(0)));  // deviations in cell units
+            h = (float)E->h_init;
+            if (status != ST_RUNNING) {
+              write_end_wide(P, E, unit, c, j, writer, y, ic, hhc, R(0), lface, status, 0);
+              active = false;
+            }
+            }
+          }
+        }
+      }
+    }
+    if (!__any_sync(FULL, active)) {
+      if (exhausted) break;
+      continue;
+    }
+    if (P.timeout_ns && ((++iter & 63) == 0)) {
+      // warp-uniform, so that the lanes of a group agree
+      if (__any_sync(FULL, globaltimer() - t_start > P.timeout_ns)) timed_out = true;
+    }
+    if (!active) continue;
+
+    int status = ST_RUNNING, lface = NO_FACE;
+    if (timed_out) status = QSL_LINE_TIMEOUT;
+    if (status == ST_RUNNING && steps >= P.max_steps) status = QSL_LINE_MAXSTEPS;
+    const R room = max_len - mu;
+    if (status == ST_RUNNING && !gt_bits(room, 0.0)) status = QSL_LINE_MAXLEN;
+    if (status == ST_RUNNING) {
+      if (!kvalid) {
+        // the lane's bilinear coefficients from the 8 corners of component c:
+        // differences along the lane's own axis (j = 3: the lower x face)
+        const size_t sy = 4 * (size_t)E->F.n[0], sz = sy * (size_t)E->F.n[1];
+        const R* p = reinterpret_cast<const R*>(E->F.v) + (size_t)ic[2] * sz + (size_t)ic[1] * sy +
+                     4 * (size_t)ic[0] + c;
+        const size_t oj = j == 1 ? sy : (j == 2 ? sz : 4);
+        const size_t os = (j == 0 || j == 3) ? sy : 4, ot = j == 2 ? sy : sz;
+        const R l00 = __ldg(p), l10 = __ldg(p + os), l01 = __ldg(p + ot), l11 = __ldg(p + os + ot);
+        const R h00 = __ldg(p + oj), h10 = __ldg(p + oj + os), h01 = __ldg(p + oj + ot), h11 = __ldg(p + oj + os + ot);
+        const int icc = sel3(c, ic[0], ic[1], ic[2]);
+        lo_dom = icc <= ilo;
+        hi_dom = icc >= ihi;
+        lo_pl = R(0);
+        hi_pl = R(1);
+        if (lo_dom) lo_pl = sel3(c, E->lo[0], E->lo[1], E->lo[2]) - R(icc);
+        if (hi_dom) hi_pl = sel3(c, E->hi[0], E->hi[1], E->hi[2]) - R(icc);
+        const R sc = raw ? R(1) : ihc;
+        const bool low = j == 3;
+        const R d00 = (low ? l00 : h00 - l00) * sc, d10 = (low ? l10 : h10 - l10) * sc;
+        const R d01 = (low ? l01 : h01 - l01) * sc, d11 = (low ? l11 : h11 - l11) * sc;
+        co[0] = d00;
+        co[1] = d10 - d00;
+        co[2] = d01 - d00;
+        co[3] = (d11 - d10) - (d01 - d00);
+        k1 = wide_rhs(W, co, raw, ihc, y);
+        c_stage += lead;
+        kvalid = true;
+      }
+      // step: controller size, capped a little beyond the first plane along k1
+      const R r_lo = lo_pl - y, r_hi = hi_pl - y;  // position lanes
+      const float vel = (float)(sgn * k1);
+      float tf = 1e30f;
+      if (vel != 0.0f) tf = __fdividef((float)(vel > 0.0f ? r_hi : r_lo), vel);
+      const float tf0 = __shfl_sync(W.gm, tf, W.pos(0)), tf1 = __shfl_sync(W.gm, tf, W.pos(1)),
+                  tf2 = __shfl_sync(W.gm, tf, W.pos(2));
+      const float tface = fminf(fminf(tf0, tf1), tf2);
+      {
+        // ask L1 for the vertices of the cell beyond that plane
+        const int pa = tf0 <= tface ? 0 : (tf1 <= tface ? 1 : 2);
+        const float v0 = __shfl_sync(W.gm, vel, W.pos(pa));
+        const int d = v0 > 0.0f ? 1 : -1;
+        int q[3] = {ic[0], ic[1], ic[2]};
+        if (pa == 0) q[0] = min(max(q[0] + d, 0), E->F.n[0] - 2);
+        else if (pa == 1) q[1] = min(max(q[1] + d, 0), E->F.n[1] - 2);
+        else q[2] = min(max(q[2] + d, 0), E->F.n[2] - 2);
+        const size_t n0 = (size_t)E->F.n[0], n01 = n0 * (size_t)E->F.n[1];
+        prefetch_l1(E->F.v + ((size_t)(q[2] + ((l >> 2) & 1)) * n01 + (size_t)(q[1] + ((l >> 1) & 1)) * n0 +
+                              (size_t)(q[0] + (l & 1))));
+      }
+      float hsF = fminf(h, h_max);
+      R hs;
+      bool capped = false;
+      if ((float)room > 1.001f * hsF) {
+        hs = (R)hsF;
+      } else {  // near the maximum length: the cap in FP64
+        capped = room <= (R)hsF;
+        hs = capped ? room : (R)hsF;
+        hsF = (float)hs;
+      }
+      const float hf = 1.25f * fmaxf(tface, 0.0f) + tiny;
+      if (hf < hsF) {
+        hsF = hf;
+        hs = (R)hf;
+        capped = false;
+      }
+      const R hh = sgn * hs;
+      // stages on K_i = hh k_i
+      const R K1 = hh * k1;
+      const R K2 = hh * wide_rhs(W, co, raw, ihc, fma(R(DA21), K1, y));
+      const R K3 = hh * wide_rhs(W, co, raw, ihc, fma(R(DA32), K2, fma(R(DA31), K1, y)));
+      const R K4 = hh * wide_rhs(W, co, raw, ihc, fma(R(DA43), K3, fma(R(DA42), K2, fma(R(DA41), K1, y))));
+      const R K5 = hh * wide_rhs(W, co, raw, ihc,
+                                 fma(R(DA54), K4, fma(R(DA53), K3, fma(R(DA52), K2, fma(R(DA51), K1, y)))));
+      const R K6 = hh * wide_rhs(W, co, raw, ihc,
+                                 fma(R(DA65), K5, fma(R(DA64), K4, fma(R(DA63), K3, fma(R(DA62), K2, fma(R(DA61), K1, y))))));
+      const R dy = fma(R(DB6), K6, fma(R(DB5), K5, fma(R(DB4), K4, fma(R(DB3), K3, R(DB1) * K1))));
+      const R t = y + dy;
+      const R k7 = wide_rhs(W, co, raw, ihc, t);
+      const R K7 = hh * k7;
+      c_stage += lead ? 6 : 0;
+      steps += 1;
+      float err;
+      {
+        const float e = fabsf((float)fma(R(DE7), K7, fma(R(DE6), K6, fma(R(DE5), K5, fma(R(DE4), K4,
+                              fma(R(DE3), K3, R(DE1) * K1)))))) * hcf;
+        const float base = j == 0 ? fmaf((float)sel3(c, ic[0], ic[1], ic[2]), hcf, orgf) : 0.0f;
+        const float m = fmaxf(fabsf(fmaf((float)y, hcf, base)), fabsf(fmaf((float)t, hcf, base)));
+        err = __fdividef(e, fmaf(tolr, m, tola));
+        const int r0 = W.pos(c);
+        err = fmaxf(fmaxf(__shfl_sync(W.gm, err, r0), __shfl_sync(W.gm, err, r0 + 1)), __shfl_sync(W.gm, err, r0 + 2));
+        err = fmaxf(fmaxf(__shfl_sync(W.gm, err, W.pos(0)), __shfl_sync(W.gm, err, W.pos(1))),
+                    __shfl_sync(W.gm, err, W.pos(2)));
+      }
+      const bool bad = __any_sync(W.gm, (__double2hiint(t) & 0x7ff00000) == 0x7ff00000);
+      if (bad) {
+        status = QSL_LINE_NONFINITE;
+      } else if (err > 1.0f) {
+        c_rej += lead;
+        h = hsF * fmaxf(0.2f, 0.9f * __powf(err, -0.25f));
+        if (h < h_min) status = QSL_LINE_STALL;
+      } else {
+        c_acc += lead;
+        const float hnext = hsF * ((err == 0.0f) ? 5.0f : fminf(5.0f, 0.9f * __powf(err, -0.2f)));
+        const R c4 = fma(R(DD7), K7, fma(R(DD6), K6, fma(R(DD5), K5, fma(R(DD4), K4, fma(R(DD3), K3, R(DD1) * K1)))));
+        const R bspl = K1 - dy;
+        const R c3 = (dy - K7) - bspl;
+        // the plane of the lane's axis that the step ends beyond (at most one)
+        const R band = R(16) * eps_of<R>();
+        const bool o_lo = gt_bits(r_lo - dy, lo_dom ? R(0) : band), o_hi = gt_bits(dy - r_hi, hi_dom ? R(0) : band);
+        R thc = R(2);
+        if (j == 0 && (o_lo || o_hi)) thc = cross_root(o_lo ? r_lo : r_hi, dy, bspl, c3, c4, o_lo ? 0 : 1);
+        // earliest crossing over the axes; ties go to the lower plane id
+        const R q0 = gsh(W.gm, thc, W.pos(0)), q1 = gsh(W.gm, thc, W.pos(1)), q2 = gsh(W.gm, thc, W.pos(2));
+        R th = R(2);
+        int ax_c = -1;
+        if (gt_bits(th, q0)) { th = q0; ax_c = 0; }
+        if (gt_bits(th, q1)) { th = q1; ax_c = 1; }
+        if (gt_bits(th, q2)) { th = q2; ax_c = 2; }
+        if (ax_c < 0) {
+          // the step stays in the cell: accept it; k7 is the next k1
+          y = t;
+          k1 = k7;
+          R t1 = hs - muc, t2 = mu + t1;
+          muc = (t2 - mu) - t1;
+          mu = t2;
+          h = hnext;
+          zc = 0;
+          if (capped) status = QSL_LINE_MAXLEN;
+        } else {
+          // advance to the plane on the dense output and snap onto it
+          const R s1 = R(1) - th;
+          y += th * fma(s1, fma(th, fma(s1, c4, c3), bspl), dy);
+          const int flags = (o_lo ? 0 : 1) | ((o_lo ? lo_dom : hi_dom) ? 2 : 0);
+          const int fl = __shfl_sync(W.gm, flags, W.pos(ax_c));
+          const int up_c = fl & 1;
+          if (j == 0 && c == ax_c) y = up_c ? hi_pl : lo_pl;
+          const R dl = th * hs;
+          R t1 = dl - muc, t2 = mu + t1;
+          muc = (t2 - mu) - t1;
+          mu = t2;
+          c_land += lead;
+          if (fl & 2) {
+            status = QSL_LINE_OK;
+            lface = 2 * ax_c + up_c;
+          } else {
+            // enter the neighbouring cell
+            zc = ((float)dl < tiny) ? zc + 1 : 0;
+            const int na = sel3(ax_c, ic[0], ic[1], ic[2]) + (up_c ? 1 : -1);
+            if (zc > 3 || na < 0 || na > sel3(ax_c, E->F.n[0], E->F.n[1], E->F.n[2]) - 2) {
+              // grazing a face back and forth: stay in this cell for one step
+              zc = 0;
+            } else {
+              if (ax_c == 0) ic[0] = na;
+              else if (ax_c == 1) ic[1] = na;
+              else ic[2] = na;
+              if (j == 0 && c == ax_c) y = up_c ? R(0) : R(1);
+              kvalid = false;
+            }
+            h = fmaxf(hnext, hsF);
+          }
+        }
+      }
+    }
+    if (status != ST_RUNNING) {
+      write_end_wide(P, E, unit, c, j, writer, y, ic, hhc, mu, lface, status, steps);
+      active = false;
+    }
+  }
+  write_stats(P, lane, c_stage, c_acc, c_rej, c_land, c_lines, timed_out);
 }
 
 // ------------------------------------------------------------ lengths-only cell-wise tracer
@@ -2656,10 +3381,6 @@ __device__ __forceinline__ void ck_len_step(const V* fv, const int* n, int64_t s
     dy[i] = hh * (R(B1) * k1[i] + R(B3) * k3[i] + R(B4) * k4[i] + R(B6) * k6[i]);
     yerr[i] = hh * (R(E1) * k1[i] + R(E3) * k3[i] + R(E4) * k4[i] + R(E5) * k5[i] + R(E6) * k6[i]);
   }
-}
-
-__device__ __forceinline__ void prefetch_l1(const void* p) {
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
 // Asks L1 for the corner rows of the cell holding the local-frame point
@@ -3230,8 +3951,37 @@ Item<R> make_item(const qsl_field* f, const SeedSource& src, const TraceConfig& 
   return it;
 }
 
-// Scratch of one tracing launch: the queue head and watchdog flag (16 bytes
-// at offset 0) and one end record per unit from offset 256. `scratch` is
+// The three-lane kernel of a type and component count; FP64 with the
+// deviations runs cell_wide_kernel instead.
+template <int NC>
+inline void (*coop_kernel_fn(float*))(const TraceParams<float>) {
+  return cell_coop_kernel<float, NC>;
+}
+template <int NC>
+inline void (*coop_kernel_fn(double*))(const TraceParams<double>) {
+  return cell_coop_kernel<double, 3>;
+}
+inline void launch_wide(const TraceParams<double>& P, int blocks, int threads, int sms, cudaStream_t stream) {
+  cell_wide_kernel<<<blocks, threads, 0, stream>>>(P, sms);
+}
+inline void launch_wide(const TraceParams<float>&, int, int, int, cudaStream_t) {}
+
+// A warp of cell_kernel_f64 hands its lines to cell_wide_kernel once the queue
+// is empty and at most kHandoff of them are left: on one lane each the last
+// lines take 25 us per step, on sixteen 7. Measured (FP64 map of 82,497 seeds
+// on 128^3; never, 8, 12, 16, 24, 32 lines): 29.6, 23.9, 22.2, 20.8, 20.6,
+// 20.4 ms; 196,608 seeds: 44.6, 36.4, 34.1, 33.9, 34.1, 34.0 ms. kContMax: the
+// most handed over per launch (resident warps x kHandoff is below it).
+constexpr int kHandoff = 24;
+constexpr size_t kContMax = 1 << 16;
+template <class R>
+size_t cont_offset(size_t n_units) {
+  return (256 + sizeof(EndRec<R>) * (n_units ? n_units : 1) + 15) / 16 * 16;
+}
+
+// Scratch of one tracing launch: queue head, watchdog flag, continuation count
+// and queue head of the handed-over lines (32 bytes at offset 0), one end
+// record per unit from offset 256 and, FP64, the continuation records. `scratch` is
 // either caller-provided (no-allocation entry point, captured plans) or
 // allocated here.
 template <class R, int NC>
@@ -3245,10 +3995,10 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
   size_t n_units = (size_t)(2 * n_seeds);
   const bool own = scratch == nullptr;
   if (own)
-    QSL_CHECK_CUDA(qsl::alloc_async((void**)&scratch, 256 + sizeof(EndRec<R>) * (n_units ? n_units : 1), stream));
+    QSL_CHECK_CUDA(qsl::alloc_async((void**)&scratch, scratch_bytes(sizeof(R) == 8 ? QSL_FP64 : QSL_FP32_MIXED, n_units), stream));
   unsigned long long* head = reinterpret_cast<unsigned long long*>(scratch);
   EndRec<R>* ends = reinterpret_cast<EndRec<R>*>(reinterpret_cast<unsigned char*>(scratch) + 256);
-  QSL_CHECK_CUDA(cudaMemsetAsync(head, 0, 16, stream));
+  QSL_CHECK_CUDA(cudaMemsetAsync(head, 0, 32, stream));
   TraceParams<R> P;
   P.item0 = item0;
   P.items = items_dev;
@@ -3266,6 +4016,10 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
   P.refill_min = shape.refill_min > 0 ? shape.refill_min : 1;
   P.timeout_ns = cfg.timeout_ns;
   P.timeout_flag = reinterpret_cast<int*>(head + 1);
+  P.cont = reinterpret_cast<Cont*>(reinterpret_cast<unsigned char*>(scratch) + cont_offset<R>(n_units));
+  P.cont_count = head + 2;
+  P.handoff = 0;
+  P.cont_in = 0;
   int threads = 32 * shape.warps_per_block;
   // persistent kernel: never launch more blocks than can be resident at once
   const bool use_cell = loc && cfg.integrator == QSL_DOPRI5_CELL;
@@ -3300,19 +4054,26 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
     } else if (shape.line_lanes == 0) {
       // auto: three lanes per line up to 512 units (line directions) per SM,
       // where the launch is bound by the latency of its longest lines rather
-      // than by issue rate (measured crossover on GB300: about 640 per SM); a
-      // device-side count is a retrace list, short by construction
+      // than by issue rate (measured crossover on GB300: about 640 per SM);
+      // FP64 with the deviations: sixteen lanes per line up to the same count
+      // (32,000 seeds of a map on 128^3: 13.0 ms, one lane with the hand-over
+      // 13.4; 82,497 seeds 29.1 and 20.6); a device-side count is a retrace
+      // list, short by construction
       coop = n_seeds_dev != nullptr || 2 * n_seeds <= (int64_t)512 * sms;
     }
   }
+  // FP64 with the deviations: sixteen lanes per line in place of three
+  const bool wide = coop && sizeof(R) == 8 && NC == 9;
   size_t smem = (use_cell && !coop && !len_kernel) ? (size_t)24 * threads * sizeof(R) : 0;
   int resident = 0;
   if (ck_len)
     QSL_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, ck_len_kernel<R>, threads, 0));
   else if (len_kernel)
     QSL_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, cell_len_kernel<R>, threads, 0));
+  else if (wide)
+    QSL_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, cell_wide_kernel, threads, 0));
   else if (coop)
-    QSL_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, cell_coop_kernel<R, NC>, threads, 0));
+    QSL_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, coop_kernel_fn<NC>((R*)nullptr), threads, 0));
   else if (use_cell)
     QSL_CHECK_CUDA(
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, cell_kernel_fn<NC>((R*)nullptr), threads, smem));
@@ -3346,12 +4107,30 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
     } else if (len_kernel) {
       cell_len_kernel<R><<<blocks, threads, 0, stream>>>(P);
       qsl::count_launch();
+    } else if (wide) {
+      launch_wide(P, blocks, threads, sms, stream);
+      qsl::count_launch();
     } else if (coop) {
-      cell_coop_kernel<R, NC><<<blocks, threads, 0, stream>>>(P);
+      coop_kernel_fn<NC>((R*)nullptr)<<<blocks, threads, 0, stream>>>(P);
       qsl::count_launch();
     } else if (use_cell) {
+      // FP64, automatic lanes: the last lines of every warp go to the
+      // sixteen-lane kernel
+      if (sizeof(R) == 8 && NC == 9 && shape.line_lanes == 0 &&
+          (size_t)blocks * shape.warps_per_block * kHandoff <= kContMax)
+        P.handoff = kHandoff;
       cell_kernel_fn<NC>((R*)nullptr)<<<blocks, threads, smem, stream>>>(P);
       qsl::count_launch();
+      if (P.handoff) {
+        QSL_CHECK_CUDA(cudaGetLastError());
+        int res_w = 0;
+        QSL_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res_w, cell_wide_kernel, threads, 0));
+        TraceParams<R> Pw = P;
+        Pw.head = head + 3;
+        Pw.cont_in = 1;
+        launch_wide(Pw, sms * (res_w > 0 ? res_w : 1), threads, sms, stream);
+        qsl::count_launch();
+      }
     } else if (loc && cfg.geom == QSL_GEOM_SPHERICAL && cfg.interp_order > 1) {
       trace_kernel<R, NC, true, true, true><<<blocks, threads, 0, stream>>>(P);
       qsl::count_launch();
@@ -3412,8 +4191,10 @@ int trace_and_assemble(const qsl_field* f, const SeedSource& src, int64_t n_seed
                            shape, out, stream, stats_dev, ev, scratch);
 }
 
-size_t end_record_bytes(int precision) {
-  return precision == QSL_FP64 ? sizeof(EndRec<double>) : sizeof(EndRec<float>);
+size_t scratch_bytes(int precision, size_t n_units) {
+  if (precision == QSL_FP64)
+    return cont_offset<double>(n_units) + sizeof(Cont) * (n_units < kContMax ? n_units : kContMax);
+  return cont_offset<float>(n_units);
 }
 
 int select_retrace(const SeedSource& src, int64_t n_seeds, const LineOutputs& out, double threshold,
@@ -3637,14 +4418,14 @@ int plan_build(const qsl_batch_item* items, int n_items, const qsl_opts* o, floa
   size_t n_units = (size_t)(2 * p->total);
   PLAN_TRY(cudaMalloc(&p->table32, sizeof(qsl::Item<float>) * n_items));
   PLAN_TRY(cudaMemcpy(p->table32, t32.data(), sizeof(qsl::Item<float>) * n_items, cudaMemcpyHostToDevice));
-  PLAN_TRY(cudaMalloc(&p->scratch32, 256 + qsl::end_record_bytes(o->precision) * (n_units ? n_units : 1)));
+  PLAN_TRY(cudaMalloc(&p->scratch32, qsl::scratch_bytes(o->precision, n_units)));
   PLAN_TRY(cudaMalloc((void**)&p->stats, sizeof(qsl::DeviceStats)));
   if (o->precision == QSL_FP64 || p->retrace_q > 0) {
     PLAN_TRY(cudaMalloc(&p->table64, sizeof(qsl::Item<double>) * n_items));
     PLAN_TRY(cudaMemcpy(p->table64, t64.data(), sizeof(qsl::Item<double>) * n_items, cudaMemcpyHostToDevice));
   }
   if (p->retrace_q > 0) {
-    PLAN_TRY(cudaMalloc(&p->scratch64, 256 + sizeof(qsl::EndRec<double>) * (n_units ? n_units : 1)));
+    PLAN_TRY(cudaMalloc(&p->scratch64, qsl::scratch_bytes(QSL_FP64, n_units)));
     PLAN_TRY(cudaMalloc((void**)&p->index, sizeof(int64_t) * (p->total ? p->total : 1)));
     PLAN_TRY(cudaMalloc((void**)&p->count, sizeof(int64_t)));
     if (!q) {
