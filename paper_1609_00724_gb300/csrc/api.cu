@@ -167,7 +167,10 @@ int default_shape(const qsl_opts* o, int tangent, int precision, LaunchShape* s)
     s->blocks_per_sm = w / s->warps_per_block;
     if (s->blocks_per_sm < 1) s->blocks_per_sm = 1;
   }
-  s->refill_min = o->refill_min > 0 ? o->refill_min : 1;
+  // idle lanes before a warp refills, unless asked for: 8 or, on launches of few
+  // lines, 1 (decided at the launch)
+  s->refill_auto = o->refill_min <= 0;
+  s->refill_min = o->refill_min > 0 ? o->refill_min : 8;
   s->line_lanes = o->line_lanes;
   return QSL_OK;
 }

@@ -162,6 +162,7 @@ struct LaunchShape {
   int blocks_per_sm;
   int refill_min;
   int line_lanes;  // cell-wise tracer: 1 or 3 lanes per line, 0 = auto
+  int refill_auto; // refill_min was left to the library
 };
 
 // Runs the tracer over `n_seeds` seeds of `src` (n_seeds may live on the

@@ -4013,7 +4013,6 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
   P.tol_rel = (R)cfg.tol_rel;
   P.max_steps = cfg.max_steps;
   P.euler = cfg.integrator == QSL_EULER;
-  P.refill_min = shape.refill_min > 0 ? shape.refill_min : 1;
   P.timeout_ns = cfg.timeout_ns;
   P.timeout_flag = reinterpret_cast<int*>(head + 1);
   P.cont = reinterpret_cast<Cont*>(reinterpret_cast<unsigned char*>(scratch) + cont_offset<R>(n_units));
@@ -4099,6 +4098,16 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
   if ((int64_t)blocks * shape.warps_per_block > max_warps_needed && !n_seeds_dev)
     blocks = (int)((max_warps_needed + shape.warps_per_block - 1) / shape.warps_per_block);
   if (blocks < 1) blocks = 1;
+  // Left to the library, a warp waits for 8 idle lanes before it refills (its
+  // other lanes wait during a refill) when the launch fills the resident lanes
+  // at least four times; shorter launches are bound by their longest lines and
+  // the three-lane and sixteen-lane kernels run few lines per warp: no wait.
+  // Thresholds 1, 4, 8, 12 on long launches: 1024^2 map on 256^3 16.6, 14.1,
+  // 13.8, 14.2 ms; 512^2 Cash-Karp map at tol 1e-2 2.17, 1.90, 1.84, 1.83;
+  // volume of 8.4 M seeds 392, 360, 361, 374. 1 and 8 on a launch of 1.4 times
+  // the resident lanes: 1.18 and 1.22 ms.
+  P.refill_min = shape.refill_min > 0 ? shape.refill_min : 1;
+  if (shape.refill_auto && (coop || n_seeds_dev || 2 * n_seeds < 4 * (int64_t)blocks * threads)) P.refill_min = 1;
   if (ev) QSL_CHECK_CUDA(cudaEventRecord(ev[0], stream));
   if (n_seeds > 0) {
     if (ck_len) {
