@@ -5,130 +5,792 @@
 // forward and backward passes (FP32 master copy, Adam in FP32); every
 // contraction accumulates in FP32. Activations are NCHW float32.
 //
-// Kernels: one output pixel per thread with all output channels in registers,
-// the input tile (+1 halo) and the layer's weights staged in shared memory;
-// the weight gradient reduces over pixels per block and adds into FP32
-// gradients with one atomic per weight and block.
+// The convolutions run on the tensor cores (tcgen05) as implicit GEMMs over
+// the pixels of a tile. The activations and gradients stay FP32 values: each
+// is split into three BF16 pieces that sum to it exactly (8 bits each), the
+// pieces' products with the BF16 weights (or with the other operand's pieces)
+// are exact, and the sums are FP32. One block's tile goes through all layers
+// in shared and tensor memory, so a forward pass reads its input and writes
+// its output once.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <cstring>
 #include <vector>
 
 #include "qsl_internal.cuh"
+#include "umma.cuh"
 
 namespace {
 
-constexpr int T = 16;          // output tile edge
-constexpr int TH = T + 2;      // with halo
 constexpr int C1 = 2, C2 = 32; // input and hidden channels
 constexpr int NW1 = 32 * 2 * 9, NB1 = 32, NW2 = 32 * 32 * 9, NB2 = 32, NW3 = 32 * 9, NB3 = 1;
 constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + NW1, OFF_W2 = OFF_B1 + NB1, OFF_B2 = OFF_W2 + NW2, OFF_W3 = OFF_B2 + NB2,
               OFF_B3 = OFF_W3 + NW3, NPAR = OFF_B3 + NB3;
 
-// y[n][co][p] = act(b[co] + sum_{ci,k} w[co][ci][k] x[n][ci][p + k - 1])  (zero padding)
-// TRANSPOSE: the data gradient of a convolution: w read as w[ci][co][8 - k]
-// (channels swapped, kernel flipped), no bias; MASK: multiply by (m > 0).
-template <int CIN, int COUT, bool RELU, bool TRANSPOSE, bool BIAS>
-__global__ void __launch_bounds__(T* T) conv3x3_kernel(const float* __restrict__ x, const __nv_bfloat16* __restrict__ w,
-                                                      const float* __restrict__ b, const float* __restrict__ mask,
-                                                      float* __restrict__ y, int H, int W) {
-  extern __shared__ float sm[];
-  float* xs = sm;                    // CIN x TH x TH
-  float* ws = sm + CIN * TH * TH;    // COUT x CIN x 9 (as used)
-  const int n = blockIdx.z;
-  const int ox = blockIdx.x * T, oy = blockIdx.y * T;
-  const int tid = threadIdx.x;
-  const size_t plane = (size_t)H * W;
-  const float* xn = x + (size_t)n * CIN * plane;
-  for (int i = tid; i < CIN * TH * TH; i += T * T) {
-    int c = i / (TH * TH), r = (i / TH) % TH, q = i % TH;
-    int gy = oy + r - 1, gx = ox + q - 1;
-    xs[i] = (gy >= 0 && gy < H && gx >= 0 && gx < W) ? xn[c * plane + (size_t)gy * W + gx] : 0.0f;
-  }
-  for (int i = tid; i < COUT * CIN * 9; i += T * T) {
-    int co = i / (CIN * 9), ci = (i / 9) % CIN, k = i % 9;
-    float v;
-    if (TRANSPOSE)
-      v = __bfloat162float(w[(ci * COUT + co) * 9 + (8 - k)]);  // weights stored [CIN'=COUT][COUT'=CIN]
-    else
-      v = __bfloat162float(w[(co * CIN + ci) * 9 + k]);
-    ws[i] = v;
-  }
-  __syncthreads();
-  const int tx = tid % T, ty = tid / T;
-  const int gx = ox + tx, gy = oy + ty;
-  float acc[COUT];
-#pragma unroll
-  for (int co = 0; co < COUT; ++co) acc[co] = BIAS ? b[co] : 0.0f;
-#pragma unroll 1
-  for (int ci = 0; ci < CIN; ++ci) {
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      float v = xs[(ci * TH + ty + k / 3) * TH + tx + k % 3];
-#pragma unroll
-      for (int co = 0; co < COUT; ++co) acc[co] = fmaf(v, ws[(co * CIN + ci) * 9 + k], acc[co]);
-    }
-  }
-  if (gx < W && gy < H) {
-    float* yn = y + (size_t)n * COUT * plane + (size_t)gy * W + gx;
-    const float* mn = mask ? mask + (size_t)n * COUT * plane + (size_t)gy * W + gx : nullptr;
-#pragma unroll
-    for (int co = 0; co < COUT; ++co) {
-      float v = acc[co];
-      if (RELU) v = fmaxf(v, 0.0f);
-      if (mn && !(mn[co * plane] > 0.0f)) v = 0.0f;
-      yn[co * plane] = v;
-    }
+// ---------------------------------------------------------------- tiles
+// Forward and data-gradient tiles: rows of 32 pixels (one warp each), the
+// MMA's 128 rows are four of them. Flattened indices are row * 32 + column;
+// a tap (ky, kx) of the pixel m is the pixel m + 32 ky + kx of the layer
+// below, so the last columns of a row see the next row's first ones: each
+// layer has two valid columns less than the one below, and 2 rows less.
+constexpr int PW = 32;
+constexpr int R2 = 12, R1 = R2 + 2;         // rows of the 32-channel layers: outputs, inputs
+constexpr int M2 = R2 * PW;                 // output pixels: three MMA tiles
+constexpr int NP = R1 * PW + 8;             // input pixels (the last taps read two past the rows)
+constexpr int ZW = PW - 6, ZH = R2 - 2;     // forward: valid output columns, rows
+constexpr int DW = PW - 2, DH = R2;         // data gradient: valid columns, rows
+constexpr int NPX = (R1 + 4) * PW + 8;      // forward: network input pixels (16 rows of layer 1 are computed)
+constexpr int TILE_THREADS = 32 * R2;
+constexpr uint32_t CHUNK = NP * 16;         // bytes of one chunk plane
+constexpr uint32_t WTAP = 32 * 64;          // one tap's 32 x 32 weights
+
+struct alignas(16) TileSmem {
+  unsigned char a[12 * CHUNK];              // [piece][chunk] planes of the layer below; before that the network input
+  unsigned char w2[9 * WTAP];               // [tap][chunk][out channel][8]
+  unsigned char w1[5 * 1024];               // [tap pair][tap][out channel][8]
+  float w3[9 * 32];                         // [tap][channel]
+  float b1[32], b2[32], b3;
+  uint32_t tmem;
+  int failed;
+  uint64_t bar[4];
+};
+static_assert(sizeof(TileSmem) <= 113 * 1024, "two blocks per SM");
+static_assert(NPX * 16 + 2048 <= 12 * CHUNK && 9 * M2 * 4 <= 12 * CHUNK, "overlays of the planes");
+
+// Layer 2's weights are kept twice more in the layout of the MMA's operand,
+// [tap][chunk][N][8] (K = chunk and element): K = input channels, N = output
+// channels for the forward pass, and channels swapped, taps reversed for the
+// data gradient. They are written wherever the BF16 weights are.
+constexpr int OFF_OP = (NPAR + 7) / 8 * 8, NWB = OFF_OP + 2 * NW2;
+__device__ __forceinline__ void store_weight(__nv_bfloat16* wb, int i, float v) {
+  const __nv_bfloat16 b = __float2bfloat16_rn(v);
+  wb[i] = b;
+  if (i >= OFF_W2 && i < OFF_W2 + NW2) {
+    const int j = i - OFF_W2, co = j / (32 * 9), ci = (j / 9) % 32, k = j % 9;
+    wb[OFF_OP + ((k * 4 + ci / 8) * 32 + co) * 8 + ci % 8] = b;
+    wb[OFF_OP + NW2 + (((8 - k) * 4 + co / 8) * 32 + ci) * 8 + co % 8] = b;
   }
 }
 
-// dW[co][ci][k] += sum_p dy[n][co][p] x[n][ci][p + k - 1]; dB[co] += sum_p dy.
-// One block per (tile, image); threads own weights (strided), pixels in smem.
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(T* T) conv3x3_wgrad_kernel(const float* __restrict__ x, const float* __restrict__ dy,
-                                                            float* __restrict__ dw, float* __restrict__ db, int H,
-                                                            int W) {
-  extern __shared__ float sm[];
-  float* xs = sm;                  // CIN x TH x TH
-  float* ds = sm + CIN * TH * TH;  // COUT x T x T
-  const int n = blockIdx.z;
-  const int ox = blockIdx.x * T, oy = blockIdx.y * T;
-  const int tid = threadIdx.x;
-  const size_t plane = (size_t)H * W;
-  const float* xn = x + (size_t)n * CIN * plane;
-  const float* dn = dy + (size_t)n * COUT * plane;
-  for (int i = tid; i < CIN * TH * TH; i += T * T) {
-    int c = i / (TH * TH), r = (i / TH) % TH, q = i % TH;
-    int gy = oy + r - 1, gx = ox + q - 1;
-    xs[i] = (gy >= 0 && gy < H && gx >= 0 && gx < W) ? xn[c * plane + (size_t)gy * W + gx] : 0.0f;
+__device__ __forceinline__ void load_w2(unsigned char* w2, const __nv_bfloat16* __restrict__ op, int tid) {
+#pragma unroll
+  for (int i = tid; i < NW2 / 8; i += TILE_THREADS)
+    reinterpret_cast<uint4*>(w2)[i] = __ldg(reinterpret_cast<const uint4*>(op) + i);
+}
+
+// The 32 x 32 convolution of the planes in `a` for MMA tile t (128 pixels):
+// 9 taps x 3 pieces x 2 K steps into four accumulators of 32 columns. The
+// tensor core cuts each sum's low bits, so the leading pieces have one
+// accumulator per row of taps (six sums each; the rows are then added in
+// FP32) and the middle and last pieces, 2^-8 and 2^-16 of them, the fourth.
+// Tile 2 takes tile 0's columns (conv32_read hands them over). One thread.
+__device__ __forceinline__ void conv32_issue(TileSmem& S, uint32_t tmem, int t) {
+  const uint64_t a0 = umma::desc_k(umma::smem_addr(S.a) + t * 2048, CHUNK), w0 = umma::desc_k(umma::smem_addr(S.w2), 512);
+  const uint32_t d0 = tmem + (t & 1) * 128;
+  constexpr uint32_t id = umma::idesc(128, 32, false);
+#pragma unroll
+  for (int piece = 2; piece >= 0; --piece)
+#pragma unroll
+    for (int tap = 0; tap < 9; ++tap)
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        umma::mma(d0 + (piece ? 96 : 32 * (tap / 3)),
+                  a0 + ((piece * 4 + 2 * k) * CHUNK / 16 + (tap / 3) * PW + tap % 3), w0 + (tap * WTAP + k * 1024) / 16,
+                  id, piece == 0 ? tap % 3 > 0 || k > 0 : piece == 1 || tap > 0 || k > 0);
+  umma::commit(&S.bar[1 + t]);
+}
+
+// Waits for the MMA tile of the warp's row (warp / 4) and reads its sums; the
+// first four warps then let tile 2 be issued into the columns they have read.
+__device__ __forceinline__ bool conv32_read(TileSmem& S, uint32_t tmem, int warp, uint32_t phase, float* v) {
+  const int t = warp >> 2;
+  const uint32_t tq = tmem + ((uint32_t)(warp & 3) << 21) + (t & 1) * 128;
+  const bool ok = umma::bar_wait(&S.bar[1 + t], phase);
+  umma::fence_after();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float u[16];
+    umma::tmem_ld16(tq + 96 + 16 * h, v + 16 * h);
+#pragma unroll
+    for (int row = 0; row < 3; ++row) {
+      umma::tmem_ld16(tq + 32 * row + 16 * h, u);
+#pragma unroll
+      for (int c = 0; c < 16; ++c) v[16 * h + c] += u[c];
+    }
   }
-  for (int i = tid; i < COUT * T * T; i += T * T) {
-    int c = i / (T * T), r = (i / T) % T, q = i % T;
-    int gy = oy + r, gx = ox + q;
-    ds[i] = (gy < H && gx < W) ? dn[c * plane + (size_t)gy * W + gx] : 0.0f;
+  if (t == 0) {
+    umma::fence_before();
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    if (warp == 0 && umma::elect()) {
+      umma::fence_after();
+      conv32_issue(S, tmem, 2);
+    }
+    __syncwarp();
+  }
+  return ok;
+}
+
+// Writes a pixel's 16 channels (half h of the 32) as pieces into the planes.
+__device__ __forceinline__ void store_half(unsigned char* a, int m, int h, const float* v) {
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    uint4 p[3];
+    umma::split8(v + 8 * c, p);
+#pragma unroll
+    for (int piece = 0; piece < 3; ++piece)
+      *reinterpret_cast<uint4*>(a + (piece * 4 + 2 * h + c) * CHUNK + m * 16) = p[piece];
+  }
+}
+
+__device__ __forceinline__ void zero_tail(unsigned char* a, int tid) {
+  if (tid < 12 * (NP - R1 * PW))
+    *reinterpret_cast<uint4*>(a + (tid / (NP - R1 * PW)) * CHUNK + (R1 * PW + tid % (NP - R1 * PW)) * 16) =
+        make_uint4(0, 0, 0, 0);
+}
+
+__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(reinterpret_cast<unsigned long long&>(d))
+      : "l"(reinterpret_cast<unsigned long long&>(a)), "l"(reinterpret_cast<unsigned long long&>(b)),
+        "l"(reinterpret_cast<unsigned long long&>(c)));
+  return d;
+}
+
+struct TileGrid {
+  int n, H, W, tx, ty;  // images, tiles along x and y
+  int64_t tiles;
+};
+__device__ __forceinline__ void tile_of(const TileGrid& G, int64_t t, int w, int h, int* n, int* oy, int* ox) {
+  *ox = (int)(t % G.tx) * w;
+  t /= G.tx;
+  *oy = (int)(t % G.ty) * h;
+  *n = (int)(t / G.ty);
+}
+
+// Forward pass of one 26 x 10 pixel tile per iteration (persistent, two
+// blocks per SM), all three layers:
+//  1. the input's two channels as one 16-byte chunk of pieces per pixel
+//     (x0 hi, mid, lo, x1 hi, mid, lo, 0, 0); a K = 16 step of the MMA takes
+//     two taps of it, the ninth is paired with zeros;
+//  2. TMEM -> bias, ReLU (0 outside the image) -> pieces in the planes -> the
+//     32 x 32 convolution;
+//  3. TMEM -> bias, ReLU -> each pixel's products with layer 3's nine taps,
+//     summed over the neighbours through shared memory.
+// TRAIN keeps the activations and writes logits, otherwise probabilities.
+// Bound: the MMAs. An M = 128, K = 16 step with operands in shared memory takes
+// 59 cycles for N = 32 (72 for N = 128: the read of A sets it), 182 steps per
+// tile. 64 slices of 256 x 256: 0.69 ms, 10.6 k of the 12.1 k cycles per tile
+// and SM (the FP32 kernels, one per layer with activations in memory: 5.6 ms).
+template <bool TRAIN>
+__global__ void __launch_bounds__(TILE_THREADS, 2)
+    forward_kernel(const float* __restrict__ x, const __nv_bfloat16* __restrict__ wb, const float* __restrict__ w,
+                   float* __restrict__ a1, float* __restrict__ a2, float* __restrict__ out, const TileGrid G) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  TileSmem& S = *reinterpret_cast<TileSmem*>(smem);
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const size_t plane = (size_t)G.H * G.W;
+  load_w2(S.w2, wb + OFF_OP, tid);
+  for (int i = tid; i < 5 * 512; i += TILE_THREADS) {
+    const int e = i % 8, co = (i / 8) % 32, tap = 2 * (i / 512) + (i / 256) % 2;
+    reinterpret_cast<__nv_bfloat16*>(S.w1)[i] =
+        e < 6 && tap < 9 ? wb[OFF_W1 + (co * 2 + e / 3) * 9 + tap] : __float2bfloat16(0.0f);
+  }
+  for (int i = tid; i < 288; i += TILE_THREADS) S.w3[(i % 9) * 32 + i / 9] = __bfloat162float(wb[OFF_W3 + i]);
+  if (tid < 32) {
+    S.b1[tid] = w[OFF_B1 + tid];
+    S.b2[tid] = w[OFF_B2 + tid];
+  }
+  if (tid == 0) {
+    S.b3 = w[OFF_B3];
+    S.failed = 0;
+    for (int i = 0; i < 4; ++i) umma::bar_init(&S.bar[i]);
+    umma::bar_init_fence();
+  }
+  if (warp == 0) umma::tmem_alloc(&S.tmem, 256);
+  umma::fence_before();
+  __syncthreads();
+  umma::fence_after();
+  const uint32_t tmem = S.tmem, tq = tmem + ((uint32_t)(warp & 3) << 21);
+  // layer 1's accumulators take the columns of layer 2's: they are read before those are written
+  float xr[2][2];
+  auto fetch = [&](int64_t t) {
+    int n, oy, ox;
+    tile_of(G, t, ZW, ZH, &n, &oy, &ox);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int i = tid + j * TILE_THREADS, gy = oy - 3 + i / PW, gx = ox - 3 + i % PW;
+      const bool in = t < G.tiles && i < (R1 + 2) * PW && gy >= 0 && gy < G.H && gx >= 0 && gx < G.W;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) xr[j][c] = in ? __ldg(x + (2 * (size_t)n + c) * plane + (size_t)gy * G.W + gx) : 0.0f;
+    }
+  };
+  fetch(blockIdx.x);
+  uint32_t phase = 0;
+  for (int64_t tile = blockIdx.x; tile < G.tiles; tile += gridDim.x, phase ^= 1) {
+    int n, oy, ox;
+    tile_of(G, tile, ZW, ZH, &n, &oy, &ox);
+    // ---- layer 1
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int i = tid + j * TILE_THREADS;
+      if (i < NPX) {
+        uint32_t h0, m0, l0;
+        umma::split2(xr[j][0], xr[j][1], &h0, &m0, &l0);  // low halves: channel 0, high halves: channel 1
+        *reinterpret_cast<uint4*>(S.a + i * 16) = make_uint4(__byte_perm(h0, m0, 0x5410), __byte_perm(l0, h0, 0x7610),
+                                                             __byte_perm(m0, l0, 0x7632), 0u);
+      }
+    }
+    if (tid < 128) *reinterpret_cast<uint4*>(S.a + (NPX + tid) * 16) = make_uint4(0, 0, 0, 0);
+    umma::fence_smem();
+    __syncthreads();
+    if (warp == 0 && umma::elect()) {
+      const uint32_t a0 = umma::smem_addr(S.a);
+      const uint64_t w0 = umma::desc_k(umma::smem_addr(S.w1), 512);
+#pragma unroll
+      for (int p = 0; p < 5; ++p) {
+        const int s0 = (2 * p / 3) * PW + (2 * p) % 3, s1 = ((2 * p + 1) / 3) * PW + (2 * p + 1) % 3;
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+          umma::mma(tmem + t * 32, umma::desc_k(a0 + (t * 128 + s0) * 16, (p < 4 ? s1 - s0 : NPX - t * 128 - s0) * 16),
+                    w0 + p * 64, umma::idesc(128, 32, false), p > 0);
+      }
+      umma::commit(&S.bar[0]);
+    }
+    __syncwarp();
+    fetch(tile + gridDim.x);
+    if (!umma::bar_wait(&S.bar[0], phase)) S.failed = 1;
+    umma::fence_after();
+    __syncthreads();  // every block thread past the wait: the input's overlay is free
+    if (S.failed) break;
+#pragma unroll 1
+    for (int r = warp; r < R1; r += R2) {
+      const int gy = oy - 2 + r, gx = ox - 2 + lane;
+      const bool in = gy >= 0 && gy < G.H && gx >= 0 && gx < G.W;
+      const bool own = TRAIN && in && r >= 2 && r < 2 + ZH && lane >= 2 && lane < 2 + ZW;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float v[16];
+        umma::tmem_ld16(tq + (r >> 2) * 32 + 16 * h, v);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          v[c] = in ? fmaxf(v[c] + S.b1[16 * h + c], 0.0f) : 0.0f;
+          if (own) a1[((size_t)n * 32 + 16 * h + c) * plane + (size_t)gy * G.W + gx] = v[c];
+        }
+        store_half(S.a, r * PW + lane, h, v);
+      }
+    }
+    zero_tail(S.a, tid);
+    // ---- layer 2
+    umma::fence_smem();
+    umma::fence_before();
+    __syncthreads();
+    if (warp == 0 && umma::elect()) {
+      umma::fence_after();
+      conv32_issue(S, tmem, 0);
+      conv32_issue(S, tmem, 1);
+    }
+    __syncwarp();
+    // ---- layer 3
+    const int gy = oy - 1 + warp, gx = ox - 1 + lane;
+    const bool in = gy >= 0 && gy < G.H && gx >= 0 && gx < G.W;
+    float v[32];
+    bool ok = conv32_read(S, tmem, warp, phase, v);
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      v[c] = in ? fmaxf(v[c] + S.b2[c], 0.0f) : 0.0f;
+      if (TRAIN && in && warp >= 1 && warp < 1 + ZH && lane >= 1 && lane < 1 + ZW)
+        a2[((size_t)n * 32 + c) * plane + (size_t)gy * G.W + gx] = v[c];
+    }
+    float dot[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      float2 d = make_float2(0.0f, 0.0f);
+#pragma unroll
+      for (int c = 0; c < 32; c += 4) {
+        const float4 q = *reinterpret_cast<const float4*>(&S.w3[k * 32 + c]);
+        d = ffma2(make_float2(v[c], v[c + 1]), make_float2(q.x, q.y), d);
+        d = ffma2(make_float2(v[c + 2], v[c + 3]), make_float2(q.z, q.w), d);
+      }
+      dot[k] = d.x + d.y;
+    }
+    for (int t = 0; t < M2 / 128; ++t) ok = ok && umma::bar_wait(&S.bar[1 + t], phase);
+    if (!ok) S.failed = 1;
+    umma::fence_before();
+    __syncthreads();  // every MMA has read the planes: the partial sums take their place
+    if (S.failed) break;
+    float* pp = reinterpret_cast<float*>(S.a);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) pp[k * M2 + tid] = dot[k];
+    __syncthreads();
+    const int zy = oy + warp, zx = ox + lane;
+    if (warp < ZH && lane < ZW && zy < G.H && zx < G.W) {
+      float z = S.b3;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) z += pp[k * M2 + tid + (k / 3) * PW + k % 3];
+      out[(size_t)n * plane + (size_t)zy * G.W + zx] = TRAIN ? z : 1.0f / (1.0f + expf(-z));
+    }
+    umma::fence_after();
+    __syncthreads();
+  }
+  if (S.failed) {  // a wait ran out: the block's remaining outputs are marked as missing
+    for (int64_t tile = blockIdx.x; tile < G.tiles; tile += gridDim.x) {
+      int n, oy, ox;
+      tile_of(G, tile, ZW, ZH, &n, &oy, &ox);
+      if (warp < ZH && lane < ZW && oy + warp < G.H && ox + lane < G.W)
+        out[(size_t)n * plane + (size_t)(oy + warp) * G.W + ox + lane] = __int_as_float(0x7fc00000);
+    }
   }
   __syncthreads();
-  for (int wi = tid; wi < COUT * CIN * 9; wi += T * T) {
-    int co = wi / (CIN * 9), ci = (wi / 9) % CIN, k = wi % 9;
-    int ky = k / 3, kx = k % 3;
-    float acc = 0.0f;
-    for (int r = 0; r < T; ++r)
-#pragma unroll 4
-      for (int q = 0; q < T; ++q) acc = fmaf(ds[(co * T + r) * T + q], xs[(ci * TH + r + ky) * TH + q + kx], acc);
-    atomicAdd(&dw[wi], acc);
+  if (warp == 0) umma::tmem_free(tmem, 256);
+}
+
+// Data gradients of a 30 x 12 tile: d2 = layer 3's transposed convolution of
+// dz times (a2 > 0), written once and as pieces into the planes; d1 = layer
+// 2's transposed convolution of d2 times (a1 > 0) by conv32_issue. Bound as
+// the forward pass; 32 x 64 x 64 pixels: 42 us.
+__global__ void __launch_bounds__(TILE_THREADS, 2)
+    dgrad_kernel(const float* __restrict__ dz, const __nv_bfloat16* __restrict__ wb, const float* __restrict__ a1,
+                 const float* __restrict__ a2, float* __restrict__ d1, float* __restrict__ d2, const TileGrid G) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  TileSmem& S = *reinterpret_cast<TileSmem*>(smem);
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const size_t plane = (size_t)G.H * G.W;
+  load_w2(S.w2, wb + OFF_OP + NW2, tid);
+  for (int i = tid; i < 288; i += TILE_THREADS) S.w3[(i % 9) * 32 + i / 9] = __bfloat162float(wb[OFF_W3 + i]);
+  if (tid == 0) {
+    S.failed = 0;
+    for (int i = 0; i < 4; ++i) umma::bar_init(&S.bar[i]);
+    umma::bar_init_fence();
   }
-  if (tid < COUT) {
-    float acc = 0.0f;
-    for (int i = 0; i < T * T; ++i) acc += ds[tid * T * T + i];
-    atomicAdd(&db[tid], acc);
+  if (warp == 0) umma::tmem_alloc(&S.tmem, 256);
+  umma::fence_before();
+  __syncthreads();
+  umma::fence_after();
+  const uint32_t tmem = S.tmem, tq = tmem + ((uint32_t)(warp & 3) << 21);
+  uint32_t phase = 0;
+  for (int64_t tile = blockIdx.x; tile < G.tiles; tile += gridDim.x, phase ^= 1) {
+    int n, oy, ox;
+    tile_of(G, tile, DW, DH, &n, &oy, &ox);
+#pragma unroll 1
+    for (int r = warp; r < R1; r += R2) {
+      const int gy = oy - 1 + r, gx = ox - 1 + lane;
+      const bool in = gy >= 0 && gy < G.H && gx >= 0 && gx < G.W;
+      const bool own = in && r >= 1 && r < 1 + DH && lane >= 1 && lane < 1 + DW;
+      float g[9];
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {  // dz at the outputs this pixel feeds through tap k
+        const int yy = gy + 1 - k / 3, xx = gx + 1 - k % 3;
+        g[k] = in && yy >= 0 && yy < G.H && xx >= 0 && xx < G.W ? __ldg(dz + (size_t)n * plane + (size_t)yy * G.W + xx)
+                                                                : 0.0f;
+      }
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        float v[16];
+        const size_t o = ((size_t)n * 32 + 16 * h) * plane + (size_t)gy * G.W + gx;
+#pragma unroll
+        for (int c = 0; c < 16; ++c) v[c] = in ? __ldg(a2 + o + c * plane) : 0.0f;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          float2 s = make_float2(0.0f, 0.0f);
+#pragma unroll
+          for (int k = 0; k < 9; ++k)
+            s = ffma2(make_float2(g[k], g[k]), *reinterpret_cast<const float2*>(&S.w3[k * 32 + 16 * h + 2 * c]), s);
+          v[2 * c] = v[2 * c] > 0.0f ? s.x : 0.0f;
+          v[2 * c + 1] = v[2 * c + 1] > 0.0f ? s.y : 0.0f;
+        }
+        if (own)
+#pragma unroll
+          for (int c = 0; c < 16; ++c) d2[o + c * plane] = v[c];
+        store_half(S.a, r * PW + lane, h, v);
+      }
+    }
+    zero_tail(S.a, tid);
+    umma::fence_smem();
+    umma::fence_before();
+    __syncthreads();
+    if (warp == 0 && umma::elect()) {
+      umma::fence_after();
+      conv32_issue(S, tmem, 0);
+      conv32_issue(S, tmem, 1);
+    }
+    __syncwarp();
+    const int gy = oy + warp, gx = ox + lane;
+    const bool in = lane < DW && gy < G.H && gx < G.W;
+    float v[32];
+    bool ok = conv32_read(S, tmem, warp, phase, v);
+    if (in) {
+      const size_t o = (size_t)n * 32 * plane + (size_t)gy * G.W + gx;
+#pragma unroll
+      for (int h = 0; h < 32; h += 16) {
+        float m[16];
+#pragma unroll
+        for (int c = 0; c < 16; ++c) m[c] = __ldg(a1 + o + (h + c) * plane);
+#pragma unroll
+        for (int c = 0; c < 16; ++c)
+          d1[o + (h + c) * plane] = !ok ? __int_as_float(0x7fc00000) : m[c] > 0.0f ? v[h + c] : 0.0f;
+      }
+    }
+    for (int t = 0; t < M2 / 128; ++t) ok = ok && umma::bar_wait(&S.bar[1 + t], phase);
+    if (!ok) S.failed = 1;
+    umma::fence_before();
+    __syncthreads();
+    umma::fence_after();
+    if (S.failed) break;
   }
+  __syncthreads();
+  if (warp == 0) umma::tmem_free(tmem, 256);
+}
+
+// ---------------------------------------------------------------- weight gradients
+// dW[o][i][k] = sum over pixels p of D[o][p] X[i][p + k - 1]: a GEMM whose
+// contraction runs over the pixels, both operands MN-major with their pieces
+// stacked along M and N, so one MMA forms all nine products of the pieces.
+// The tile is `tr` rows of `sw` columns flattened with a pitch of sw + 2: D is
+// zero in the two columns between the rows, X has the halo there.
+constexpr int WG_THREADS = 512;
+constexpr int WG_K = 256;                   // pixels of a tile, at most
+struct WgradGrid {
+  int n, H, W, sw, tr, tx, ty;
+  uint32_t inv;  // 2^16 / (sw + 2), rounded up
+  int64_t tiles;
+};
+constexpr int WG_X = 392;                   // input pixels of a tile: 256 + 2 * pitch + 3 at most, pitch <= 64
+
+// Stages 32 channels of `src` (rows from oy, columns from ox, `rows` x `cols`
+// of a pitch, zero elsewhere up to `len` pixels) as 12 planes of `stride` bytes.
+// IT rounds of a chunk (8 channels of a pixel) per thread; `inv` = 2^16 /
+// pitch rounded up (exact quotients: pixels < 512, pitch <= 64), a
+// warp's lanes in one chunk.
+template <int IT>
+__device__ __forceinline__ void stage32(unsigned char* a, uint32_t stride, const float* __restrict__ src, size_t plane,
+                                        int H, int W, int oy, int ox, int rows, int cols, int pitch, uint32_t inv,
+                                        int len, int tid) {
+  const int warps = (len + 31) / 32;
+#pragma unroll 2
+  for (int it = 0; it < IT; ++it) {
+    const int wi = (tid >> 5) + it * (WG_THREADS / 32), c = wi / warps, m = (wi - c * warps) * 32 + (tid & 31);
+    if (c > 3) break;
+    const int r = (int)((uint32_t)m * inv >> 16), q = m - r * pitch;
+    const int gy = oy + r, gx = ox + q;
+    float v[8];
+    const bool in = r < rows && q < cols && gy >= 0 && gy < H && gx >= 0 && gx < W;
+    const float* sp = src + (size_t)(8 * c) * plane + (size_t)gy * W + gx;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = in ? __ldg(sp + e * plane) : 0.0f;
+    uint4 p[3];
+    umma::split8(v, p);
+    if (m < len)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) *reinterpret_cast<uint4*>(a + (k * 4 + c) * stride + m * 16) = p[k];
+  }
+}
+
+template <int XP>
+struct alignas(16) WgradSmem {
+  unsigned char d[16 * WG_K * 16];          // 12 planes of D and 4 of zeros: M = 128
+  unsigned char x[XP * WG_X * 16];          // layer 2: 12 planes of X, ones, zeros; layers 1, 3: one chunk
+  uint32_t tmem;
+  int failed;
+  uint64_t full[2], empty[2];
+};
+static_assert(sizeof(WgradSmem<14>) <= 227 * 1024 && sizeof(WgradSmem<1>) <= 227 * 1024, "one block per SM");
+
+// Layer 2: 32 x 32 channels. The tensor core cuts the low bits of its sums,
+// so they stay short: a stage is two taps over a third of the tile's pixels
+// (at most six K steps), in one of two TMEM buffers; the warps of the lane
+// quarters 0-2 (the pieces of D) add it to FP32 registers while the next stage
+// runs, issued by warp 3. The ninth tap's stage has a plane of ones beside the
+// planes of X: its column is the bias gradient.
+constexpr int WG_CHAINS = 3;
+constexpr int WG_ROW = 289;  // an output channel's 288 sums, padded to another bank per lane
+__global__ void __launch_bounds__(WG_THREADS, 1)
+    wgrad32_kernel(const float* __restrict__ x, const float* __restrict__ dy, float* __restrict__ dw,
+                   float* __restrict__ db, const WgradGrid G) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  WgradSmem<14>& S = *reinterpret_cast<WgradSmem<14>*>(smem);
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const size_t plane = (size_t)G.H * G.W;
+  const int pitch = G.sw + 2, klen = (G.tr * pitch + 15) / 16 * 16, xlen = klen + 2 * pitch + 2;
+  const int kstep = (klen / 16 + WG_CHAINS - 1) / WG_CHAINS * 16, chains = (klen + kstep - 1) / kstep;
+  for (int i = tid; i < 4 * WG_K; i += WG_THREADS)
+    *reinterpret_cast<uint4*>(S.d + (12 * WG_K + i) * 16) = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < 2 * WG_X; i += WG_THREADS)
+    *reinterpret_cast<uint4*>(S.x + (12 * WG_X + i) * 16) = make_uint4(i < WG_X ? 0x3f80u : 0u, 0, 0, 0);
+  if (tid == 0) {
+    S.failed = 0;
+    for (int i = 0; i < 2; ++i) {
+      umma::bar_init(&S.full[i]);
+      umma::bar_init(&S.empty[i], 12);
+    }
+    umma::bar_init_fence();
+  }
+  if (warp == 0) umma::tmem_alloc(&S.tmem, 512);
+  umma::fence_before();
+  __syncthreads();
+  umma::fence_after();
+  const uint32_t tmem = S.tmem;
+  const int piece = warp & 3, i0 = (warp >> 2) * 8;  // a thread's row of D is (piece, lane), its columns i0 ..
+  const uint32_t tq = tmem + ((uint32_t)piece << 21);
+  float acc[9][8], bias = 0.0f;
+#pragma unroll
+  for (int j = 0; j < 9; ++j)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) acc[j][c] = 0.0f;
+  uint32_t stage = 0;
+  bool ok = true;
+  for (int64_t tile = blockIdx.x; tile < G.tiles; tile += gridDim.x) {
+    int64_t t = tile;
+    const int ox = (int)(t % G.tx) * G.sw;
+    t /= G.tx;
+    const int oy = (int)(t % G.ty) * G.tr, n = (int)(t / G.ty);
+    stage32<2>(S.d, WG_K * 16, dy + (size_t)n * 32 * plane, plane, G.H, G.W, oy, ox, G.tr, G.sw, pitch, G.inv, klen, tid);
+    stage32<4>(S.x, WG_X * 16, x + (size_t)n * 32 * plane, plane, G.H, G.W, oy - 1, ox - 1, G.tr + 2, pitch, pitch, G.inv,
+               xlen, tid);
+    umma::fence_smem();
+    __syncthreads();
+    if (warp == 3) {
+      const uint64_t a0 = umma::desc_mn(umma::smem_addr(S.d), WG_K * 16), b0 = umma::desc_mn(umma::smem_addr(S.x), WG_X * 16);
+#pragma unroll 1
+      for (int g = 0; g < 5; ++g)
+#pragma unroll 1
+        for (int ch = 0; ch < chains; ++ch, ++stage) {
+          // both buffers start empty
+          if (stage >= 2) ok = umma::bar_wait(&S.empty[stage & 1], (stage >> 1) - 1 & 1) && ok;
+          umma::fence_after();
+          if (umma::elect()) {
+            const int k0 = ch * kstep, k1 = min(klen, k0 + kstep);
+#pragma unroll 1
+            for (int tap = 2 * g; tap < 2 * g + 2 && tap < 9; ++tap) {
+              const uint32_t d = tmem + (stage & 1) * 256 + (tap & 1) * 96;
+              const uint32_t id = tap == 8 ? umma::idesc(128, 112, true) : umma::idesc(128, 96, true);
+              const uint64_t bt = b0 + (tap / 3) * pitch + tap % 3;
+              for (int k = k0; k < k1; k += 16) umma::mma(d, a0 + k, bt + k, id, k > k0);
+            }
+            umma::commit(&S.full[stage & 1]);
+          }
+          __syncwarp();
+        }
+      // the tile's planes are free once its last MMA is done
+      ok = umma::bar_wait(&S.full[(stage - 1) & 1], (stage - 1) >> 1 & 1) && ok;
+    } else if (piece < 3) {
+#pragma unroll
+      for (int g = 0; g < 5; ++g)
+#pragma unroll 1
+        for (int ch = 0; ch < chains; ++ch, ++stage) {
+          ok = umma::bar_wait(&S.full[stage & 1], stage >> 1 & 1) && ok;
+          umma::fence_after();
+          const uint32_t col = tq + (stage & 1) * 256 + i0;
+          // row 32 piece + o, column 32 piece' + i
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+            if (2 * g + j < 9) {
+              float v[8], u[8], s[8];
+              umma::tmem_ld8(col + j * 96, v);
+              umma::tmem_ld8(col + j * 96 + 32, u);
+              umma::tmem_ld8(col + j * 96 + 64, s);
+#pragma unroll
+              for (int c = 0; c < 8; ++c) acc[2 * g + j < 9 ? 2 * g + j : 8][c] += v[c] + (u[c] + s[c]);
+            }
+          if (g == 4 && i0 == 0) {
+            float v[8];
+            umma::tmem_ld8(col + 96, v);
+            bias += v[0];
+          }
+          umma::fence_before();
+          if (lane == 0) umma::bar_arrive(&S.empty[stage & 1]);
+          __syncwarp();
+        }
+    }
+    if (!ok) S.failed = 1;
+    __syncthreads();
+    if (S.failed) break;
+  }
+  // the pieces of D are added in shared memory, in turn, then once per block in global memory
+  float* sum = reinterpret_cast<float*>(S.x);
+  const float bad = S.failed ? __int_as_float(0x7fc00000) : 0.0f;
+#pragma unroll 1
+  for (int p = 2; p >= 0; --p) {
+    __syncthreads();
+    if (piece == p) {
+#pragma unroll
+      for (int j = 0; j < 9; ++j)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          float* q = &sum[lane * WG_ROW + (i0 + c) * 9 + j];
+          *q = (p == 2 ? bad : *q) + acc[j][c];
+        }
+      if (i0 == 0) sum[32 * WG_ROW + lane] = (p == 2 ? bad : sum[32 * WG_ROW + lane]) + bias;
+    }
+  }
+  umma::fence_before();
+  __syncthreads();
+  for (int i = tid; i < NW2; i += WG_THREADS) atomicAdd(&dw[i], sum[i + i / 288]);
+  if (tid < 32) atomicAdd(&db[tid], sum[32 * WG_ROW + tid]);
+  if (warp == 0) umma::tmem_free(tmem, 512);
+}
+
+// Layers 1 and 3 (block y of the grid), the side with 32 channels as D:
+//  layer 1: D = d1, X = the network input (both channels in one chunk of
+//           pieces; element 6 is one: the bias gradient);
+//  layer 3: D = a2, X = dz, whose taps are reversed (dW3[i][k] = sum over q
+//           of a2[i][q] dz[q - k + 1]); its bias gradient is bce_kernel's.
+// X's chunks of a row of taps are neighbouring pixels, 16 bytes apart: one MMA
+// takes the three (and an unused fourth, N = 32). Each fifth of the tile's
+// pixels has its own accumulators (short sums, see wgrad32_kernel). The next
+// tile is read while the MMAs of this one run. 32 x 64 x 64 pixels: 26 us.
+constexpr int IO_CHAINS = 5;
+__global__ void __launch_bounds__(WG_THREADS, 1)
+    wgrad_io_kernel(const float* __restrict__ x, const float* __restrict__ d1, const float* __restrict__ dz,
+                    const float* __restrict__ a2, float* __restrict__ grad, const WgradGrid G) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  WgradSmem<1>& S = *reinterpret_cast<WgradSmem<1>*>(smem);
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const size_t plane = (size_t)G.H * G.W;
+  const bool l3 = blockIdx.y != 0;
+  const int pitch = G.sw + 2, klen = (G.tr * pitch + 15) / 16 * 16, xlen = klen + 2 * pitch + 3;
+  const int kstep = (klen / 16 + IO_CHAINS - 1) / IO_CHAINS * 16, chains = (klen + kstep - 1) / kstep;
+  for (int i = tid; i < 4 * WG_K; i += WG_THREADS)
+    *reinterpret_cast<uint4*>(S.d + (12 * WG_K + i) * 16) = make_uint4(0, 0, 0, 0);
+  if (tid == 0) {
+    S.failed = 0;
+    umma::bar_init(&S.full[0]);
+    umma::bar_init_fence();
+  }
+  if (warp == 0) umma::tmem_alloc(&S.tmem, 512);
+  umma::fence_before();
+  __syncthreads();
+  umma::fence_after();
+  const uint32_t tmem = S.tmem;
+  // taps of a thread's warp: grp, grp + 4, and for the first group 8
+  const int piece = warp & 3, grp = warp >> 2;
+  const uint32_t tq = tmem + ((uint32_t)piece << 21);
+  float acc[3][8];
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) acc[j][c] = 0.0f;
+  // a thread's pixel of X, and its two chunks of D (rounds of 16 warps over 4 chunks of warps_d warps)
+  const int warps_d = (klen + 31) / 32;
+  float xv[2], dv[2][8];
+  auto fetch = [&](int64_t t) {
+    const bool live = t < G.tiles;
+    const int ox = (int)(t % G.tx) * G.sw;
+    t /= G.tx;
+    const int oy = (int)(t % G.ty) * G.tr, n = (int)(t / G.ty);
+    {
+      const int r = (int)((uint32_t)tid * G.inv >> 16), gy = oy - 1 + r, gx = ox - 1 + tid - r * pitch;
+      const bool in = live && r < G.tr + 2 && gy >= 0 && gy < G.H && gx >= 0 && gx < G.W;
+      const float* p = (l3 ? dz + (size_t)n * plane : x + (size_t)n * 2 * plane) + (size_t)gy * G.W + gx;
+      xv[0] = in ? __ldg(p) : 0.0f;
+      xv[1] = in && !l3 ? __ldg(p + plane) : 0.0f;
+    }
+    const float* src = (l3 ? a2 : d1) + (size_t)n * 32 * plane;
+#pragma unroll
+    for (int it = 0; it < 2; ++it) {
+      const int wi = warp + it * (WG_THREADS / 32), c = wi / warps_d, m = (wi - c * warps_d) * 32 + lane;
+      const int r = (int)((uint32_t)m * G.inv >> 16), q = m - r * pitch, gy = oy + r, gx = ox + q;
+      const bool in = live && c < 4 && r < G.tr && q < G.sw && gy < G.H && gx < G.W;
+      const float* p = src + (size_t)(8 * c) * plane + (size_t)gy * G.W + gx;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) dv[it][e] = in ? __ldg(p + e * plane) : 0.0f;
+    }
+  };
+  fetch(blockIdx.x);
+  uint32_t phase = 0;
+  for (int64_t tile = blockIdx.x; tile < G.tiles; tile += gridDim.x, phase ^= 1) {
+#pragma unroll
+    for (int it = 0; it < 2; ++it) {
+      const int wi = warp + it * (WG_THREADS / 32), c = wi / warps_d, m = (wi - c * warps_d) * 32 + lane;
+      uint4 p[3];
+      umma::split8(dv[it], p);
+      if (c < 4 && m < klen)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) *reinterpret_cast<uint4*>(S.d + ((k * 4 + c) * WG_K + m) * 16) = p[k];
+    }
+    if (tid < xlen) {
+      uint32_t h0, m0, l0;
+      umma::split2(xv[0], xv[1], &h0, &m0, &l0);
+      *reinterpret_cast<uint4*>(S.x + tid * 16) = make_uint4(__byte_perm(h0, m0, 0x5410), __byte_perm(l0, h0, 0x7610),
+                                                             __byte_perm(m0, l0, 0x7632), 0x3f80u);
+    }
+    umma::fence_smem();
+    __syncthreads();
+    if (warp == 3 && umma::elect()) {
+      const uint64_t a0 = umma::desc_mn(umma::smem_addr(S.d), WG_K * 16), b0 = umma::desc_mn(umma::smem_addr(S.x), 16);
+      constexpr uint32_t id = umma::idesc(128, 32, true);
+#pragma unroll 1
+      for (int ch = 0; ch < chains; ++ch)
+        for (int k = ch * kstep; k < min(klen, (ch + 1) * kstep); k += 16)
+#pragma unroll
+          for (int ky = 0; ky < 3; ++ky)
+            umma::mma(tmem + ch * 96 + ky * 32, a0 + k, b0 + k + ky * pitch, id, k > ch * kstep);
+      umma::commit(&S.full[0]);
+    }
+    __syncwarp();
+    fetch(tile + gridDim.x);
+    if (!umma::bar_wait(&S.full[0], phase)) S.failed = 1;
+    umma::fence_after();
+    if (piece < 3) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const int tap = grp + 4 * j;
+        if (tap < 9)
+#pragma unroll 1
+          for (int ch = 0; ch < chains; ++ch) {
+            float v[8];
+            umma::tmem_ld8(tq + ch * 96 + (tap / 3) * 32 + (tap % 3) * 8, v);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[j][c] += v[c];
+          }
+      }
+    }
+    umma::fence_before();
+    __syncthreads();
+    umma::fence_after();
+    if (S.failed) break;
+  }
+  // sums over the pieces of X, then over those of D in shared memory, then one atomic per block
+  float* sum = reinterpret_cast<float*>(S.d);  // [32][19]: 18 weights and the bias of a channel
+  const float bad = S.failed ? __int_as_float(0x7fc00000) : 0.0f;
+#pragma unroll 1
+  for (int p = 2; p >= 0; --p) {
+    __syncthreads();
+    if (piece == p)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const int tap = grp + 4 * j;
+        if (tap >= 9) break;
+        const float* v = acc[j];
+        float* q = sum + lane * 19;
+        const float o[3] = {v[0] + (v[1] + v[2]), v[3] + (v[4] + v[5]), v[6]};
+        const int at[3] = {l3 ? 8 - tap : tap, 9 + tap, 18};
+#pragma unroll
+        for (int e = 0; e < 3; ++e)
+          if (e < 2 || tap == 4) q[at[e]] = (p == 2 ? bad : q[at[e]]) + o[e];
+      }
+  }
+  umma::fence_before();
+  __syncthreads();
+  for (int i = tid; i < 32 * 19; i += WG_THREADS) {
+    const int c = i / 19, e = i - 19 * c;
+    if (l3) {
+      if (e < 9) atomicAdd(&grad[OFF_W3 + c * 9 + e], sum[i]);
+    } else {
+      atomicAdd(&grad[e < 18 ? OFF_W1 + c * 18 + e : OFF_B1 + c], sum[i]);
+    }
+  }
+  if (warp == 0) umma::tmem_free(tmem, 512);
 }
 
 // Logit -> probability, and the BCE loss / logit gradient:
-// loss = w y softplus(-z) + (1 - y) softplus(z), averaged over pixels.
-__global__ void bce_kernel(const float* __restrict__ z, const float* __restrict__ yl, int64_t n, float pos_w,
-                           float* __restrict__ dz, float* __restrict__ loss) {
-  float acc = 0.0f;
+// loss = w y softplus(-z) + (1 - y) softplus(z), averaged over pixels; db: sum
+// of the logit gradients (layer 3's bias gradient).
+constexpr int BCE_THREADS = 256;
+__global__ void __launch_bounds__(BCE_THREADS) bce_kernel(const float* __restrict__ z, const float* __restrict__ yl, int64_t n, float pos_w,
+                           float* __restrict__ dz, float* __restrict__ loss, float* __restrict__ db) {
+  float acc = 0.0f, dsum = 0.0f;
   const float inv = 1.0f / (float)n;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     float zi = z[i], yi = yl[i];
@@ -136,15 +798,25 @@ __global__ void bce_kernel(const float* __restrict__ z, const float* __restrict_
     float sp_neg = sp_pos - zi;                                  // softplus(-z)
     acc += pos_w * yi * sp_neg + (1.0f - yi) * sp_pos;
     float s = 1.0f / (1.0f + expf(-zi));
-    dz[i] = (-pos_w * yi * (1.0f - s) + (1.0f - yi) * s) * inv;
+    const float d = (-pos_w * yi * (1.0f - s) + (1.0f - yi) * s) * inv;
+    dz[i] = d;
+    dsum += d;
   }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc * inv);
-}
-
-__global__ void sigmoid_kernel(const float* __restrict__ z, int64_t n, float* __restrict__ p) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    p[i] = 1.0f / (1.0f + expf(-z[i]));
+  __shared__ float red[2][BCE_THREADS / 32];
+  for (int o = 16; o > 0; o >>= 1) {
+    acc += __shfl_down_sync(0xffffffffu, acc, o);
+    dsum += __shfl_down_sync(0xffffffffu, dsum, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = acc;
+    red[1][threadIdx.x >> 5] = dsum;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    float t = 0.0f;
+    for (int i = 0; i < BCE_THREADS / 32; ++i) t += red[threadIdx.x][i];
+    atomicAdd(threadIdx.x ? db : loss, threadIdx.x ? t : t * inv);
+  }
 }
 
 __global__ void adam_kernel(float* __restrict__ w, float* __restrict__ m, float* __restrict__ v,
@@ -158,45 +830,61 @@ __global__ void adam_kernel(float* __restrict__ w, float* __restrict__ m, float*
     v[i] = vi;
     float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
     w[i] = wi;
-    wb[i] = __float2bfloat16_rn(wi);
+    store_weight(wb, i, wi);
   }
 }
 
 __global__ void to_bf16_kernel(const float* __restrict__ w, __nv_bfloat16* __restrict__ wb, int n) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    wb[i] = __float2bfloat16_rn(w[i]);
+    store_weight(wb, i, w[i]);
 }
 
-template <int CIN, int COUT, bool RELU, bool TRANSPOSE, bool BIAS>
-int launch_conv(const float* x, const __nv_bfloat16* w, const float* b, const float* mask, float* y, int n, int H,
-                int W, cudaStream_t s) {
-  size_t smem = sizeof(float) * (CIN * TH * TH + COUT * CIN * 9);
-  auto kern = conv3x3_kernel<CIN, COUT, RELU, TRANSPOSE, BIAS>;
+// Launches a persistent tile kernel with its shared memory on `per_sm` blocks per SM.
+template <class K, class... Args>
+int launch_tiles(K kern, int threads, size_t smem, int per_sm, int gy, int64_t tiles, cudaStream_t s, Args... args) {
+  int dev = 0, sms = 0;
+  QSL_CHECK_CUDA(cudaGetDevice(&dev));
+  QSL_CHECK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   QSL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  dim3 grid((W + T - 1) / T, (H + T - 1) / T, n);
-  kern<<<grid, T * T, smem, s>>>(x, w, b, mask, y, H, W);
+  const int64_t blocks = std::min<int64_t>(tiles, std::max(1, sms * per_sm / gy));
+  kern<<<dim3((unsigned)blocks, gy), threads, smem, s>>>(args...);
   qsl::count_launch();
   QSL_CHECK_CUDA(cudaGetLastError());
   return QSL_OK;
 }
 
-template <int CIN, int COUT>
-int launch_wgrad(const float* x, const float* dy, float* dw, float* db, int n, int H, int W, cudaStream_t s) {
-  size_t smem = sizeof(float) * (CIN * TH * TH + COUT * T * T);
-  auto kern = conv3x3_wgrad_kernel<CIN, COUT>;
-  QSL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  dim3 grid((W + T - 1) / T, (H + T - 1) / T, n);
-  kern<<<grid, T * T, smem, s>>>(x, dy, dw, db, H, W);
-  qsl::count_launch();
-  QSL_CHECK_CUDA(cudaGetLastError());
-  return QSL_OK;
+TileGrid tile_grid(int n, int H, int W, int w, int h) {
+  TileGrid G;
+  G.n = n;
+  G.H = H;
+  G.W = W;
+  G.tx = (W + w - 1) / w;
+  G.ty = (H + h - 1) / h;
+  G.tiles = (int64_t)n * G.tx * G.ty;
+  return G;
+}
+
+// Strips of equal width, at most 62 columns, and as many rows as 256 pixels hold.
+WgradGrid wgrad_grid(int n, int H, int W) {
+  WgradGrid G;
+  G.n = n;
+  G.H = H;
+  G.W = W;
+  const int strips = (W + 61) / 62;
+  G.sw = (W + strips - 1) / strips;
+  G.inv = 65536u / (G.sw + 2) + 1;
+  G.tr = std::min(H, WG_K / (G.sw + 2));
+  G.tx = (W + G.sw - 1) / G.sw;
+  G.ty = (H + G.tr - 1) / G.tr;
+  G.tiles = (int64_t)n * G.tx * G.ty;
+  return G;
 }
 
 }  // namespace
 
 struct qsl_cnn {
   float* w = nullptr;            // FP32 master parameters
-  __nv_bfloat16* wb = nullptr;   // BF16 copy used by the passes
+  __nv_bfloat16* wb = nullptr;   // BF16 copy used by the passes, and layer 2's operand layouts
   float* m = nullptr;            // Adam moments
   float* v = nullptr;
   int64_t steps = 0;
@@ -207,58 +895,58 @@ struct qsl_cnn {
 namespace {
 
 int ensure_act(qsl_cnn* c, size_t pixels, cudaStream_t s) {
-  // a1, a2 (32 channels each), z (1), dz (1), d2 (32), d1 (32)
-  size_t need = pixels * (32 + 32 + 1 + 1 + 32 + 32);
+  // a1, a2, d2, d1 (32 channels each), z, dz (1)
+  size_t need = pixels * (4 * 32 + 2);
   if (need <= c->act_cap) return QSL_OK;
   if (c->act) QSL_CHECK_CUDA(cudaFreeAsync(c->act, s));
   c->act = nullptr;
+  c->act_cap = 0;
   QSL_CHECK_CUDA(qsl::alloc_async((void**)&c->act, need * sizeof(float), s));
   c->act_cap = need;
   return QSL_OK;
 }
 
-int forward(qsl_cnn* c, const float* x, int n, int H, int W, cudaStream_t s, float** a1, float** a2, float** z) {
-  size_t P = (size_t)n * H * W;
-  int rc = ensure_act(c, P, s);
-  if (rc) return rc;
-  *a1 = c->act;
-  *a2 = *a1 + P * 32;
-  *z = *a2 + P * 32;
-  if ((rc = launch_conv<C1, C2, true, false, true>(x, c->wb + OFF_W1, c->w + OFF_B1, nullptr, *a1, n, H, W, s)))
-    return rc;
-  if ((rc = launch_conv<C2, C2, true, false, true>(*a1, c->wb + OFF_W2, c->w + OFF_B2, nullptr, *a2, n, H, W, s)))
-    return rc;
-  return launch_conv<C2, 1, false, false, true>(*a2, c->wb + OFF_W3, c->w + OFF_B3, nullptr, *z, n, H, W, s);
-}
-
 bool dims_ok(int n, int H, int W) { return n >= 1 && H >= 1 && W >= 1 && (int64_t)n * H * W <= (1ll << 31); }
 
-// Network input of each z-slice of a coarse volume (one block per slice):
+// Network input of each z-slice of a coarse volume:
 // channel 0 the FLEDGE map over its largest finite value in the slice
 // (non-finite entries 0), channel 1 (log10 Q - 2) / 2 clamped to [-2, 3], a
 // missing Q (NaN) counted as the floor Q = 2 and an infinite one as the top
 // of the range.
-__global__ void __launch_bounds__(256) features_kernel(const float* __restrict__ S, const float* __restrict__ Q,
-                                                       int64_t plane, float* __restrict__ X) {
-  __shared__ float red[256];
-  const int z = blockIdx.x;
+// A slice belongs to a cluster of 8 blocks that share its maximum.
+constexpr int FEAT_CLUSTER = 8, FEAT_THREADS = 512;
+__global__ void __cluster_dims__(FEAT_CLUSTER, 1, 1) __launch_bounds__(FEAT_THREADS)
+    features_kernel(const float* __restrict__ S, const float* __restrict__ Q, int64_t plane, float* __restrict__ X) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  __shared__ float red[FEAT_THREADS / 32], block_max;
+  const int z = blockIdx.x / FEAT_CLUSTER, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t first = (int64_t)cluster.block_rank() * FEAT_THREADS + threadIdx.x, step = FEAT_CLUSTER * FEAT_THREADS;
   const float* s = S + (size_t)z * plane;
   const float* q = Q + (size_t)z * plane;
   float m = 0.0f;
-  for (int64_t i = threadIdx.x; i < plane; i += blockDim.x) {
+#pragma unroll 4
+  for (int64_t i = first; i < plane; i += step) {
     const float v = s[i];
     if (isfinite(v) && v > m) m = v;
   }
-  red[threadIdx.x] = m;
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) red[warp] = m;
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] = fmaxf(red[threadIdx.x], red[threadIdx.x + o]);
-    __syncthreads();
+  if (warp == 0) {
+    m = lane < FEAT_THREADS / 32 ? red[lane] : 0.0f;
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) block_max = m;
   }
-  const float smax = fmaxf(red[0], 1e-12f);
+  cluster.sync();
+  m = 0.0f;
+  for (int r = 0; r < FEAT_CLUSTER; ++r) m = fmaxf(m, *cluster.map_shared_rank(&block_max, r));
+  cluster.sync();  // no block leaves while another reads its maximum
+  const float smax = fmaxf(m, 1e-12f);
   float* x0 = X + (size_t)z * 2 * plane;
   float* x1 = x0 + plane;
-  for (int64_t i = threadIdx.x; i < plane; i += blockDim.x) {
+#pragma unroll 2
+  for (int64_t i = first; i < plane; i += step) {
     const float v = s[i] / smax;
     x0[i] = isfinite(v) ? v : 0.0f;
     float qv = q[i];
@@ -303,9 +991,14 @@ int qsl_cnn_features(const float* S, const float* Q, int nz, int ny, int nx, flo
     qsl::set_error("qsl_cnn_features: bad arguments");
     return QSL_EINVAL;
   }
-  features_kernel<<<nz, 256, 0, (cudaStream_t)stream_>>>(S, Q, (int64_t)ny * nx, X);
-  qsl::count_launch();
-  QSL_CHECK_CUDA(cudaGetLastError());
+  const int64_t plane = (int64_t)ny * nx;
+  constexpr int MAX_SLICES = 1 << 24;  // per launch
+  for (int z = 0; z < nz; z += std::min(MAX_SLICES, nz - z)) {
+    features_kernel<<<std::min(MAX_SLICES, nz - z) * FEAT_CLUSTER, FEAT_THREADS, 0, (cudaStream_t)stream_>>>(
+        S + z * plane, Q + z * plane, plane, X + 2 * z * plane);
+    qsl::count_launch();
+    QSL_CHECK_CUDA(cudaGetLastError());
+  }
   return QSL_OK;
 }
 
@@ -330,7 +1023,7 @@ int qsl_cnn_create(const float* params, qsl_cnn** out) {
   }
   qsl_cnn* c = new qsl_cnn();
   cudaError_t e = cudaMalloc((void**)&c->w, NPAR * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&c->wb, NPAR * sizeof(__nv_bfloat16));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&c->wb, NWB * sizeof(__nv_bfloat16));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->m, NPAR * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->v, NPAR * sizeof(float));
   if (e == cudaSuccess) e = cudaMemcpy(c->w, params, NPAR * sizeof(float), cudaMemcpyHostToDevice);
@@ -367,14 +1060,9 @@ int qsl_cnn_forward(qsl_cnn* c, const float* x, int n, int H, int W, float* prob
     qsl::set_error("bad CNN forward arguments");
     return QSL_EINVAL;
   }
-  float *a1, *a2, *z;
-  int rc = forward(c, x, n, H, W, s, &a1, &a2, &z);
-  if (rc) return rc;
-  int64_t P = (int64_t)n * H * W;
-  sigmoid_kernel<<<(int)std::min<int64_t>((P + 255) / 256, 4096), 256, 0, s>>>(z, P, prob);
-  qsl::count_launch();
-  QSL_CHECK_CUDA(cudaGetLastError());
-  return QSL_OK;
+  const TileGrid G = tile_grid(n, H, W, ZW, ZH);
+  return launch_tiles(forward_kernel<false>, TILE_THREADS, sizeof(TileSmem), 2, 1, G.tiles, s, x, c->wb, c->w,
+                      (float*)nullptr, (float*)nullptr, prob, G);
 }
 
 int qsl_cnn_loss_grad(qsl_cnn* c, const float* x, const float* y, int n, int H, int W, float pos_weight, float* loss,
@@ -384,26 +1072,27 @@ int qsl_cnn_loss_grad(qsl_cnn* c, const float* x, const float* y, int n, int H, 
     qsl::set_error("bad CNN loss/gradient arguments");
     return QSL_EINVAL;
   }
-  float *a1, *a2, *z;
-  int rc = forward(c, x, n, H, W, s, &a1, &a2, &z);
-  if (rc) return rc;
   size_t P = (size_t)n * H * W;
-  float* dz = z + P;
-  float* d2 = dz + P;
-  float* d1 = d2 + P * 32;
+  int rc = ensure_act(c, P, s);
+  if (rc) return rc;
+  float *a1 = c->act, *a2 = a1 + P * 32, *d2 = a2 + P * 32, *d1 = d2 + P * 32, *z = d1 + P * 32, *dz = z + P;
   QSL_CHECK_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), s));
   QSL_CHECK_CUDA(cudaMemsetAsync(grad, 0, NPAR * sizeof(float), s));
-  bce_kernel<<<(int)std::min<size_t>((P + 255) / 256, 4096), 256, 0, s>>>(z, y, (int64_t)P, pos_weight, dz, loss);
+  const TileGrid GF = tile_grid(n, H, W, ZW, ZH), GD = tile_grid(n, H, W, DW, DH);
+  if ((rc = launch_tiles(forward_kernel<true>, TILE_THREADS, sizeof(TileSmem), 2, 1, GF.tiles, s, x, c->wb, c->w, a1, a2,
+                         z, GF)))
+    return rc;
+  bce_kernel<<<(int)std::min<size_t>((P + BCE_THREADS - 1) / BCE_THREADS, 1024), BCE_THREADS, 0, s>>>(z, y, (int64_t)P, pos_weight, dz, loss,
+                                                                          grad + OFF_B3);
   qsl::count_launch();
   QSL_CHECK_CUDA(cudaGetLastError());
-  // layer 3: dW3, dB3; d2 = conv^T(dz) masked by a2 > 0 (ReLU)
-  if ((rc = launch_wgrad<C2, 1>(a2, dz, grad + OFF_W3, grad + OFF_B3, n, H, W, s))) return rc;
-  if ((rc = launch_conv<1, C2, false, true, false>(dz, c->wb + OFF_W3, nullptr, a2, d2, n, H, W, s))) return rc;
-  // layer 2
-  if ((rc = launch_wgrad<C2, C2>(a1, d2, grad + OFF_W2, grad + OFF_B2, n, H, W, s))) return rc;
-  if ((rc = launch_conv<C2, C2, false, true, false>(d2, c->wb + OFF_W2, nullptr, a1, d1, n, H, W, s))) return rc;
-  // layer 1
-  return launch_wgrad<C1, C2>(x, d1, grad + OFF_W1, grad + OFF_B1, n, H, W, s);
+  if ((rc = launch_tiles(dgrad_kernel, TILE_THREADS, sizeof(TileSmem), 2, 1, GD.tiles, s, dz, c->wb, a1, a2, d1, d2, GD)))
+    return rc;
+  const WgradGrid GW = wgrad_grid(n, H, W);
+  if ((rc = launch_tiles(wgrad32_kernel, WG_THREADS, sizeof(WgradSmem<14>), 1, 1, GW.tiles, s, a1, d2, grad + OFF_W2,
+                         grad + OFF_B2, GW)))
+    return rc;
+  return launch_tiles(wgrad_io_kernel, WG_THREADS, sizeof(WgradSmem<1>), 1, 2, GW.tiles, s, x, d1, dz, a2, grad, GW);
 }
 
 int qsl_cnn_adam_step(qsl_cnn* c, const float* grad, float lr, float beta1, float beta2, float eps, void* stream_) {
