@@ -115,7 +115,9 @@ typedef struct qsl_opts {
                               3 = a group of three lanes (one per axis), 0 = auto (three
                               up to 512 line directions per SM, where a launch is bound
                               by the latency of its longest lines; results agree to
-                              rounding)                                                  */
+                              rounding). QSL_RKCK54 in FP64 on uniform Cartesian grids
+                              with trilinear interpolation: 1 or 3 = one lane, 0 = auto
+                              (sixteen lanes up to the same count)                       */
   int32_t interp_order;    /* Sec. "Interpolation schemes": 1 (or 0) trilinear, 2 triquadratic
                               (Dodgson's interpolating quadratic, 27 vertices), 3 tricubic
                               (Keys cubic convolution, 64 vertices); 2 and 3 need a uniform

@@ -500,6 +500,7 @@ struct TraceParams {
   unsigned long long* cont_count;
   int handoff;                     // cell_kernel_f64: hand over a warp's lines at or below this many, 0 = never
   int cont_in;                     // cell_wide_kernel: trace the handed-over lines
+  int64_t few;                     // ck_wide_kernel traces launches of at most this many units, trace_kernel the others
 };
 
 // Problem and seed of launch seed j: global id, item, position.
@@ -628,6 +629,7 @@ __global__ void __launch_bounds__(256) trace_kernel(const __grid_constant__ Trac
     int64_t c = 2 * (*P.n_seeds_dev);
     total = c < total ? c : total;
   }
+  if (total <= P.few) return;
   // lanes of each warp that take work: all 32 when the units fill every
   // resident warp, fewer when they do not, so that a launch of few (and
   // typically long) lines spreads them over all warps and a lane's path is not
@@ -2485,10 +2487,76 @@ __device__ __forceinline__ double wide_rhs(const WideLane& W, const double* co, 
   return W.j == 0 ? b * ihc : (ihc * rm) * fma(-b, bs, g);
 }
 
-__global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ TraceParams<double> P, int sms) {
+// First state of a line on its group's lanes: the reference vertex, the lane's
+// component y (position offset, or deviation in cell units) and, for lines that
+// end where they start, the status and face.
+__device__ __forceinline__ int wide_start(const Item<double>* E, const double* xd, double sgn, int c, int j, double ihc,
+                                          int* ic, double* y, int* face) {
   typedef double R;
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
+  R yf[9];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    double fa = (xd[a] - E->org_d[a]) * E->inv_h_d[a];
+    double fl = floor(fmin(fmax(fa, 0.0), (double)(E->F.n[a] - 2)));
+    ic[a] = (int)fl;
+    yf[a] = fa - fl;
+  }
+#pragma unroll
+  for (int i = 3; i < 9; ++i) yf[i] = R(0);
+  *face = NO_FACE;
+  int status = ST_RUNNING;
+  bool outside = false;
+#pragma unroll
+  for (int f = 0; f < 6; ++f)
+    if (face_g<R, true>(E->lo, E->hi, ic, f, yf, (const R*)nullptr) > R(0)) outside = true;
+  if (outside || !isfinite(xd[0]) || !isfinite(xd[1]) || !isfinite(xd[2])) {
+    status = QSL_LINE_OUTSIDE;
+  } else {
+    Interp<R> I0;
+    interp<R, R, false, false, true, false>(E->F, yf[0], yf[1], yf[2], I0, ic);
+    R m0 = sqrt(I0.b[0] * I0.b[0] + I0.b[1] * I0.b[1] + I0.b[2] * I0.b[2]);
+    if (!(m0 > R(0))) {
+      status = QSL_LINE_NULL;
+    } else {
+      // Eq. ic (same construction as the other tracers)
+      R u0[3] = {I0.b[0] / m0, I0.b[1] / m0, I0.b[2] / m0};
+      int ax = 0;
+      if (fabs(u0[1]) < fabs(u0[ax])) ax = 1;
+      if (fabs(u0[2]) < fabs(u0[ax])) ax = 2;
+      R av[3];
+      if (ax == 0) { av[0] = 0; av[1] = -u0[2]; av[2] = u0[1]; }
+      else if (ax == 1) { av[0] = u0[2]; av[1] = 0; av[2] = -u0[0]; }
+      else { av[0] = -u0[1]; av[1] = u0[0]; av[2] = 0; }
+      R an = sqrt(av[0] * av[0] + av[1] * av[1] + av[2] * av[2]);
+      av[0] /= an;
+      av[1] /= an;
+      av[2] /= an;
+      yf[3] = av[0];
+      yf[4] = av[1];
+      yf[5] = av[2];
+      yf[6] = u0[1] * av[2] - u0[2] * av[1];
+      yf[7] = u0[2] * av[0] - u0[0] * av[2];
+      yf[8] = u0[0] * av[1] - u0[1] * av[0];
+#pragma unroll
+      for (int f = 0; f < 6; ++f) {
+        if (status == ST_RUNNING && face_g<R, true>(E->lo, E->hi, ic, f, yf, (const R*)nullptr) == R(0)) {
+          R bn = I0.b[f >> 1] * sgn;
+          R outw = (f & 1) ? bn : -bn;
+          if (outw > R(0)) {
+            status = QSL_LINE_OK;
+            *face = f;
+          }
+        }
+      }
+    }
+  }
+  const R x_c = sel3(c, yf[0], yf[1], yf[2]), d1_c = sel3(c, yf[3], yf[4], yf[5]), d2_c = sel3(c, yf[6], yf[7], yf[8]);
+  *y = j == 0 ? x_c : (j == 1 ? d1_c * ihc : (j == 2 ? d2_c * ihc : R(0)));  // deviations in cell units
+  return status;
+}
+
+// The lane roles of a 16-lane group.
+__device__ __forceinline__ WideLane wide_lane(int lane) {
   const int l = lane & 15;
   WideLane W;
   W.gb = lane & 16;
@@ -2498,6 +2566,15 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
   W.s_src = (W.j == 0 || W.j == 3) ? W.pos(1) : W.pos(0);
   W.t_src = W.j == 2 ? W.pos(1) : W.pos(2);
   W.p1_src = W.pos(W.c) + (W.j == 0 ? 3 : 1);
+  return W;
+}
+
+__global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ TraceParams<double> P, int sms) {
+  typedef double R;
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int l = lane & 15;
+  const WideLane W = wide_lane(lane);
   const int c = W.c, j = W.j;
   const bool lead = l == 0, writer = l < 12 && j < 3;
   int64_t total = P.n_units;
@@ -2581,70 +2658,12 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
 #pragma unroll
               for (int a = 0; a < 3; ++a) ic[a] = k->ic[a];
             } else {
-            R yf[9];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-              double fa = (xd[a] - E->org_d[a]) * E->inv_h_d[a];
-              double fl = floor(fmin(fmax(fa, 0.0), (double)(E->F.n[a] - 2)));
-              ic[a] = (int)fl;
-              yf[a] = fa - fl;
-            }
-#pragma unroll
-            for (int i = 3; i < 9; ++i) yf[i] = R(0);
             mu = 0;
             muc = 0;
             steps = 0;
             zc = 0;
-            int lface = NO_FACE;
-            int status = ST_RUNNING;
-            bool outside = false;
-#pragma unroll
-            for (int f = 0; f < 6; ++f)
-              if (face_g<R, true>(E->lo, E->hi, ic, f, yf, (const R*)nullptr) > R(0)) outside = true;
-            if (outside || !isfinite(xd[0]) || !isfinite(xd[1]) || !isfinite(xd[2])) {
-              status = QSL_LINE_OUTSIDE;
-            } else {
-              Interp<R> I0;
-              interp<R, R, false, false, true, false>(E->F, yf[0], yf[1], yf[2], I0, ic);
-              R m0 = sqrt(I0.b[0] * I0.b[0] + I0.b[1] * I0.b[1] + I0.b[2] * I0.b[2]);
-              if (!(m0 > R(0))) {
-                status = QSL_LINE_NULL;
-              } else {
-                // Eq. ic (same construction as the other tracers)
-                R u0[3] = {I0.b[0] / m0, I0.b[1] / m0, I0.b[2] / m0};
-                int ax = 0;
-                if (fabs(u0[1]) < fabs(u0[ax])) ax = 1;
-                if (fabs(u0[2]) < fabs(u0[ax])) ax = 2;
-                R av[3];
-                if (ax == 0) { av[0] = 0; av[1] = -u0[2]; av[2] = u0[1]; }
-                else if (ax == 1) { av[0] = u0[2]; av[1] = 0; av[2] = -u0[0]; }
-                else { av[0] = -u0[1]; av[1] = u0[0]; av[2] = 0; }
-                R an = sqrt(av[0] * av[0] + av[1] * av[1] + av[2] * av[2]);
-                av[0] /= an;
-                av[1] /= an;
-                av[2] /= an;
-                yf[3] = av[0];
-                yf[4] = av[1];
-                yf[5] = av[2];
-                yf[6] = u0[1] * av[2] - u0[2] * av[1];
-                yf[7] = u0[2] * av[0] - u0[0] * av[2];
-                yf[8] = u0[0] * av[1] - u0[1] * av[0];
-#pragma unroll
-                for (int f = 0; f < 6; ++f) {
-                  if (status == ST_RUNNING && face_g<R, true>(E->lo, E->hi, ic, f, yf, (const R*)nullptr) == R(0)) {
-                    R bn = I0.b[f >> 1] * sgn;
-                    R outw = (f & 1) ? bn : -bn;
-                    if (outw > R(0)) {
-                      status = QSL_LINE_OK;
-                      lface = f;
-                    }
-                  }
-                }
-              }
-            }
-            const R x_c = sel3(c, yf[0], yf[1], yf[2]), d1_c = sel3(c, yf[3], yf[4], yf[5]),
-                    d2_c = sel3(c, yf[6], yf[7], yf[8]);
-            y = j == 0 ? x_c : (j == 1 ? d1_c * ihc : (j == 2 ? d2_c * ihc : R(0)));  // deviations in cell units
+            int lface;
+            const int status = wide_start(E, xd, sgn, c, j, ihc, ic, &y, &lface);
             h = (float)E->h_init;
             if (status != ST_RUNNING) {
               write_end_wide(P, E, unit, c, j, writer, y, ic, hhc, R(0), lface, status, 0);
@@ -2832,6 +2851,343 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
             }
             h = fmaxf(hnext, hsF);
           }
+        }
+      }
+    }
+    if (status != ST_RUNNING) {
+      write_end_wide(P, E, unit, c, j, writer, y, ic, hhc, mu, lface, status, steps);
+      active = false;
+    }
+  }
+  write_stats(P, lane, c_stage, c_acc, c_rej, c_land, c_lines, timed_out);
+}
+
+// ------------------------------------------------------------ Cash-Karp, sixteen lanes per line (FP64)
+// Largest integer not above x: the FP32 floor, corrected by the sign and the
+// exponent of x minus it (an FP64 comparison is an FP64-pipe instruction).
+__device__ __forceinline__ int floor_bits(double x) {
+  int f = (int)floorf((float)x);
+  const double d = x - (double)f;
+  if (__double2hiint(d) < 0 && d != 0.0) --f;
+  else if (__double2hiint(d) >= 0x3ff00000) ++f;
+  return f;
+}
+
+// err^(-1 / N) to FP64 precision: the FP32 power and two Newton steps (its
+// error of 1e-6 to 1e-12 and 1e-16), 12 FP64 instructions where pow has over
+// 100. Outside FP32's range, or where the step factor is cut off anyway: the
+// FP32 power. Step sizes that differ in their last FP32 digits end, over some
+// hundred steps, in other step sequences and other results to within the
+// method's own error; this keeps the launch's results those of trace_kernel.
+template <int N>
+__device__ __forceinline__ double inv_root(double err) {
+  const float ef = fminf((float)err, 3e38f);
+  const float y0 = powf(fmaxf(ef, 1e-30f), -1.0f / N);
+  if (!(ef > 1e-6f && ef < 1e6f)) return (double)y0;
+  double y = (double)y0;
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const double y2 = y * y, yn = N == 4 ? y2 * y2 : y2 * y2 * y;
+    y = fma(y * (1.0 / N), fma(-err, yn, 1.0), y);
+  }
+  return y;
+}
+
+// The cell a group's last stage was in, and the lane's bilinear coefficients there.
+struct WideCell {
+  int i[3];
+  double co[4];
+};
+
+// Stage derivative of the lane's component for the stage value t, a position
+// offset from the vertex icc of the lane's axis or a deviation in cell units.
+// The cell is kept while consecutive stages stay in it.
+__device__ __forceinline__ double ck_wide_rhs(const WideLane& W, const FieldView<double>& F, bool raw, double ihc, int icc,
+                                              int nc, double lim, double t, WideCell& C) {
+  // cell and fraction along the lane's own axis, then the other axes' cells
+  const double x = gsh(W.gm, t, W.pos(W.c));
+  const float xf = (float)x;
+  const int fl = fabsf(xf) < 1e6f ? floor_bits(x) : (int)floor(fmin(fmax(x, -lim), lim));
+  const int i = min(max(icc + fl, 0), nc - 2);
+  if (W.j == 0) t = x - (double)(i - icc);
+  const int i0 = __shfl_sync(W.gm, i, W.pos(0)), i1 = __shfl_sync(W.gm, i, W.pos(1)), i2 = __shfl_sync(W.gm, i, W.pos(2));
+  if (i0 != C.i[0] || i1 != C.i[1] || i2 != C.i[2]) {
+    C.i[0] = i0;
+    C.i[1] = i1;
+    C.i[2] = i2;
+    const int j = W.j;
+    const size_t sy = 4 * (size_t)F.n[0], sz = sy * (size_t)F.n[1];
+    const double* p = reinterpret_cast<const double*>(F.v) + (size_t)i2 * sz + (size_t)i1 * sy + 4 * (size_t)i0 + W.c;
+    const size_t oj = j == 1 ? sy : (j == 2 ? sz : 4);
+    const size_t os = (j == 0 || j == 3) ? sy : 4, ot = j == 2 ? sy : sz;
+    const double l00 = __ldg(p), l10 = __ldg(p + os), l01 = __ldg(p + ot), l11 = __ldg(p + os + ot);
+    const double h00 = __ldg(p + oj), h10 = __ldg(p + oj + os), h01 = __ldg(p + oj + ot), h11 = __ldg(p + oj + os + ot);
+    const bool low = j == 3;
+    const double d00 = low ? l00 : h00 - l00, d10 = low ? l10 : h10 - l10;
+    const double d01 = low ? l01 : h01 - l01, d11 = low ? l11 : h11 - l11;
+    C.co[0] = d00;
+    C.co[1] = d10 - d00;
+    C.co[2] = d01 - d00;
+    C.co[3] = (d11 - d10) - C.co[2];
+  }
+  const double k = wide_rhs(W, C.co, raw, ihc, t);
+  return raw ? k : k * ihc;
+}
+
+// trace_kernel's Cash-Karp tracer (local frame, trilinear, Cartesian) with the
+// lanes of cell_wide_kernel: one component per lane. An FP64 warp instruction
+// takes 64 cycles of its warp whatever its active lanes, and a lone line on one
+// lane needs about 1,900 of them per step; here a stage needs about 20 to 30.
+// 3,600 seeds on 128^3: tol 1e-2 10.7 -> 2.4 ms, 1e-5 41.7 -> 8.7, 1e-6 163 ->
+// 31; the same Q and lengths but for the last digits of a few at 1e-5 and below.
+// The step controller is FP64 like trace_kernel's (its power by inv_root).
+// The launch serves at most P.few units, trace_kernel beside it more.
+__global__ void __launch_bounds__(256) ck_wide_kernel(const __grid_constant__ TraceParams<double> P, int sms) {
+  typedef double R;
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, l = lane & 15;
+  const WideLane W = wide_lane(lane);
+  const int c = W.c, j = W.j;
+  const bool lead = l == 0, writer = l < 12 && j < 3;
+  int64_t total = P.n_units;
+  if (P.n_seeds_dev) {
+    int64_t cnt = 2 * (*P.n_seeds_dev);
+    total = cnt < total ? cnt : total;
+  }
+  if (total > P.few) return;
+  const int wpb = blockDim.x >> 5;
+  const int64_t warps_total = (int64_t)gridDim.x * wpb;
+  // rank of this warp: first warps of the first `sms` blocks, their second warps, ...
+  const int64_t wave = blockIdx.x / sms, in_wave = blockIdx.x % sms;
+  const int64_t nb = min((int64_t)sms, (int64_t)gridDim.x - wave * sms);
+  const int64_t rank = wave * sms * wpb + (int64_t)(threadIdx.x >> 5) * nb + in_wave;
+  if (rank >= total) return;
+  const bool usable = total > warps_total || W.gb == 0;
+  const Item<R>* E = &P.item0;
+
+  bool active = false, exhausted = false, raw = false, capped = false;
+  int64_t unit = 0;
+  R y = 0, ihc = 1, hhc = 1, orgc = 0, lim = 0;
+  int ic[3] = {0, 0, 0}, icc = 0, nc = 2;
+  WideCell C;
+  C.i[0] = -1;
+  R mu = 0, muc = 0, sgn = 1, h = 0;
+  int steps = 0, phase = 0;
+  // face landing state
+  R la = 0, lb = 0, lga = 0, lgb = 0, lhm = 0;
+  int lface = 0, lside = 0, lit = 0, lround = 0;
+  unsigned long long c_stage = 0, c_acc = 0, c_rej = 0, c_land = 0, c_lines = 0;
+  int iter = 0;
+  bool timed_out = false;
+  const unsigned long long t_start = P.timeout_ns ? globaltimer() : 0ull;
+
+  for (;;) {
+    if (!exhausted) {
+      const unsigned need = __ballot_sync(FULL, usable && lead && !active);
+      const int nneed = __popc(need);
+      if (nneed > 0) {
+        const int leader = __ffs(need) - 1;
+        unsigned long long base = 0;
+        if (lane == leader) base = atomicAdd(P.head, (unsigned long long)nneed);
+        base = __shfl_sync(FULL, base, leader);
+        if ((int64_t)(base + nneed) >= total) exhausted = true;
+        if (usable && ((need >> W.gb) & 1u)) {
+          const int64_t myu = (int64_t)base + __popc(need & ((1u << W.gb) - 1u));
+          if (myu < total) {
+            unit = myu;
+            active = true;
+            if (lead) c_lines += (myu & 1) == 0;
+            int64_t g;
+            double xd[3];
+            E = resolve_seed(P, unit >> 1, &g, xd);
+            sgn = (unit & 1) ? R(-1) : R(1);
+            raw = E->F.raw != 0;
+            ihc = sel3(c, E->F.inv_h[0], E->F.inv_h[1], E->F.inv_h[2]);
+            hhc = R(1) / ihc;
+            orgc = sel3(c, E->F.org[0], E->F.org[1], E->F.org[2]);
+            nc = sel3(c, E->F.n[0], E->F.n[1], E->F.n[2]);
+            lim = R(nc);
+            const int status = wide_start(E, xd, sgn, c, j, ihc, ic, &y, &lface);
+            icc = sel3(c, ic[0], ic[1], ic[2]);
+            C.i[0] = -1;
+            mu = 0;
+            muc = 0;
+            steps = 0;
+            phase = 0;
+            h = E->h_init;
+            if (status != ST_RUNNING) {
+              write_end_wide(P, E, unit, c, j, writer, y, ic, hhc, R(0), lface, status, 0);
+              active = false;
+            }
+          }
+        }
+      }
+    }
+    if (!__any_sync(FULL, active)) {
+      if (exhausted) break;
+      continue;
+    }
+    if (P.timeout_ns && ((++iter & 63) == 0)) {
+      // warp-uniform, so that the lanes of a group agree
+      if (__any_sync(FULL, globaltimer() - t_start > P.timeout_ns)) timed_out = true;
+    }
+    if (!active) continue;
+
+    int status = ST_RUNNING;
+    if (timed_out) status = QSL_LINE_TIMEOUT;
+    R hs = lhm;
+    if (status == ST_RUNNING && phase == 0) {
+      if (steps >= P.max_steps) status = QSL_LINE_MAXSTEPS;
+      const R room = E->max_len - mu;
+      if (status == ST_RUNNING && !gt_bits(room, 0.0)) status = QSL_LINE_MAXLEN;
+      hs = gt_bits(h, E->h_max) ? E->h_max : h;
+      capped = !gt_bits(room, hs);
+      if (capped) hs = room;
+    }
+    if (status == ST_RUNNING) {
+      const R hh = sgn * hs;
+      const R K1 = hh * ck_wide_rhs(W, E->F, raw, ihc, icc, nc, lim, y, C);
+      const R K2 = hh * ck_wide_rhs(W, E->F, raw, ihc, icc, nc, lim, fma(R(A21), K1, y), C);
+      const R K3 = hh * ck_wide_rhs(W, E->F, raw, ihc, icc, nc, lim, fma(R(A32), K2, fma(R(A31), K1, y)), C);
+      const R K4 = hh * ck_wide_rhs(W, E->F, raw, ihc, icc, nc, lim, fma(R(A43), K3, fma(R(A42), K2, fma(R(A41), K1, y))), C);
+      const R K5 = hh * ck_wide_rhs(W, E->F, raw, ihc, icc, nc, lim,
+                                    fma(R(A54), K4, fma(R(A53), K3, fma(R(A52), K2, fma(R(A51), K1, y)))), C);
+      const R K6 = hh * ck_wide_rhs(W, E->F, raw, ihc, icc, nc, lim,
+                                    fma(R(A65), K5, fma(R(A64), K4, fma(R(A63), K3, fma(R(A62), K2, fma(R(A61), K1, y))))), C);
+      const R dy = fma(R(B6), K6, fma(R(B4), K4, fma(R(B3), K3, R(B1) * K1)));
+      c_stage += lead ? 6 : 0;
+      steps += 1;
+      if (phase == 0) {
+        const R ye = fma(R(E6), K6, fma(R(E5), K5, fma(R(E4), K4, fma(R(E3), K3, R(E1) * K1))));
+        const R yn = y + dy;
+        // error against tolerance in domain units
+        const R base = j == 0 ? fma(R(icc), hhc, orgc) : R(0);
+        const R ya = fabs(fma(y, hhc, base)), yb = fabs(fma(yn, hhc, base));
+        const R e = j == 3 ? R(0) : fabs(ye) * hhc;
+        const R sc = fma(P.tol_rel, gt_bits(ya, yb) ? ya : yb, P.tol_abs);
+        const bool finite = !__any_sync(W.gm, j != 3 && (__double2hiint(yn) & 0x7ff00000) == 0x7ff00000);
+        // largest ratio: on the bit patterns (no FP64 comparisons); 0 / 0 counts as 0
+        const float scf = (float)sc;
+        R err = j == 3 ? R(0) : (scf > 1e-30f && scf < 1e30f ? e * rcp_fp64(sc) : (e > R(0) ? e / sc : R(0)));
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+          const R other = __shfl_xor_sync(W.gm, err, o);
+          err = gt_bits(other, err) ? other : err;
+        }
+        if (!finite) {
+          status = QSL_LINE_NONFINITE;
+        } else if (gt_bits(err, R(1))) {
+          c_rej += lead;
+          const R f = R(0.9) * inv_root<4>(err);
+          h = hs * (gt_bits(f, R(0.2)) ? f : R(0.2));
+          if (gt_bits(E->h_min, h)) status = QSL_LINE_STALL;
+        } else {
+          c_acc += lead;
+          const R r_lo = (sel3(c, E->lo[0], E->lo[1], E->lo[2]) - R(icc)) - y,
+                  r_hi = (sel3(c, E->hi[0], E->hi[1], E->hi[2]) - R(icc)) - y;
+          const bool out = j == 0 && (gt_bits(r_lo - dy, 0.0) || gt_bits(dy - r_hi, 0.0));
+          if (!__any_sync(W.gm, out)) {
+            y = yn;
+            // move the reference vertex with the line (exact shifts)
+            int ni = icc;
+            if (j == 0) {
+              ni = min(max(icc + floor_bits(y), 0), nc - 2);
+              y -= R(ni - icc);
+            }
+            icc = __shfl_sync(W.gm, ni, W.pos(c));
+#pragma unroll
+            for (int a = 0; a < 3; ++a) ic[a] = __shfl_sync(W.gm, icc, W.pos(a));
+            const R t1 = hs - muc, t2 = mu + t1;  // compensated sum of the step lengths
+            muc = (t2 - mu) - t1;
+            mu = t2;
+            if (capped) status = QSL_LINE_MAXLEN;
+            else {
+              const R f = R(0.9) * inv_root<5>(err);
+              h = hs * (gt_bits(f, R(5)) ? R(5) : f);
+            }
+          } else {
+            // leave the domain: land exactly on the exit face
+            phase = 1;
+            const R yp[3] = {gsh(W.gm, y, W.pos(0)), gsh(W.gm, y, W.pos(1)), gsh(W.gm, y, W.pos(2))};
+            const R dp[3] = {gsh(W.gm, dy, W.pos(0)), gsh(W.gm, dy, W.pos(1)), gsh(W.gm, dy, W.pos(2))};
+            lface = chord_face<R, true>(E->lo, E->hi, ic, yp, dp);
+            la = 0;
+            lb = hs;
+            lga = face_gs<R, true>(E->lo, E->hi, ic, lface, yp, (const R*)nullptr);
+            lgb = face_gs<R, true>(E->lo, E->hi, ic, lface, yp, dp);
+            lside = 0;
+            lit = 0;
+            lround = 0;
+            lhm = la + (lb - la) * lga / (lga - lgb);
+            if (!(lga < R(0))) {
+              // the step starts on this face and ends beyond it again: seek an inside point first
+              lside = 2;
+              lhm = R(0.5) * lb;
+            }
+          }
+        }
+      } else {
+        c_land += lead;
+        lit += 1;
+        const R yp[3] = {gsh(W.gm, y, W.pos(0)), gsh(W.gm, y, W.pos(1)), gsh(W.gm, y, W.pos(2))};
+        const R dp[3] = {gsh(W.gm, dy, W.pos(0)), gsh(W.gm, dy, W.pos(1)), gsh(W.gm, dy, W.pos(2))};
+        const R gm = face_gs<R, true>(E->lo, E->hi, ic, lface, yp, dp);
+        // converged when within the landing tolerance or at the resolution of
+        // the step increment along the face normal
+        const R dn = fabs(sel3(lface >> 1, dp[0], dp[1], dp[2]));
+        const R gtol = fmax(E->land_tol, R(4) * eps_of<R>() * dn);
+        if (lside == 2 && lit < 60 && isfinite(gm)) {
+          // seeking an inside point below the outside step lb
+          if (gm < R(0)) {
+            la = lhm;
+            lga = gm;
+            lside = 0;
+            lhm = la + (lb - la) * lga / (lga - lgb);
+          } else {
+            lb = lhm;
+            lgb = gm;
+            lhm = R(0.5) * lhm;
+          }
+        } else if (fabs(gm) <= gtol || lit >= 60 || !isfinite(gm) || !(lb - la > eps_of<R>() * lb)) {
+          R worst = R(-1);
+#pragma unroll
+          for (int f = 0; f < 6; ++f)
+            if (f != lface) worst = fmax(worst, face_g<R, true>(E->lo, E->hi, ic, f, yp, dp));
+          if (worst > gtol && lround < 8) {
+            // the landed point is outside another face: that face was crossed first
+            lround += 1;
+            lface = chord_face<R, true>(E->lo, E->hi, ic, yp, dp);
+            la = 0;
+            lb = lhm;
+            lga = face_gs<R, true>(E->lo, E->hi, ic, lface, yp, (const R*)nullptr);
+            lgb = face_gs<R, true>(E->lo, E->hi, ic, lface, yp, dp);
+            lside = 0;
+            lit = 0;
+            lhm = la + (lb - la) * lga / (lga - lgb);
+            if (!(lga < R(0))) {
+              lside = 2;
+              lhm = R(0.5) * lb;
+            }
+          } else {
+            y += dy;
+            const R t1 = lhm - muc, t2 = mu + t1;
+            muc = (t2 - mu) - t1;
+            mu = t2;
+            status = QSL_LINE_OK;
+          }
+        } else {
+          if (gm > R(0)) {
+            lb = lhm;
+            lgb = gm;
+            if (lside == 1) lga *= R(0.5);
+            lside = 1;
+          } else {
+            la = lhm;
+            lga = gm;
+            if (lside == -1) lgb *= R(0.5);
+            lside = -1;
+          }
+          lhm = la + (lb - la) * lga / (lga - lgb);
         }
       }
     }
@@ -3965,6 +4321,10 @@ inline void launch_wide(const TraceParams<double>& P, int blocks, int threads, i
   cell_wide_kernel<<<blocks, threads, 0, stream>>>(P, sms);
 }
 inline void launch_wide(const TraceParams<float>&, int, int, int, cudaStream_t) {}
+inline void launch_ck_wide(const TraceParams<double>& P, int blocks, int threads, int sms, cudaStream_t stream) {
+  ck_wide_kernel<<<blocks, threads, 0, stream>>>(P, sms);
+}
+inline void launch_ck_wide(const TraceParams<float>&, int, int, int, cudaStream_t) {}
 
 // A warp of cell_kernel_f64 hands its lines to cell_wide_kernel once the queue
 // is empty and at most kHandoff of them are left: on one lane each the last
@@ -3973,6 +4333,11 @@ inline void launch_wide(const TraceParams<float>&, int, int, int, cudaStream_t) 
 // 20.4 ms; 196,608 seeds: 44.6, 36.4, 34.1, 33.9, 34.1, 34.0 ms. kContMax: the
 // most handed over per launch (resident warps x kHandoff is below it).
 constexpr int kHandoff = 24;
+// Units per SM up to which the FP64 Cash-Karp launch takes sixteen lanes per
+// line. Measured on 128^3, one lane and sixteen: 32,400 seeds (426 per SM) at
+// tol 1e-2 11.9 and 7.7 ms, raw fields 14.5 and 12.7, at 1e-6 183 and 71;
+// 65,536 seeds 17.2 and 14.5, raw 20.8 and 23.7.
+constexpr int kCkWidePerSm = 512;
 constexpr size_t kContMax = 1 << 16;
 template <class R>
 size_t cont_offset(size_t n_units) {
@@ -4019,6 +4384,7 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
   P.cont_count = head + 2;
   P.handoff = 0;
   P.cont_in = 0;
+  P.few = -1;
   int threads = 32 * shape.warps_per_block;
   // persistent kernel: never launch more blocks than can be resident at once
   const bool use_cell = loc && cfg.integrator == QSL_DOPRI5_CELL;
@@ -4150,8 +4516,25 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
       trace_kernel<R, NC, true, true><<<blocks, threads, 0, stream>>>(P);
       qsl::count_launch();
     } else if (loc) {
-      trace_kernel<R, NC, true><<<blocks, threads, 0, stream>>>(P);
-      qsl::count_launch();
+      // FP64 Cash-Karp with the deviations, automatic lanes: few lines run on
+      // sixteen lanes each. The length of a retrace list is known on the device
+      // only, so both kernels are launched and one of them leaves at once.
+      bool one_lane = true;
+      if (sizeof(R) == 8 && NC == 9 && shape.line_lanes == 0 && !P.euler) {
+        P.few = (int64_t)kCkWidePerSm * sms;
+        if (n_seeds_dev || 2 * n_seeds <= P.few) {
+          int res_w = 0;
+          QSL_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res_w, ck_wide_kernel, threads, 0));
+          launch_ck_wide(P, sms * (res_w > 0 ? res_w : 1), threads, sms, stream);
+          qsl::count_launch();
+          QSL_CHECK_CUDA(cudaGetLastError());
+          one_lane = n_seeds_dev != nullptr;
+        }
+      }
+      if (one_lane) {
+        trace_kernel<R, NC, true><<<blocks, threads, 0, stream>>>(P);
+        qsl::count_launch();
+      }
     } else {
       trace_kernel<R, NC, false><<<blocks, threads, 0, stream>>>(P);
       qsl::count_launch();
