@@ -29,47 +29,60 @@ constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + NW1, OFF_W2 = OFF_B1 + NB1, OFF_B2 =
               OFF_B3 = OFF_W3 + NW3, NPAR = OFF_B3 + NB3;
 
 // ---------------------------------------------------------------- tiles
-// Forward and data-gradient tiles: rows of 32 pixels (one warp each), the
-// MMA's 128 rows are four of them. Flattened indices are row * 32 + column;
-// a tap (ky, kx) of the pixel m is the pixel m + 32 ky + kx of the layer
-// below, so the last columns of a row see the next row's first ones: each
-// layer has two valid columns less than the one below, and 2 rows less.
+// Data-gradient tiles: rows of 32 pixels (one warp each), the MMA's 128 rows
+// are four of them. Flattened indices are row * 32 + column; a tap (ky, kx) of
+// the pixel m is the pixel m + 32 ky + kx of the layer above, so the last two
+// columns of a row see the next row's first ones and are not used.
 constexpr int PW = 32;
 constexpr int R2 = 12, R1 = R2 + 2;         // rows of the 32-channel layers: outputs, inputs
 constexpr int M2 = R2 * PW;                 // output pixels: three MMA tiles
 constexpr int NP = R1 * PW + 8;             // input pixels (the last taps read two past the rows)
-constexpr int ZW = PW - 6, ZH = R2 - 2;     // forward: valid output columns, rows
-constexpr int DW = PW - 2, DH = R2;         // data gradient: valid columns, rows
-constexpr int NPX = (R1 + 4) * PW + 8;      // forward: network input pixels (16 rows of layer 1 are computed)
+constexpr int DW = PW - 2, DH = R2;         // valid columns, rows
 constexpr int TILE_THREADS = 32 * R2;
 constexpr uint32_t CHUNK = NP * 16;         // bytes of one chunk plane
 constexpr uint32_t WTAP = 32 * 64;          // one tap's 32 x 32 weights
 
 struct alignas(16) TileSmem {
-  unsigned char a[12 * CHUNK];              // [piece][chunk] planes of the layer below; before that the network input
+  unsigned char a[12 * CHUNK];              // [piece][chunk] planes of the layer above's gradient
   unsigned char w2[9 * WTAP];               // [tap][chunk][out channel][8]
-  unsigned char w1[5 * 1024];               // [tap pair][tap][out channel][8]
   float w3[9 * 32];                         // [tap][channel]
-  float b1[32], b2[32], b3;
   uint32_t tmem;
   int failed;
-  uint64_t bar[4];
+  uint64_t bar[3];
 };
 static_assert(sizeof(TileSmem) <= 113 * 1024, "two blocks per SM");
-static_assert(NPX * 16 + 2048 <= 12 * CHUNK && 9 * M2 * 4 <= 12 * CHUNK, "overlays of the planes");
 
-// Layer 2's weights are kept twice more in the layout of the MMA's operand,
-// [tap][chunk][N][8] (K = chunk and element): K = input channels, N = output
-// channels for the forward pass, and channels swapped, taps reversed for the
-// data gradient. They are written wherever the BF16 weights are.
-constexpr int OFF_OP = (NPAR + 7) / 8 * 8, NWB = OFF_OP + 2 * NW2;
+// Layer 2's weights are kept twice more in the layouts of the MMA's operand
+// (K = chunk and element): forward [kx][chunk][ky][output channel][8] over the
+// input channels, data gradient [tap][chunk][input channel][8] over the output
+// channels with the taps reversed. They are written wherever the BF16 weights
+// are.
+// Layer 1's are kept as [rotation][MMA][tap of two][output channel][8] (see
+// forward_kernel): element 3 c + 0, 1, 2 the weight of input channel c for each
+// piece, element 6 a piece of the bias.
+constexpr int NOP1 = 3 * 5 * 512;
+constexpr int OFF_OP = (NPAR + 7) / 8 * 8, OFF_OP1 = OFF_OP + 2 * NW2, NWB = OFF_OP1 + NOP1;
 __device__ __forceinline__ void store_weight(__nv_bfloat16* wb, int i, float v) {
   const __nv_bfloat16 b = __float2bfloat16_rn(v);
   wb[i] = b;
   if (i >= OFF_W2 && i < OFF_W2 + NW2) {
     const int j = i - OFF_W2, co = j / (32 * 9), ci = (j / 9) % 32, k = j % 9;
-    wb[OFF_OP + ((k * 4 + ci / 8) * 32 + co) * 8 + ci % 8] = b;
+    wb[OFF_OP + (((k % 3) * 4 + ci / 8) * 96 + (k / 3) * 32 + co) * 8 + ci % 8] = b;
     wb[OFF_OP + NW2 + (((8 - k) * 4 + co / 8) * 32 + ci) * 8 + co % 8] = b;
+  } else if (i < NW1) {
+    // input slots 0 and 1 at kx: MMA kx; slot 2 at kx = 0, 1: MMA 3; at kx = 2: MMA 4
+    const int co = i / 18, c = (i / 9) % 2, ky = (i / 3) % 3, kx = i % 3;
+    for (int rot = 0; rot < 3; ++rot) {
+      const int slot = (rot + ky) % 3, p = slot < 2 ? kx : 3 + kx / 2, half = slot < 2 ? slot : kx % 2;
+      for (int e = 0; e < 3; ++e) wb[OFF_OP1 + rot * 2560 + p * 512 + half * 256 + co * 8 + 3 * c + e] = b;
+    }
+  } else if (i >= OFF_B1 && i < OFF_B1 + NB1) {
+    // the bias, exactly, in three pieces against the ones of slot 0
+    uint32_t pc[3];
+    umma::split2(v, 0.0f, pc, pc + 1, pc + 2);
+    for (int rot = 0; rot < 3; ++rot)
+      for (int p = 0; p < 3; ++p)
+        wb[OFF_OP1 + rot * 2560 + p * 512 + (i - OFF_B1) * 8 + 6] = __ushort_as_bfloat16((unsigned short)pc[p]);
   }
 }
 
@@ -98,7 +111,7 @@ __device__ __forceinline__ void conv32_issue(TileSmem& S, uint32_t tmem, int t) 
         umma::mma(d0 + (piece ? 96 : 32 * (tap / 3)),
                   a0 + ((piece * 4 + 2 * k) * CHUNK / 16 + (tap / 3) * PW + tap % 3), w0 + (tap * WTAP + k * 1024) / 16,
                   id, piece == 0 ? tap % 3 > 0 || k > 0 : piece == 1 || tap > 0 || k > 0);
-  umma::commit(&S.bar[1 + t]);
+  umma::commit(&S.bar[t]);
 }
 
 // Waits for the MMA tile of the warp's row (warp / 4) and reads its sums; the
@@ -106,7 +119,7 @@ __device__ __forceinline__ void conv32_issue(TileSmem& S, uint32_t tmem, int t) 
 __device__ __forceinline__ bool conv32_read(TileSmem& S, uint32_t tmem, int warp, uint32_t phase, float* v) {
   const int t = warp >> 2;
   const uint32_t tq = tmem + ((uint32_t)(warp & 3) << 21) + (t & 1) * 128;
-  const bool ok = umma::bar_wait(&S.bar[1 + t], phase);
+  const bool ok = umma::bar_wait(&S.bar[t], phase);
   umma::fence_after();
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -132,6 +145,7 @@ __device__ __forceinline__ bool conv32_read(TileSmem& S, uint32_t tmem, int warp
 }
 
 // Writes a pixel's 16 channels (half h of the 32) as pieces into the planes.
+template <uint32_t PLANE>
 __device__ __forceinline__ void store_half(unsigned char* a, int m, int h, const float* v) {
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
@@ -139,7 +153,7 @@ __device__ __forceinline__ void store_half(unsigned char* a, int m, int h, const
     umma::split8(v + 8 * c, p);
 #pragma unroll
     for (int piece = 0; piece < 3; ++piece)
-      *reinterpret_cast<uint4*>(a + (piece * 4 + 2 * h + c) * CHUNK + m * 16) = p[piece];
+      *reinterpret_cast<uint4*>(a + (piece * 4 + 2 * h + c) * PLANE + m * 16) = p[piece];
   }
 }
 
@@ -169,187 +183,304 @@ __device__ __forceinline__ void tile_of(const TileGrid& G, int64_t t, int w, int
   *n = (int)(t / G.ty);
 }
 
-// Forward pass of one 26 x 10 pixel tile per iteration (persistent, two
-// blocks per SM), all three layers:
-//  1. the input's two channels as one 16-byte chunk of pieces per pixel
-//     (x0 hi, mid, lo, x1 hi, mid, lo, 0, 0); a K = 16 step of the MMA takes
-//     two taps of it, the ninth is paired with zeros;
-//  2. TMEM -> bias, ReLU (0 outside the image) -> pieces in the planes -> the
-//     32 x 32 convolution;
-//  3. TMEM -> bias, ReLU -> each pixel's products with layer 3's nine taps,
-//     summed over the neighbours through shared memory.
+// ---------------------------------------------------------------- forward pass
+// All three layers, row by row: a block marches down the rows of a task, 128
+// pixels (the MMA's rows) at a time: one segment of 128 columns, or 2 or 4
+// segments of 64 or 32 that march through different tasks of the same height.
+// A layer's last two columns of a segment see the next one, so a segment of P
+// columns yields P - 6.
+//  1. The network input as one 16-byte chunk of pieces per pixel (x0 hi, mid,
+//     lo, x1 hi, mid, lo, 1, 0; the one for the bias); the last three rows in
+//     three slots. A K = 16
+//     step takes two taps; the slot of a row rotates, and the weights with it
+//     (three copies); the ninth tap is paired with zeros.
+//  2. TMEM -> ReLU (0 outside the image) -> pieces in shared memory. The
+//     N = 96 columns of an MMA are the three output rows that this row feeds
+//     (tap rows 0, 1, 2): the read of the 128 x 16 operand, 59 cycles for N =
+//     32 and 67 for N = 96, sets the pace. 18 MMAs per row against 54.
+//  3. A pixel stays in its TMEM lane, so its thread adds the row sums of three
+//     successive rows in registers: bias, ReLU, the products with layer 3's
+//     nine taps, which are summed over the rows in registers and over the
+//     columns through shared memory.
+// Warps 0-3 make layer 1's output, warps 4-7 read layer 2's, warp 8 issues the
+// MMAs. The tensor core cuts the low bits of its sums: a sum is six K steps of
+// leading pieces after the middle and last ones, the rest is FP32 addition.
 // TRAIN keeps the activations and writes logits, otherwise probabilities.
-// Bound: the MMAs. An M = 128, K = 16 step with operands in shared memory takes
-// 59 cycles for N = 32 (72 for N = 128: the read of A sets it), 182 steps per
-// tile. 64 slices of 256 x 256: 0.69 ms, 10.6 k of the 12.1 k cycles per tile
-// and SM (the FP32 kernels, one per layer with activations in memory: 5.6 ms).
+// Bound: shared memory, about 2,100 of the 2,350 cycles per row and SM (the
+// MMAs' operands half of it, layer 3's weights a quarter). 64 slices of 256 x
+// 256: 0.43 ms. Tiles of 32 x 12 pixels with N = 32 took 0.69 ms (54 MMAs of 59
+// cycles per 128 pixels), FP32 kernels, one per layer, 5.6 ms. Eight warps on
+// layer 2's side instead of four: 0.58 against 0.51 ms at that stage (spills).
+constexpr int SP = 128, SPAD = SP + 8;      // pixels of a row step; the taps read two past them
+constexpr uint32_t ROW = SPAD * 16;         // bytes of a chunk plane
+constexpr uint32_t W2KX = 4 * 96 * 16;      // bytes of one kx of layer 2's weights
+constexpr int FWD_THREADS = 288;
+
+struct alignas(16) FwdSmem {
+  unsigned char a[2][12 * ROW];             // layer 1's row: [piece][chunk] planes, two rows
+  unsigned char x[3][ROW];                  // the network input's rows, slot = row mod 3
+  unsigned char zero[SP * 16];
+  unsigned char w2[3 * W2KX];
+  unsigned char w1[3 * 5 * 1024];           // [rotation][MMA][tap of two][output channel][8]
+  float w3[9 * 32];                         // [tap][channel]
+  alignas(16) float b2[32];
+  float b3;
+  float z[2][3][SPAD];                      // layer 3's sums over the rows, per tap column
+  uint32_t tmem;
+  // layer 1's sums ready [2], input row written, planes written [2], layer 2's sums ready [2] and read [2]
+  uint64_t l1[2], xw, aw[2], l2[2], rd[2];
+};
+static_assert(sizeof(FwdSmem) <= 113 * 1024, "two blocks per SM");
+
+struct FwdGrid {
+  int H, W, P, nseg, zw, h, tx, ty;  // segment columns, segments per row step, output columns and rows of a task, tasks along x, y
+  int64_t tasks, groups;             // groups of nseg tasks
+};
+
 template <bool TRAIN>
-__global__ void __launch_bounds__(TILE_THREADS, 2)
+__global__ void __launch_bounds__(FWD_THREADS, 2)
     forward_kernel(const float* __restrict__ x, const __nv_bfloat16* __restrict__ wb, const float* __restrict__ w,
-                   float* __restrict__ a1, float* __restrict__ a2, float* __restrict__ out, const TileGrid G) {
+                   float* __restrict__ a1, float* __restrict__ a2, float* __restrict__ out, const FwdGrid G) {
   extern __shared__ __align__(16) unsigned char smem[];
-  TileSmem& S = *reinterpret_cast<TileSmem*>(smem);
+  FwdSmem& S = *reinterpret_cast<FwdSmem*>(smem);
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const size_t plane = (size_t)G.H * G.W;
-  load_w2(S.w2, wb + OFF_OP, tid);
-  for (int i = tid; i < 5 * 512; i += TILE_THREADS) {
-    const int e = i % 8, co = (i / 8) % 32, tap = 2 * (i / 512) + (i / 256) % 2;
-    reinterpret_cast<__nv_bfloat16*>(S.w1)[i] =
-        e < 6 && tap < 9 ? wb[OFF_W1 + (co * 2 + e / 3) * 9 + tap] : __float2bfloat16(0.0f);
-  }
-  for (int i = tid; i < 288; i += TILE_THREADS) S.w3[(i % 9) * 32 + i / 9] = __bfloat162float(wb[OFF_W3 + i]);
-  if (tid < 32) {
-    S.b1[tid] = w[OFF_B1 + tid];
-    S.b2[tid] = w[OFF_B2 + tid];
-  }
+  for (int i = tid; i < NW2 / 8; i += FWD_THREADS)
+    reinterpret_cast<uint4*>(S.w2)[i] = __ldg(reinterpret_cast<const uint4*>(wb + OFF_OP) + i);
+  for (int i = tid; i < NOP1 / 8; i += FWD_THREADS)
+    reinterpret_cast<uint4*>(S.w1)[i] = __ldg(reinterpret_cast<const uint4*>(wb + OFF_OP1) + i);
+  for (int i = tid; i < 288; i += FWD_THREADS) S.w3[(i % 9) * 32 + i / 9] = __bfloat162float(wb[OFF_W3 + i]);
+  if (tid < 32) S.b2[tid] = w[OFF_B2 + tid];
+  // what no row writes: the planes' and input rows' tails, the zero rows
+  if (tid < 27 * 8)
+    *reinterpret_cast<uint4*>((tid < 24 * 8 ? S.a[0] + (tid / 8) * ROW : S.x[0] + (tid / 8 - 24) * ROW) +
+                              (SP + tid % 8) * 16) = make_uint4(0, 0, 0, 0);
+  if (tid < SP) *reinterpret_cast<uint4*>(S.zero + tid * 16) = make_uint4(0, 0, 0, 0);
   if (tid == 0) {
     S.b3 = w[OFF_B3];
-    S.failed = 0;
-    for (int i = 0; i < 4; ++i) umma::bar_init(&S.bar[i]);
+    for (int i = 0; i < 2; ++i) {
+      umma::bar_init(&S.l1[i]);
+      umma::bar_init(&S.l2[i]);
+      umma::bar_init(&S.aw[i], 4);
+      umma::bar_init(&S.rd[i], 4);
+    }
+    umma::bar_init(&S.xw, 4);
     umma::bar_init_fence();
   }
   if (warp == 0) umma::tmem_alloc(&S.tmem, 256);
+  umma::fence_smem();
   umma::fence_before();
   __syncthreads();
   umma::fence_after();
-  const uint32_t tmem = S.tmem, tq = tmem + ((uint32_t)(warp & 3) << 21);
-  // layer 1's accumulators take the columns of layer 2's: they are read before those are written
-  float xr[2][2];
-  auto fetch = [&](int64_t t) {
-    int n, oy, ox;
-    tile_of(G, t, ZW, ZH, &n, &oy, &ox);
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int i = tid + j * TILE_THREADS, gy = oy - 3 + i / PW, gx = ox - 3 + i % PW;
-      const bool in = t < G.tiles && i < (R1 + 2) * PW && gy >= 0 && gy < G.H && gx >= 0 && gx < G.W;
-#pragma unroll
-      for (int c = 0; c < 2; ++c) xr[j][c] = in ? __ldg(x + (2 * (size_t)n + c) * plane + (size_t)gy * G.W + gx) : 0.0f;
-    }
-  };
-  fetch(blockIdx.x);
-  uint32_t phase = 0;
-  for (int64_t tile = blockIdx.x; tile < G.tiles; tile += gridDim.x, phase ^= 1) {
-    int n, oy, ox;
-    tile_of(G, tile, ZW, ZH, &n, &oy, &ox);
-    // ---- layer 1
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int i = tid + j * TILE_THREADS;
-      if (i < NPX) {
+  const uint32_t tmem = S.tmem;  // layer 1: 2 x 32 columns; layer 2: 2 x 96 from column 64
+  const uint32_t tq = tmem + ((uint32_t)(warp & 3) << 21);
+  const int rows = G.h + 4;      // layer 1 rows of a task; its network input rows: two more
+  uint32_t g = 0;                // rows done: buffer g & 1, its use g >> 1
+  bool ok = true;                // false once a wait has run out: nothing more is waited for or signalled
+
+  // of the block's 288 x 96 registers: 128 x 72, 128 x 120, 32 x 96
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+    const int p = tid, sg = p / G.P, lc = p - sg * G.P;
+    for (int64_t grp = blockIdx.x; grp < G.groups; grp += gridDim.x) {
+      int64_t t = grp * G.nseg + sg;
+      const bool live = t < G.tasks && sg < G.nseg;
+      const int ox = (int)(t % G.tx) * G.zw;
+      t /= G.tx;
+      const int y0 = (int)(t % G.ty) * G.h;
+      const size_t n = (size_t)(t / G.ty);
+      const int xc = ox - 3 + lc;
+      const bool xin = live && xc >= 0 && xc < G.W;
+      const float* xp = x + 2 * n * plane + xc;
+      float x0 = 0.0f, x1 = 0.0f;
+      auto fetch = [&](int r) {
+        const int gy = y0 - 3 + r;
+        const bool in = xin && gy >= 0 && gy < G.H;
+        x0 = in ? __ldg(xp + (size_t)gy * G.W) : 0.0f;
+        x1 = in ? __ldg(xp + plane + (size_t)gy * G.W) : 0.0f;
+      };
+      // writes the fetched row into its slot and fetches another
+      auto put = [&](int r, int next) {
         uint32_t h0, m0, l0;
-        umma::split2(xr[j][0], xr[j][1], &h0, &m0, &l0);  // low halves: channel 0, high halves: channel 1
-        *reinterpret_cast<uint4*>(S.a + i * 16) = make_uint4(__byte_perm(h0, m0, 0x5410), __byte_perm(l0, h0, 0x7610),
-                                                             __byte_perm(m0, l0, 0x7632), 0u);
-      }
-    }
-    if (tid < 128) *reinterpret_cast<uint4*>(S.a + (NPX + tid) * 16) = make_uint4(0, 0, 0, 0);
-    umma::fence_smem();
-    __syncthreads();
-    if (warp == 0 && umma::elect()) {
-      const uint32_t a0 = umma::smem_addr(S.a);
-      const uint64_t w0 = umma::desc_k(umma::smem_addr(S.w1), 512);
-#pragma unroll
-      for (int p = 0; p < 5; ++p) {
-        const int s0 = (2 * p / 3) * PW + (2 * p) % 3, s1 = ((2 * p + 1) / 3) * PW + (2 * p + 1) % 3;
-#pragma unroll
-        for (int t = 0; t < 4; ++t)
-          umma::mma(tmem + t * 32, umma::desc_k(a0 + (t * 128 + s0) * 16, (p < 4 ? s1 - s0 : NPX - t * 128 - s0) * 16),
-                    w0 + p * 64, umma::idesc(128, 32, false), p > 0);
-      }
-      umma::commit(&S.bar[0]);
-    }
-    __syncwarp();
-    fetch(tile + gridDim.x);
-    if (!umma::bar_wait(&S.bar[0], phase)) S.failed = 1;
-    umma::fence_after();
-    __syncthreads();  // every block thread past the wait: the input's overlay is free
-    if (S.failed) break;
+        umma::split2(x0, x1, &h0, &m0, &l0);  // low halves: channel 0, high halves: channel 1
+        *reinterpret_cast<uint4*>(S.x[r % 3] + p * 16) = make_uint4(
+            __byte_perm(h0, m0, 0x5410), __byte_perm(l0, h0, 0x7610), __byte_perm(m0, l0, 0x7632), 0x3f80u);
+        fetch(next);
+      };
+      fetch(0);
+      put(0, 1);
+      put(1, 2);
+      put(2, 3);
+      umma::fence_smem();
+      __syncwarp();
+      if (lane == 0 && ok) umma::bar_arrive(&S.xw);
 #pragma unroll 1
-    for (int r = warp; r < R1; r += R2) {
-      const int gy = oy - 2 + r, gx = ox - 2 + lane;
-      const bool in = gy >= 0 && gy < G.H && gx >= 0 && gx < G.W;
-      const bool own = TRAIN && in && r >= 2 && r < 2 + ZH && lane >= 2 && lane < 2 + ZW;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        float v[16];
-        umma::tmem_ld16(tq + (r >> 2) * 32 + 16 * h, v);
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          v[c] = in ? fmaxf(v[c] + S.b1[16 * h + c], 0.0f) : 0.0f;
-          if (own) a1[((size_t)n * 32 + 16 * h + c) * plane + (size_t)gy * G.W + gx] = v[c];
+      for (int r = 0; r < rows; ++r, ++g) {
+        const int b = g & 1;
+        ok = ok && umma::bar_wait(&S.l1[b], g >> 1 & 1);
+        umma::fence_after();
+        if (r + 1 < rows) {  // the slot of row r is free
+          put(r + 3, r + 4);
+          umma::fence_smem();
+          __syncwarp();
+          if (lane == 0 && ok) umma::bar_arrive(&S.xw);
         }
-        store_half(S.a, r * PW + lane, h, v);
+        const int gy = y0 - 2 + r, gx = xc + 1;
+        const bool in = live && gy >= 0 && gy < G.H && gx >= 0 && gx < G.W;
+        const bool own = TRAIN && in && r >= 2 && r < 2 + G.h && lc >= 2 && lc < 2 + G.zw;
+        float v[TRAIN ? 32 : 16];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float* vh = v + (TRAIN ? 16 * h : 0);
+          umma::tmem_ld16(tq + b * 32 + 16 * h, vh);
+#pragma unroll
+          for (int c = 0; c < 16; ++c) vh[c] = in ? fmaxf(vh[c], 0.0f) : 0.0f;
+          // the planes are free once the MMAs of two rows ago are done
+          if (h == 0 && g >= 2) ok = ok && umma::bar_wait(&S.l2[b], (g >> 1) - 1 & 1);
+          store_half<ROW>(S.a[b], p, h, vh);
+        }
+        umma::fence_smem();
+        umma::fence_before();
+        __syncwarp();
+        if (lane == 0 && ok) umma::bar_arrive(&S.aw[b]);
+        if (TRAIN && own) {
+          float* q = a1 + n * 32 * plane + (size_t)gy * G.W + gx;
+#pragma unroll
+          for (int c = 0; c < 32; ++c, q += plane) *q = v[c % (TRAIN ? 32 : 16)];
+        }
       }
     }
-    zero_tail(S.a, tid);
-    // ---- layer 2
-    umma::fence_smem();
-    umma::fence_before();
-    __syncthreads();
-    if (warp == 0 && umma::elect()) {
+  } else if (warp < 8) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
+    const int p = tid - SP, sg = p / G.P, lc = p - sg * G.P;
+    for (int64_t grp = blockIdx.x; grp < G.groups; grp += gridDim.x) {
+      int64_t t = grp * G.nseg + sg;
+      const bool live = t < G.tasks && sg < G.nseg;
+      const int ox = (int)(t % G.tx) * G.zw;
+      t /= G.tx;
+      const int y0 = (int)(t % G.ty) * G.h;
+      const size_t n = (size_t)(t / G.ty);
+      float A[32], B[32];        // tap rows 0 + 1 of the row before, tap row 0 of this one
+      float za[3], zb[3];        // layer 3: rows of taps 0 + 1, 0
+#pragma unroll
+      for (int c = 0; c < 32; ++c) A[c] = B[c] = 0.0f;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) za[k] = zb[k] = 0.0f;
+#pragma unroll 1
+      for (int r = 0; r < rows; ++r, ++g) {
+        const int b = g & 1;
+        ok = ok && umma::bar_wait(&S.l2[b], g >> 1 & 1);
+        umma::fence_after();
+        // layer 2's row that this row completes
+        const int gy = y0 - 3 + r, gx = ox - 1 + lc;
+        const bool in = live && r >= 2 && gy >= 0 && gy < G.H && gx >= 0 && gx < G.W;
+        const bool own = TRAIN && in && r >= 3 && r < 3 + G.h && lc >= 1 && lc < 1 + G.zw;
+        float2 dot[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) dot[k] = make_float2(0.0f, 0.0f);
+        float* a2p = TRAIN ? a2 + n * 32 * plane + (int64_t)gy * G.W + gx : nullptr;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int c0 = 8 * q;
+          float v[8], u[8];
+          umma::tmem_ld8(tq + 64 + b * 96 + 64 + c0, v);
+          const float4 e0 = *reinterpret_cast<const float4*>(&S.b2[c0]), e1 = *reinterpret_cast<const float4*>(&S.b2[c0 + 4]);
+          const float bias[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            v[c] = in ? fmaxf(A[c0 + c] + v[c] + bias[c], 0.0f) : 0.0f;
+            if (TRAIN && own) *a2p = v[c];
+            if (TRAIN) a2p += plane;
+          }
+          umma::tmem_ld8(tq + 64 + b * 96 + 32 + c0, u);
+#pragma unroll
+          for (int c = 0; c < 8; ++c) A[c0 + c] = B[c0 + c] + u[c];
+          umma::tmem_ld8(tq + 64 + b * 96 + c0, B + c0);
+#pragma unroll
+          for (int k = 0; k < 9; ++k)
+#pragma unroll
+            for (int c = 0; c < 8; c += 4) {
+              const float4 f = *reinterpret_cast<const float4*>(&S.w3[k * 32 + c0 + c]);
+              dot[k] = ffma2(make_float2(v[c], v[c + 1]), make_float2(f.x, f.y), dot[k]);
+              dot[k] = ffma2(make_float2(v[c + 2], v[c + 3]), make_float2(f.z, f.w), dot[k]);
+            }
+        }
+        umma::fence_before();
+        __syncwarp();
+        if (lane == 0 && ok) umma::bar_arrive(&S.rd[b]);
+        // layer 3's row that this row completes
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          S.z[b][k][p] = za[k] + (dot[6 + k].x + dot[6 + k].y);
+          za[k] = zb[k] + (dot[3 + k].x + dot[3 + k].y);
+          zb[k] = dot[k].x + dot[k].y;
+        }
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        const int zy = y0 + r - 4, zx = ox + lc;
+        if (live && r >= 4 && zy < G.H && lc < G.zw && zx < G.W) {
+          const float z = S.b3 + ((S.z[b][0][p] + S.z[b][1][p + 1]) + S.z[b][2][p + 2]);
+          // a wait that ran out leaves the output marked as missing
+          out[n * plane + (size_t)zy * G.W + zx] = !ok ? __int_as_float(0x7fc00000) : TRAIN ? z : 1.0f / (1.0f + expf(-z));
+        }
+      }
+    }
+  } else {
+    const uint64_t w2 = umma::desc_k(umma::smem_addr(S.w2), 96 * 16), w1 = umma::desc_k(umma::smem_addr(S.w1), 512);
+    const uint32_t x0 = umma::smem_addr(S.x);
+    uint32_t xn = 0;
+    // layer 1's row r of the task, row number gl of the block
+    auto layer1 = [&](int r, uint32_t gl) {
+      ok = ok && umma::bar_wait(&S.xw, xn & 1);
+      ++xn;
       umma::fence_after();
-      conv32_issue(S, tmem, 0);
-      conv32_issue(S, tmem, 1);
-    }
-    __syncwarp();
-    // ---- layer 3
-    const int gy = oy - 1 + warp, gx = ox - 1 + lane;
-    const bool in = gy >= 0 && gy < G.H && gx >= 0 && gx < G.W;
-    float v[32];
-    bool ok = conv32_read(S, tmem, warp, phase, v);
+      if (ok && umma::elect()) {
+        const uint64_t wr = w1 + (r % 3) * (5 * 64);
+        const uint32_t d = tmem + (gl & 1) * 32;
+        constexpr uint32_t id = umma::idesc(128, 32, false);
 #pragma unroll
-    for (int c = 0; c < 32; ++c) {
-      v[c] = in ? fmaxf(v[c] + S.b2[c], 0.0f) : 0.0f;
-      if (TRAIN && in && warp >= 1 && warp < 1 + ZH && lane >= 1 && lane < 1 + ZW)
-        a2[((size_t)n * 32 + c) * plane + (size_t)gy * G.W + gx] = v[c];
-    }
-    float dot[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      float2 d = make_float2(0.0f, 0.0f);
-#pragma unroll
-      for (int c = 0; c < 32; c += 4) {
-        const float4 q = *reinterpret_cast<const float4*>(&S.w3[k * 32 + c]);
-        d = ffma2(make_float2(v[c], v[c + 1]), make_float2(q.x, q.y), d);
-        d = ffma2(make_float2(v[c + 2], v[c + 3]), make_float2(q.z, q.w), d);
+        for (int q = 0; q < 3; ++q) umma::mma(d, umma::desc_k(x0 + q * 16, ROW), wr + q * 64, id, q > 0);
+        umma::mma(d, umma::desc_k(x0 + 2 * ROW, 16), wr + 3 * 64, id, true);
+        umma::mma(d, umma::desc_k(x0 + 2 * ROW + 32, ROW - 32), wr + 4 * 64, id, true);
+        umma::commit(&S.l1[gl & 1]);
       }
-      dot[k] = d.x + d.y;
-    }
-    for (int t = 0; t < M2 / 128; ++t) ok = ok && umma::bar_wait(&S.bar[1 + t], phase);
-    if (!ok) S.failed = 1;
-    umma::fence_before();
-    __syncthreads();  // every MMA has read the planes: the partial sums take their place
-    if (S.failed) break;
-    float* pp = reinterpret_cast<float*>(S.a);
+      __syncwarp();
+    };
+    for (int64_t grp = blockIdx.x; grp < G.groups; grp += gridDim.x) {
+      layer1(0, g);
+#pragma unroll 1
+      for (int r = 0; r < rows; ++r, ++g) {
+        if (r + 1 < rows) layer1(r + 1, g + 1);
+        const int b = g & 1;
+        ok = ok && umma::bar_wait(&S.aw[b], g >> 1 & 1);
+        if (g >= 2) ok = ok && umma::bar_wait(&S.rd[b], (g >> 1) - 1 & 1);
+        umma::fence_after();
+        if (ok && umma::elect()) {
+          const uint64_t a = umma::desc_k(umma::smem_addr(S.a[b]), ROW);
+          constexpr uint32_t id = umma::idesc(128, 96, false);
 #pragma unroll
-    for (int k = 0; k < 9; ++k) pp[k * M2 + tid] = dot[k];
-    __syncthreads();
-    const int zy = oy + warp, zx = ox + lane;
-    if (warp < ZH && lane < ZW && zy < G.H && zx < G.W) {
-      float z = S.b3;
+          for (int piece = 2; piece >= 0; --piece)
 #pragma unroll
-      for (int k = 0; k < 9; ++k) z += pp[k * M2 + tid + (k / 3) * PW + k % 3];
-      out[(size_t)n * plane + (size_t)zy * G.W + zx] = TRAIN ? z : 1.0f / (1.0f + expf(-z));
-    }
-    umma::fence_after();
-    __syncthreads();
-  }
-  if (S.failed) {  // a wait ran out: the block's remaining outputs are marked as missing
-    for (int64_t tile = blockIdx.x; tile < G.tiles; tile += gridDim.x) {
-      int n, oy, ox;
-      tile_of(G, tile, ZW, ZH, &n, &oy, &ox);
-      if (warp < ZH && lane < ZW && oy + warp < G.H && ox + lane < G.W)
-        out[(size_t)n * plane + (size_t)(oy + warp) * G.W + ox + lane] = __int_as_float(0x7fc00000);
+            for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+              for (int k = 0; k < 2; ++k)
+                umma::mma(tmem + 64 + b * 96, a + ((piece * 4 + 2 * k) * ROW / 16 + kx),
+                          w2 + (kx * W2KX + k * 2 * 1536) / 16, id, piece < 2 || kx > 0 || k > 0);
+          umma::commit(&S.l2[b]);
+        }
+        __syncwarp();
+      }
     }
   }
+  umma::fence_before();
   __syncthreads();
   if (warp == 0) umma::tmem_free(tmem, 256);
 }
 
 // Data gradients of a 30 x 12 tile: d2 = layer 3's transposed convolution of
 // dz times (a2 > 0), written once and as pieces into the planes; d1 = layer
-// 2's transposed convolution of d2 times (a1 > 0) by conv32_issue. Bound as
-// the forward pass; 32 x 64 x 64 pixels: 42 us.
+// 2's transposed convolution of d2 times (a1 > 0) by conv32_issue. Bound: the
+// MMAs (59 cycles each, set by the read of A, 162 per tile) and the reads of a1
+// and a2; 32 x 64 x 64 pixels: 41 us.
 __global__ void __launch_bounds__(TILE_THREADS, 2)
     dgrad_kernel(const float* __restrict__ dz, const __nv_bfloat16* __restrict__ wb, const float* __restrict__ a1,
                  const float* __restrict__ a2, float* __restrict__ d1, float* __restrict__ d2, const TileGrid G) {
@@ -361,7 +492,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
   for (int i = tid; i < 288; i += TILE_THREADS) S.w3[(i % 9) * 32 + i / 9] = __bfloat162float(wb[OFF_W3 + i]);
   if (tid == 0) {
     S.failed = 0;
-    for (int i = 0; i < 4; ++i) umma::bar_init(&S.bar[i]);
+    for (int i = 0; i < 3; ++i) umma::bar_init(&S.bar[i]);
     umma::bar_init_fence();
   }
   if (warp == 0) umma::tmem_alloc(&S.tmem, 256);
@@ -403,7 +534,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
         if (own)
 #pragma unroll
           for (int c = 0; c < 16; ++c) d2[o + c * plane] = v[c];
-        store_half(S.a, r * PW + lane, h, v);
+        store_half<CHUNK>(S.a, r * PW + lane, h, v);
       }
     }
     zero_tail(S.a, tid);
@@ -432,7 +563,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
           d1[o + (h + c) * plane] = !ok ? __int_as_float(0x7fc00000) : m[c] > 0.0f ? v[h + c] : 0.0f;
       }
     }
-    for (int t = 0; t < M2 / 128; ++t) ok = ok && umma::bar_wait(&S.bar[1 + t], phase);
+    for (int t = 0; t < M2 / 128; ++t) ok = ok && umma::bar_wait(&S.bar[t], phase);
     if (!ok) S.failed = 1;
     umma::fence_before();
     __syncthreads();
@@ -468,20 +599,23 @@ __device__ __forceinline__ void stage32(unsigned char* a, uint32_t stride, const
                                         int H, int W, int oy, int ox, int rows, int cols, int pitch, uint32_t inv,
                                         int len, int tid) {
   const int warps = (len + 31) / 32;
-#pragma unroll 2
+  float v[IT][8];  // every round's loads are under way before the first is split
+#pragma unroll
   for (int it = 0; it < IT; ++it) {
     const int wi = (tid >> 5) + it * (WG_THREADS / 32), c = wi / warps, m = (wi - c * warps) * 32 + (tid & 31);
-    if (c > 3) break;
     const int r = (int)((uint32_t)m * inv >> 16), q = m - r * pitch;
     const int gy = oy + r, gx = ox + q;
-    float v[8];
-    const bool in = r < rows && q < cols && gy >= 0 && gy < H && gx >= 0 && gx < W;
+    const bool in = c < 4 && r < rows && q < cols && gy >= 0 && gy < H && gx >= 0 && gx < W;
     const float* sp = src + (size_t)(8 * c) * plane + (size_t)gy * W + gx;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = in ? __ldg(sp + e * plane) : 0.0f;
+    for (int e = 0; e < 8; ++e) v[it][e] = in ? __ldg(sp + e * plane) : 0.0f;
+  }
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int wi = (tid >> 5) + it * (WG_THREADS / 32), c = wi / warps, m = (wi - c * warps) * 32 + (tid & 31);
     uint4 p[3];
-    umma::split8(v, p);
-    if (m < len)
+    umma::split8(v[it], p);
+    if (c < 4 && m < len)
 #pragma unroll
       for (int k = 0; k < 3; ++k) *reinterpret_cast<uint4*>(a + (k * 4 + c) * stride + m * 16) = p[k];
   }
@@ -864,6 +998,49 @@ TileGrid tile_grid(int n, int H, int W, int w, int h) {
   return G;
 }
 
+// Segment width (the one that wastes least of a row), equal output columns per
+// task, and the rows per task that let the blocks, two per SM, finish soonest
+// (a task computes four rows more than it yields).
+FwdGrid fwd_grid(int n, int H, int W, int slots) {
+  FwdGrid G;
+  G.H = H;
+  G.W = W;
+  int64_t best = INT64_MAX;
+  for (int P = 32; P <= SP; P *= 2) {
+    const int64_t tx = ((int64_t)W + P - 7) / (P - 6), cost = tx * P;
+    if (cost < best) {
+      best = cost;
+      G.P = P;
+      G.tx = (int)tx;
+    }
+  }
+  G.nseg = SP / G.P;
+  G.zw = (W + G.tx - 1) / G.tx;
+  int64_t time = INT64_MAX;
+  for (int ty = 1; ty <= std::min(H, 1024); ++ty) {
+    const int h = (int)(((int64_t)H + ty - 1) / ty);
+    const int64_t groups = ((int64_t)n * G.tx * ty + G.nseg - 1) / G.nseg, t = (groups + slots - 1) / slots * (h + 4);
+    if (t < time) {
+      time = t;
+      G.h = h;
+      G.ty = (H + h - 1) / h;
+    }
+  }
+  G.tasks = (int64_t)n * G.tx * G.ty;
+  G.groups = (G.tasks + G.nseg - 1) / G.nseg;
+  return G;
+}
+
+int launch_forward(bool train, const float* x, const __nv_bfloat16* wb, const float* w, float* a1, float* a2, float* out, int n, int H, int W,
+                   cudaStream_t s) {
+  int dev = 0, sms = 0;
+  QSL_CHECK_CUDA(cudaGetDevice(&dev));
+  QSL_CHECK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const FwdGrid G = fwd_grid(n, H, W, 2 * sms);
+  return launch_tiles(train ? forward_kernel<true> : forward_kernel<false>, FWD_THREADS, sizeof(FwdSmem), 2, 1, G.groups, s,
+                      x, wb, w, a1, a2, out, G);
+}
+
 // Strips of equal width, at most 62 columns, and as many rows as 256 pixels hold.
 WgradGrid wgrad_grid(int n, int H, int W) {
   WgradGrid G;
@@ -884,7 +1061,7 @@ WgradGrid wgrad_grid(int n, int H, int W) {
 
 struct qsl_cnn {
   float* w = nullptr;            // FP32 master parameters
-  __nv_bfloat16* wb = nullptr;   // BF16 copy used by the passes, and layer 2's operand layouts
+  __nv_bfloat16* wb = nullptr;   // BF16 copy used by the passes, and the operand layouts
   float* m = nullptr;            // Adam moments
   float* v = nullptr;
   int64_t steps = 0;
@@ -1027,6 +1204,7 @@ int qsl_cnn_create(const float* params, qsl_cnn** out) {
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->m, NPAR * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->v, NPAR * sizeof(float));
   if (e == cudaSuccess) e = cudaMemcpy(c->w, params, NPAR * sizeof(float), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemset(c->wb, 0, NWB * sizeof(__nv_bfloat16));  // the operands' unused elements
   if (e == cudaSuccess) e = cudaMemset(c->m, 0, NPAR * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(c->v, 0, NPAR * sizeof(float));
   if (e != cudaSuccess) {
@@ -1060,9 +1238,7 @@ int qsl_cnn_forward(qsl_cnn* c, const float* x, int n, int H, int W, float* prob
     qsl::set_error("bad CNN forward arguments");
     return QSL_EINVAL;
   }
-  const TileGrid G = tile_grid(n, H, W, ZW, ZH);
-  return launch_tiles(forward_kernel<false>, TILE_THREADS, sizeof(TileSmem), 2, 1, G.tiles, s, x, c->wb, c->w,
-                      (float*)nullptr, (float*)nullptr, prob, G);
+  return launch_forward(false, x, c->wb, c->w, nullptr, nullptr, prob, n, H, W, s);
 }
 
 int qsl_cnn_loss_grad(qsl_cnn* c, const float* x, const float* y, int n, int H, int W, float pos_weight, float* loss,
@@ -1078,9 +1254,8 @@ int qsl_cnn_loss_grad(qsl_cnn* c, const float* x, const float* y, int n, int H, 
   float *a1 = c->act, *a2 = a1 + P * 32, *d2 = a2 + P * 32, *d1 = d2 + P * 32, *z = d1 + P * 32, *dz = z + P;
   QSL_CHECK_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), s));
   QSL_CHECK_CUDA(cudaMemsetAsync(grad, 0, NPAR * sizeof(float), s));
-  const TileGrid GF = tile_grid(n, H, W, ZW, ZH), GD = tile_grid(n, H, W, DW, DH);
-  if ((rc = launch_tiles(forward_kernel<true>, TILE_THREADS, sizeof(TileSmem), 2, 1, GF.tiles, s, x, c->wb, c->w, a1, a2,
-                         z, GF)))
+  const TileGrid GD = tile_grid(n, H, W, DW, DH);
+  if ((rc = launch_forward(true, x, c->wb, c->w, a1, a2, z, n, H, W, s)))
     return rc;
   bce_kernel<<<(int)std::min<size_t>((P + BCE_THREADS - 1) / BCE_THREADS, 1024), BCE_THREADS, 0, s>>>(z, y, (int64_t)P, pos_weight, dz, loss,
                                                                           grad + OFF_B3);

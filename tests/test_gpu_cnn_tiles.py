@@ -1,6 +1,6 @@
-"""The tensor-core network kernels at the edges of their tiles (26 x 10 forward,
-30 x 12 data gradient, strips of at most 62 columns for the weight gradients)
-against the FP64 oracle, and with an infinite input."""
+"""The tensor-core network kernels at the edges of their segments and tiles
+(26, 58 or 122 columns forward, 30 x 12 data gradient, strips of at most 62
+columns for the weight gradients) against the FP64 oracle, and with an infinite input."""
 import numpy as np
 import pytest
 import torch
@@ -22,7 +22,7 @@ def _problem(seed, n, h, w):
 
 
 @pytest.mark.parametrize("n,h,w", [(1, 1, 1), (3, 2, 1), (2, 1, 130), (1, 10, 26), (2, 11, 27), (1, 12, 30), (1, 13, 31),
-                                   (2, 3, 62), (1, 5, 63), (1, 131, 3), (700, 3, 5)])
+                                   (2, 3, 62), (1, 5, 63), (1, 131, 3), (700, 3, 5), (1, 9, 58), (5, 7, 59), (1, 4, 122), (3, 2, 123)])
 def test_tile_edges_match_oracle(n, h, w):
     """FP32 sums of at most 288 terms per output and n h w terms per gradient
     entry: 1e-5 of a probability, 1e-4 of a block's largest gradient, the
