@@ -63,55 +63,84 @@ __global__ void __launch_bounds__(TX2* TY2) sobel2d_kernel(const float* __restri
   S[(int64_t)i0 * n1 + i1] = sqrtf(g0 * g0 + g1 * g1);
 }
 
-constexpr int TX3 = 32, TY3 = 4, TZ3 = 4;
+constexpr int TX3 = 32, TY3 = 8, TZ3 = 8;
 
+// Tile of 32 x 8 points over (i2, i1) marching along i0, one barrier per plane
+// (two slots). A thread keeps its 3 x 3 neighbourhood of the last three planes
+// in registers: 9 shared-memory reads per point (54 with the planes kept in
+// shared memory), and where it loads from is worked out once. The differences
+// are taken before the smoothing sums, so a smooth map keeps its precision.
+// 256 x 256 x 128: 50 us (32 x 4 tiles, planes in shared memory: 80 us);
+// the read and the write take 10 us of HBM, instructions set the time.
 __global__ void __launch_bounds__(TX3* TY3) sobel3d_kernel(const float* __restrict__ L, int n0, int n1, int n2,
                                                          const unsigned* fill_bits, float* __restrict__ S) {
-  // tile over (i1, i2) with a 1-point halo, marching along i0 with a rolling
-  // window of three planes
-  __shared__ float t[3][TY3 + 2][TX3 + 2];
+  constexpr int W = TX3 + 2, CELLS = (TY3 + 2) * W, IT = (CELLS + TX3 * TY3 - 1) / (TX3 * TY3);
+  __shared__ float t[2][CELLS];
   const float fill = *fill_bits ? ord2f(*fill_bits) : 0.0f;
-  int i2b = blockIdx.x * TX3, i1b = blockIdx.y * TY3;
-  int z0 = blockIdx.z * TZ3;
-  int z1 = min(z0 + TZ3, n0);
-  auto load_plane = [&](int slot, int i0) {
-    int ii0 = refl(i0, n0);
-    for (int k = threadIdx.y * TX3 + threadIdx.x; k < (TY3 + 2) * (TX3 + 2); k += TX3 * TY3) {
-      int r = k / (TX3 + 2), c = k % (TX3 + 2);
-      int i1 = refl(i1b + r - 1, n1), i2 = refl(i2b + c - 1, n2);
-      i1 = min(max(i1, 0), n1 - 1);
-      i2 = min(max(i2, 0), n2 - 1);
-      t[slot][r][c] = fetch(L, ((int64_t)ii0 * n1 + i1) * n2 + i2, fill);
-    }
+  const int i2b = blockIdx.x * TX3, i1b = blockIdx.y * TY3;
+  const int z0 = blockIdx.z * TZ3, z1 = min(z0 + TZ3, n0);
+  const int tid = threadIdx.y * TX3 + threadIdx.x;
+  const int64_t plane = (int64_t)n1 * n2;
+  int64_t at[IT];
+#pragma unroll
+  for (int k = 0; k < IT; ++k) {
+    const int cell = min(tid + k * TX3 * TY3, CELLS - 1), r = cell / W, c = cell % W;
+    const int i1 = min(max(refl(i1b + r - 1, n1), 0), n1 - 1), i2 = min(max(refl(i2b + c - 1, n2), 0), n2 - 1);
+    at[k] = (int64_t)i1 * n2 + i2;
+  }
+  float next[IT];
+  auto load = [&](int i0) {
+    const float* p = L + min(max(refl(i0, n0), 0), n0 - 1) * plane;
+#pragma unroll
+    for (int k = 0; k < IT; ++k) next[k] = fetch(p, at[k], fill);
   };
-  load_plane(0, z0 - 1);
-  load_plane(1, z0);
+  auto store = [&](int slot) {
+#pragma unroll
+    for (int k = 0; k < IT; ++k)
+      if (tid + k * TX3 * TY3 < CELLS) t[slot][tid + k * TX3 * TY3] = next[k];
+  };
+  const int i1 = i1b + threadIdx.y, i2 = i2b + threadIdx.x, o = (threadIdx.y + 1) * W + threadIdx.x + 1;
+  float m[9], q[9], p[9];  // the neighbourhood in the planes i0 - 1, i0, i0 + 1
+  auto read = [&](int slot, float* v) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) v[3 * a + b] = t[slot][o + (a - 1) * W + b - 1];
+  };
+  load(z0 - 1);
+  store(0);
+  load(z0);
+  __syncthreads();
+  read(0, m);
+  store(1);
+  load(z0 + 1);
+  __syncthreads();
+  read(1, q);
+#pragma unroll 2
   for (int i0 = z0; i0 < z1; ++i0) {
-    load_plane((i0 - z0 + 2) % 3, i0 + 1);
+    const int slot = (i0 - z0) & 1;
+    store(slot);
+    load(i0 + 2);
     __syncthreads();
-    int pm = (i0 - z0) % 3, pc = (i0 - z0 + 1) % 3, pp = (i0 - z0 + 2) % 3;
-    int r = threadIdx.y + 1, c = threadIdx.x + 1;
+    read(slot, p);
     // smoothing weights [1,2,1] on the two other axes; derivative [-1,0,1]
     float g0 = 0, g1 = 0, g2 = 0;
 #pragma unroll
-    for (int a = -1; a <= 1; ++a)
+    for (int a = 0; a < 3; ++a)
 #pragma unroll
-      for (int b = -1; b <= 1; ++b) {
-        float w = (a == 0 ? 2.0f : 1.0f) * (b == 0 ? 2.0f : 1.0f);
-        g0 += w * (t[pp][r + a][c + b] - t[pm][r + a][c + b]);
+      for (int b = 0; b < 3; ++b) {
+        const float w = (a == 1 ? 2.0f : 1.0f) * (b == 1 ? 2.0f : 1.0f);
+        const float* v = a == 0 ? m : (a == 1 ? q : p);
+        g0 += w * (p[3 * a + b] - m[3 * a + b]);
+        g1 += w * (v[6 + b] - v[b]);
+        g2 += w * (v[3 * b + 2] - v[3 * b]);
       }
+    if (i1 < n1 && i2 < n2) S[i0 * plane + (int64_t)i1 * n2 + i2] = sqrtf(g0 * g0 + g1 * g1 + g2 * g2);
 #pragma unroll
-    for (int a = -1; a <= 1; ++a)
-#pragma unroll
-      for (int b = -1; b <= 1; ++b) {
-        int plane = a < 0 ? pm : (a == 0 ? pc : pp);
-        float w = (a == 0 ? 2.0f : 1.0f) * (b == 0 ? 2.0f : 1.0f);
-        g1 += w * (t[plane][r + 1][c + b] - t[plane][r - 1][c + b]);
-        g2 += w * (t[plane][r + b][c + 1] - t[plane][r + b][c - 1]);
-      }
-    int i1 = i1b + threadIdx.y, i2 = i2b + threadIdx.x;
-    if (i1 < n1 && i2 < n2) S[((int64_t)i0 * n1 + i1) * n2 + i2] = sqrtf(g0 * g0 + g1 * g1 + g2 * g2);
-    __syncthreads();
+    for (int k = 0; k < 9; ++k) {
+      m[k] = q[k];
+      q[k] = p[k];
+    }
   }
 }
 
