@@ -503,12 +503,13 @@ struct TraceParams {
   int64_t few;                     // ck_wide_kernel traces launches of at most this many units, trace_kernel the others
 };
 
-// Problem and seed of launch seed j: global id, item, position.
-template <class R>
+// Problem and seed of launch seed j: global id, item, position. ITEMS = false:
+// the launch has the one item of its parameters.
+template <class R, bool ITEMS = true>
 __device__ __forceinline__ const Item<R>* resolve_seed(const TraceParams<R>& P, int64_t j, int64_t* g, double* x) {
   int64_t s = P.index ? P.index[j] : j;
   const Item<R>* E = &P.item0;
-  if (P.items) {
+  if (ITEMS && P.items) {
     int lo = 0, hi = P.n_items - 1;  // last item with seed_start <= s
     while (lo < hi) {
       int mid = (lo + hi + 1) >> 1;
@@ -1283,7 +1284,7 @@ __device__ __forceinline__ void dev_to_domain(R* y, const R* hh3) {
   }
 }
 
-template <class R, int NC>
+template <class R, int NC, bool ITEMS>
 __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
   constexpr bool F64 = sizeof(R) == 8;
   extern __shared__ __align__(32) unsigned char smem_raw[];
@@ -1347,7 +1348,8 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
             c_lines += (myu & 1) == 0;
             int64_t g;
             double xd[3];
-            E = resolve_seed(P, unit >> 1, &g, xd);
+            if (ITEMS) E = resolve_seed<R, true>(P, unit >> 1, &g, xd);
+            else resolve_seed<R, false>(P, unit >> 1, &g, xd);
             sgn = (unit & 1) ? R(-1) : R(1);
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
@@ -1868,20 +1870,25 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
 // the last lines 20.6 ms). FP32: at most 168 registers, so three blocks of 128
 // threads stay resident per SM (the allocation granularity would make 170 a
 // two-block kernel); FP64 keeps the compiler's choice (a cap would spill).
-template <int NC>
+// ITEMS: the problem comes from the launch's table; without one it is read from
+// the parameter bank instead of through a pointer (a dozen loads per step:
+// 256 x 256 x 128 volume 313 -> 306 ms, 1024^2 map 20.7 -> 20.4, refined map 48.6
+// -> 47.9). The same in
+// trace_kernel cost 15 % (its register allocation changes).
+template <int NC, bool ITEMS>
 __global__ void __maxnreg__(168) cell_kernel_f32(const __grid_constant__ TraceParams<float> P) {
-  cell_trace<float, NC>(P);
+  cell_trace<float, NC, ITEMS>(P);
 }
 template <int NC>
 __global__ void __launch_bounds__(256) cell_kernel_f64(const __grid_constant__ TraceParams<double> P) {
-  cell_trace<double, NC>(P);
+  cell_trace<double, NC, true>(P);
 }
 template <int NC>
-inline void (*cell_kernel_fn(float*))(const TraceParams<float>) {
-  return cell_kernel_f32<NC>;
+inline void (*cell_kernel_fn(float*, bool items))(const TraceParams<float>) {
+  return items ? cell_kernel_f32<NC, true> : cell_kernel_f32<NC, false>;
 }
 template <int NC>
-inline void (*cell_kernel_fn(double*))(const TraceParams<double>) {
+inline void (*cell_kernel_fn(double*, bool))(const TraceParams<double>) {
   return cell_kernel_f64<NC>;
 }
 
@@ -4388,6 +4395,7 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
   int threads = 32 * shape.warps_per_block;
   // persistent kernel: never launch more blocks than can be resident at once
   const bool use_cell = loc && cfg.integrator == QSL_DOPRI5_CELL;
+  const bool items = items_dev != nullptr;
   // lengths only, unless three lanes per line are asked for: the one-lane
   // polynomial kernel when every lane of the resident grid takes at most one
   // line direction (refinement passes; launches bound by their longest line)
@@ -4441,7 +4449,7 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
     QSL_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, coop_kernel_fn<NC>((R*)nullptr), threads, 0));
   else if (use_cell)
     QSL_CHECK_CUDA(
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, cell_kernel_fn<NC>((R*)nullptr), threads, smem));
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, cell_kernel_fn<NC>((R*)nullptr, items), threads, smem));
   else if (loc && cfg.geom == QSL_GEOM_SPHERICAL && cfg.interp_order > 1)
     QSL_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, trace_kernel<R, NC, true, true, true>,
                                                                  threads, 0));
@@ -4494,7 +4502,7 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
       if (sizeof(R) == 8 && NC == 9 && shape.line_lanes == 0 &&
           (size_t)blocks * shape.warps_per_block * kHandoff <= kContMax)
         P.handoff = kHandoff;
-      cell_kernel_fn<NC>((R*)nullptr)<<<blocks, threads, smem, stream>>>(P);
+      cell_kernel_fn<NC>((R*)nullptr, items)<<<blocks, threads, smem, stream>>>(P);
       qsl::count_launch();
       if (P.handoff) {
         QSL_CHECK_CUDA(cudaGetLastError());
