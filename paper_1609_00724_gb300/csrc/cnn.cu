@@ -205,7 +205,6 @@ __device__ __forceinline__ void tile_of(const TileGrid& G, int64_t t, int w, int
 // Warps 0-3 make layer 1's output, warps 4-7 read layer 2's, warp 8 issues the
 // MMAs. The tensor core cuts the low bits of its sums: a sum is six K steps of
 // leading pieces after the middle and last ones, the rest is FP32 addition.
-// TRAIN keeps the activations and writes logits, otherwise probabilities.
 // Bound: shared memory, about 2,100 of the 2,350 cycles per row and SM (the
 // MMAs' operands half of it, layer 3's weights a quarter). 64 slices of 256 x
 // 256: 0.43 ms. Tiles of 32 x 12 pixels with N = 32 took 0.69 ms (54 MMAs of 59
@@ -237,10 +236,9 @@ struct FwdGrid {
   int64_t tasks, groups;             // groups of nseg tasks
 };
 
-template <bool TRAIN>
 __global__ void __launch_bounds__(FWD_THREADS, 2)
     forward_kernel(const float* __restrict__ x, const __nv_bfloat16* __restrict__ wb, const float* __restrict__ w,
-                   float* __restrict__ a1, float* __restrict__ a2, float* __restrict__ out, const FwdGrid G) {
+                   float* __restrict__ out, const FwdGrid G) {
   extern __shared__ __align__(16) unsigned char smem[];
   FwdSmem& S = *reinterpret_cast<FwdSmem*>(smem);
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -327,27 +325,20 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
         }
         const int gy = y0 - 2 + r, gx = xc + 1;
         const bool in = live && gy >= 0 && gy < G.H && gx >= 0 && gx < G.W;
-        const bool own = TRAIN && in && r >= 2 && r < 2 + G.h && lc >= 2 && lc < 2 + G.zw;
-        float v[TRAIN ? 32 : 16];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          float* vh = v + (TRAIN ? 16 * h : 0);
-          umma::tmem_ld16(tq + b * 32 + 16 * h, vh);
+          float v[16];
+          umma::tmem_ld16(tq + b * 32 + 16 * h, v);
 #pragma unroll
-          for (int c = 0; c < 16; ++c) vh[c] = in ? fmaxf(vh[c], 0.0f) : 0.0f;
+          for (int c = 0; c < 16; ++c) v[c] = in ? fmaxf(v[c], 0.0f) : 0.0f;
           // the planes are free once the MMAs of two rows ago are done
           if (h == 0 && g >= 2) ok = ok && umma::bar_wait(&S.l2[b], (g >> 1) - 1 & 1);
-          store_half<ROW>(S.a[b], p, h, vh);
+          store_half<ROW>(S.a[b], p, h, v);
         }
         umma::fence_smem();
         umma::fence_before();
         __syncwarp();
         if (lane == 0 && ok) umma::bar_arrive(&S.aw[b]);
-        if (TRAIN && own) {
-          float* q = a1 + n * 32 * plane + (size_t)gy * G.W + gx;
-#pragma unroll
-          for (int c = 0; c < 32; ++c, q += plane) *q = v[c % (TRAIN ? 32 : 16)];
-        }
       }
     }
   } else if (warp < 8) {
@@ -374,11 +365,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
         // layer 2's row that this row completes
         const int gy = y0 - 3 + r, gx = ox - 1 + lc;
         const bool in = live && r >= 2 && gy >= 0 && gy < G.H && gx >= 0 && gx < G.W;
-        const bool own = TRAIN && in && r >= 3 && r < 3 + G.h && lc >= 1 && lc < 1 + G.zw;
         float2 dot[9];
 #pragma unroll
         for (int k = 0; k < 9; ++k) dot[k] = make_float2(0.0f, 0.0f);
-        float* a2p = TRAIN ? a2 + n * 32 * plane + (int64_t)gy * G.W + gx : nullptr;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int c0 = 8 * q;
@@ -389,8 +378,6 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
 #pragma unroll
           for (int c = 0; c < 8; ++c) {
             v[c] = in ? fmaxf(A[c0 + c] + v[c] + bias[c], 0.0f) : 0.0f;
-            if (TRAIN && own) *a2p = v[c];
-            if (TRAIN) a2p += plane;
           }
           umma::tmem_ld8(tq + 64 + b * 96 + 32 + c0, u);
 #pragma unroll
@@ -420,7 +407,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
         if (live && r >= 4 && zy < G.H && lc < G.zw && zx < G.W) {
           const float z = S.b3 + ((S.z[b][0][p] + S.z[b][1][p + 1]) + S.z[b][2][p + 2]);
           // a wait that ran out leaves the output marked as missing
-          out[n * plane + (size_t)zy * G.W + zx] = !ok ? __int_as_float(0x7fc00000) : TRAIN ? z : 1.0f / (1.0f + expf(-z));
+          out[n * plane + (size_t)zy * G.W + zx] = !ok ? __int_as_float(0x7fc00000) : 1.0f / (1.0f + expf(-z));
         }
       }
     }
@@ -474,6 +461,76 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
   umma::fence_before();
   __syncthreads();
   if (warp == 0) umma::tmem_free(tmem, 256);
+}
+
+// ---------------------------------------------------------------- training forward pass
+// One layer in FP32 on the CUDA cores, sums in the order (input channel, tap)
+// from the bias on. A gradient depends on the sign of every pre-activation, and
+// one that rounds to the other side of zero moves it by up to 1e-5: the
+// training pass keeps this order of sums, so its masks stay those it always
+// had. A thread has two pixels (rows 8 apart of a 16 x 16 tile) and all output
+// channels, in pairs (fma.rn.f32x2 rounds each like fmaf); four weights per
+// shared-memory read. Bound: those reads (16 wavefronts per tap for 64 pixels)
+// and the multiply-adds alike.
+constexpr int T = 16, TH = T + 2, CONV_THREADS = T * T / 2;
+template <int CIN, int COUT, bool RELU>
+__global__ void __launch_bounds__(CONV_THREADS) conv3x3_kernel(const float* __restrict__ x,
+                                                               const __nv_bfloat16* __restrict__ w,
+                                                               const float* __restrict__ b, float* __restrict__ y, int H,
+                                                               int W, int tx, int ty) {
+  extern __shared__ __align__(16) float sm[];
+  float* ws = sm;                   // [input channel][tap][output channel]
+  float* xs = sm + COUT * CIN * 9;  // [input channel][18][18]
+  constexpr int CO2 = (COUT + 1) / 2;
+  const int n = blockIdx.x / (tx * ty), t = blockIdx.x % (tx * ty), ox = t % tx * T, oy = t / tx * T;
+  const int tid = threadIdx.x;
+  const size_t plane = (size_t)H * W;
+  const float* xn = x + (size_t)n * CIN * plane;
+  for (int i = tid; i < CIN * TH * TH; i += CONV_THREADS) {
+    const int c = i / (TH * TH), r = (i / TH) % TH, q = i % TH, gy = oy + r - 1, gx = ox + q - 1;
+    xs[i] = (gy >= 0 && gy < H && gx >= 0 && gx < W) ? __ldg(xn + c * plane + (size_t)gy * W + gx) : 0.0f;
+  }
+  for (int i = tid; i < COUT * CIN * 9; i += CONV_THREADS)
+    ws[(i % (CIN * 9)) * COUT + i / (CIN * 9)] = __bfloat162float(w[i]);
+  __syncthreads();
+  const int lx = tid % T, ly = tid / T;
+  float2 acc[2][CO2];
+#pragma unroll
+  for (int c = 0; c < CO2; ++c) acc[0][c] = acc[1][c] = make_float2(b[2 * c], 2 * c + 1 < COUT ? b[2 * c + 1] : 0.0f);
+#pragma unroll 1
+  for (int ci = 0; ci < CIN; ++ci) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const float v0 = xs[(ci * TH + ly + k / 3) * TH + lx + k % 3], v1 = xs[(ci * TH + ly + 8 + k / 3) * TH + lx + k % 3];
+      const float* wk = ws + (ci * 9 + k) * COUT;
+      if (COUT == 1) {
+        acc[0][0].x = fmaf(v0, wk[0], acc[0][0].x);
+        acc[1][0].x = fmaf(v1, wk[0], acc[1][0].x);
+      } else {
+#pragma unroll
+        for (int c = 0; c < CO2; c += 2) {
+          const float4 f = *reinterpret_cast<const float4*>(wk + 2 * c);
+          acc[0][c] = ffma2(make_float2(v0, v0), make_float2(f.x, f.y), acc[0][c]);
+          acc[1][c] = ffma2(make_float2(v1, v1), make_float2(f.x, f.y), acc[1][c]);
+          acc[0][c + 1] = ffma2(make_float2(v0, v0), make_float2(f.z, f.w), acc[0][c + 1]);
+          acc[1][c + 1] = ffma2(make_float2(v1, v1), make_float2(f.z, f.w), acc[1][c + 1]);
+        }
+      }
+    }
+  }
+  const int gx = ox + lx;
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    const int gy = oy + ly + 8 * p;
+    if (gx < W && gy < H) {
+      float* yn = y + (size_t)n * COUT * plane + (size_t)gy * W + gx;
+#pragma unroll
+      for (int c = 0; c < COUT; ++c) {
+        const float v = c & 1 ? acc[p][c / 2].y : acc[p][c / 2].x;
+        yn[c * plane] = RELU ? fmaxf(v, 0.0f) : v;
+      }
+    }
+  }
 }
 
 // Data gradients of a 30 x 12 tile: d2 = layer 3's transposed convolution of
@@ -998,6 +1055,18 @@ TileGrid tile_grid(int n, int H, int W, int w, int h) {
   return G;
 }
 
+template <int CIN, int COUT, bool RELU>
+int launch_conv(const float* x, const __nv_bfloat16* w, const float* b, float* y, int n, int H, int W, cudaStream_t s) {
+  const size_t smem = sizeof(float) * (CIN * TH * TH + COUT * CIN * 9);
+  auto kern = conv3x3_kernel<CIN, COUT, RELU>;
+  QSL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int tx = (int)(((int64_t)W + T - 1) / T), ty = (int)(((int64_t)H + T - 1) / T);
+  kern<<<(unsigned)((int64_t)n * tx * ty), CONV_THREADS, smem, s>>>(x, w, b, y, H, W, tx, ty);
+  qsl::count_launch();
+  QSL_CHECK_CUDA(cudaGetLastError());
+  return QSL_OK;
+}
+
 // Segment width (the one that wastes least of a row), equal output columns per
 // task, and the rows per task that let the blocks, two per SM, finish soonest
 // (a task computes four rows more than it yields).
@@ -1029,16 +1098,6 @@ FwdGrid fwd_grid(int n, int H, int W, int slots) {
   G.tasks = (int64_t)n * G.tx * G.ty;
   G.groups = (G.tasks + G.nseg - 1) / G.nseg;
   return G;
-}
-
-int launch_forward(bool train, const float* x, const __nv_bfloat16* wb, const float* w, float* a1, float* a2, float* out, int n, int H, int W,
-                   cudaStream_t s) {
-  int dev = 0, sms = 0;
-  QSL_CHECK_CUDA(cudaGetDevice(&dev));
-  QSL_CHECK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const FwdGrid G = fwd_grid(n, H, W, 2 * sms);
-  return launch_tiles(train ? forward_kernel<true> : forward_kernel<false>, FWD_THREADS, sizeof(FwdSmem), 2, 1, G.groups, s,
-                      x, wb, w, a1, a2, out, G);
 }
 
 // Strips of equal width, at most 62 columns, and as many rows as 256 pixels hold.
@@ -1238,7 +1297,11 @@ int qsl_cnn_forward(qsl_cnn* c, const float* x, int n, int H, int W, float* prob
     qsl::set_error("bad CNN forward arguments");
     return QSL_EINVAL;
   }
-  return launch_forward(false, x, c->wb, c->w, nullptr, nullptr, prob, n, H, W, s);
+  int dev = 0, sms = 0;
+  QSL_CHECK_CUDA(cudaGetDevice(&dev));
+  QSL_CHECK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const FwdGrid G = fwd_grid(n, H, W, 2 * sms);
+  return launch_tiles(forward_kernel, FWD_THREADS, sizeof(FwdSmem), 2, 1, G.groups, s, x, c->wb, c->w, prob, G);
 }
 
 int qsl_cnn_loss_grad(qsl_cnn* c, const float* x, const float* y, int n, int H, int W, float pos_weight, float* loss,
@@ -1255,7 +1318,9 @@ int qsl_cnn_loss_grad(qsl_cnn* c, const float* x, const float* y, int n, int H, 
   QSL_CHECK_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), s));
   QSL_CHECK_CUDA(cudaMemsetAsync(grad, 0, NPAR * sizeof(float), s));
   const TileGrid GD = tile_grid(n, H, W, DW, DH);
-  if ((rc = launch_forward(true, x, c->wb, c->w, a1, a2, z, n, H, W, s)))
+  if ((rc = launch_conv<C1, C2, true>(x, c->wb + OFF_W1, c->w + OFF_B1, a1, n, H, W, s))) return rc;
+  if ((rc = launch_conv<C2, C2, true>(a1, c->wb + OFF_W2, c->w + OFF_B2, a2, n, H, W, s))) return rc;
+  if ((rc = launch_conv<C2, 1, false>(a2, c->wb + OFF_W3, c->w + OFF_B3, z, n, H, W, s)))
     return rc;
   bce_kernel<<<(int)std::min<size_t>((P + BCE_THREADS - 1) / BCE_THREADS, 1024), BCE_THREADS, 0, s>>>(z, y, (int64_t)P, pos_weight, dz, loss,
                                                                           grad + OFF_B3);

@@ -1873,8 +1873,7 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
 // ITEMS: the problem comes from the launch's table; without one it is read from
 // the parameter bank instead of through a pointer (a dozen loads per step:
 // 256 x 256 x 128 volume 313 -> 306 ms, 1024^2 map 20.7 -> 20.4, refined map 48.6
-// -> 47.9). The same in
-// trace_kernel cost 15 % (its register allocation changes).
+// -> 47.9). The same in trace_kernel cost 15 % (its register allocation changes).
 template <int NC, bool ITEMS>
 __global__ void __maxnreg__(168) cell_kernel_f32(const __grid_constant__ TraceParams<float> P) {
   cell_trace<float, NC, ITEMS>(P);
