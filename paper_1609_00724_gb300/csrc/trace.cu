@@ -474,9 +474,9 @@ struct Item {
 struct Cont {
   double muc;
   int64_t unit;
+  double h;
   int ic[3];
-  float h;
-  int zc, pad;
+  int zc;
 };
 
 template <class R>
@@ -1090,6 +1090,67 @@ __device__ __forceinline__ bool gt_bits(double x, double thr) {
   return __double_as_longlong(x) > __double_as_longlong(thr);
 }
 
+__device__ __forceinline__ double min_bits(double x, double y) { return gt_bits(x, y) ? y : x; }  // x, y >= 0
+__device__ __forceinline__ double max_bits(double x, double y) { return gt_bits(x, y) ? x : y; }
+
+// a / b within two roundings: the hardware's approximate reciprocal (about 20
+// bits, not an FP64-pipe instruction), one Newton step and a corrected quotient,
+// 5 FP64 instructions. Where b or the quotient is near the ends of the range, and
+// for b = 0 and infinite a, the division.
+__device__ __forceinline__ double quot(double a, double b) {
+  double x;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(b));
+  x = fma(fma(-b, x, 1.0), x, x);
+  const double q = a * x;
+  const unsigned eb = (__double2hiint(b) & 0x7ff00000) - 0x01000000u, eq = __double2hiint(q) & 0x7ff00000;
+  if (eb > 0x7e000000u || eq == 0x7ff00000u) return a / b;
+  return fma(fma(-b, q, a), x, q);
+}
+
+// The step of the FP64 cell-wise tracers: the controller's h, at most h_max and
+// the room left, or a little beyond the first plane along the derivative (tface
+// >= 0, the time to it) where that comes first. capped: it ends at the maximum
+// length.
+__device__ __forceinline__ double wide_step(double h, double h_max, double room, double tface, double tiny, bool* capped) {
+  const double hcap = min_bits(h, h_max), hf = fma(1.25, tface, tiny);
+  *capped = !gt_bits(room, hcap);
+  const double hs = *capped ? room : hcap;
+  if (!gt_bits(hs, hf)) return hs;
+  *capped = false;
+  return hf;
+}
+// Time to the plane at the offset r along an axis with the velocity vel, `far`
+// (at least 0) when it never comes or comes later.
+__device__ __forceinline__ double plane_time(double r, double vel, double far) {
+  if (((__double2hiint(vel) & 0x7fffffff) | __double2loint(vel)) == 0) return far;
+  const double q = quot(r, vel);
+  return min_bits(far, __double2hiint(q) < 0 ? 0.0 : q);
+}
+// Error e of a component against its tolerance. SKIP: 0 if it is below 2^-13 of
+// it (compared by exponents and leading digits), where it does not bear on
+// next_step; most steps, cut at a cell face, are there.
+template <bool SKIP>
+__device__ __forceinline__ double err_ratio(double e, double size, double tol_abs, double tol_rel) {
+  const double sc = fma(tol_rel, size, tol_abs);
+  if (SKIP && __double2hiint(e) < __double2hiint(sc) - (13 << 20)) return 0.0;
+  return quot(e, sc);
+}
+// Next step after a step hs with the error err (accepted up to 1): 0.9 hs times
+// err^(-1/4) and at least a fifth of it, or err^(-1/5) and at most five times.
+// The power: FP32's y (some 1e-6) times the third-order expansion of (1 - d)^(-1/N)
+// in d = 1 - err y^N; 10 FP64 instructions, pow has over 100. Not where the factor
+// is cut off (err below (0.9 / 5)^5 = 1.9e-4 or above (0.9 / 0.2)^4 = 410).
+__device__ __forceinline__ double next_step(double hs, double err) {
+  const bool rej = gt_bits(err, 1.0);
+  const float ef = fminf((float)err, 3e38f);
+  if (!(ef > 1.8e-4f)) return hs * 5.0;
+  if (!(ef < 420.0f)) return hs * 0.2;
+  const double y = (double)__powf(ef, rej ? -0.25f : -0.2f), y2 = y * y;
+  const double d = fma(-err, y2 * y2 * (rej ? 1.0 : y), 1.0);
+  const double f = 0.9 * fma(y * d, fma(rej ? 0.15625 : 0.12, d, rej ? 0.25 : 0.2), y);
+  return hs * (rej ? max_bits(f, 0.2) : min_bits(f, 5.0));
+}
+
 // The search runs in FP32 (an FP64 instruction takes 64 cycles of a warp on
 // GB300 whether or not it depends on the one before, an FP32 one about 1 to
 // 5), then Newton corrections with an FP64 residual and the FP32 derivative
@@ -1320,10 +1381,7 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
   int ic[3] = {0, 0, 0};
   R mu = 0, muc = 0, h = 0, sgn = 1;
   int steps = 0, zc = 0;
-  // FP64: the step controller's FP32 copies of the line's scales, and the
-  // cells beyond which a domain bound comes before the cell's own face
-  float hcf[3] = {1.0f, 1.0f, 1.0f}, orgf[3] = {0.0f, 0.0f, 0.0f}, hF = 0.0f, tinyF = 0.0f, hmaxF = 0.0f;
-  const float tolaF = (float)P.tol_abs, tolrF = (float)P.tol_rel;
+  // FP64: the cells beyond which a domain bound comes before the cell's own face
   int ilo[3] = {0, 0, 0}, ihi[3] = {0, 0, 0};
   unsigned long long c_stage = 0, c_acc = 0, c_rej = 0, c_land = 0, c_lines = 0;
   int iter = 0;
@@ -1360,14 +1418,9 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
             if constexpr (F64) {
 #pragma unroll
               for (int a = 0; a < 3; ++a) {
-                hcf[a] = (float)hh3[a];
-                orgf[a] = (float)E->F.org[a];
                 ilo[a] = (int)floor(E->lo[a]);
                 ihi[a] = (int)ceil(E->hi[a]) - 1;
               }
-              tinyF = (float)tiny;
-              hmaxF = (float)E->h_max;
-              hF = (float)E->h_init;
             }
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
@@ -1469,7 +1522,7 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
             e.steps = steps;
             k.muc = muc;
             k.unit = unit;
-            k.h = hF;
+            k.h = h;
             k.zc = zc;
             active = false;
           }
@@ -1533,7 +1586,6 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
       bool lo_dom[3], hi_dom[3];
       R hs;
       bool capped;
-      float hsF = 0.0f;
       if constexpr (F64) {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -1544,28 +1596,14 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
           if (lo_dom[a]) lo_pl[a] = E->lo[a] - R(ic[a]);
           if (hi_dom[a]) hi_pl[a] = E->hi[a] - R(ic[a]);
         }
-        float tfc = 1e30f;
+        R tface = R(1e30);
+        const int flip = (int)((unit & 1) << 31);  // the sign of the direction
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-          const float vel = (float)(sgn * k1[a]);
-          if (vel != 0.0f) tfc = fminf(tfc, __fdividef((float)((vel > 0.0f ? hi_pl[a] : lo_pl[a]) - y[a]), vel));
+          const R vel = __hiloint2double(__double2hiint(k1[a]) ^ flip, __double2loint(k1[a]));
+          tface = plane_time((__double2hiint(vel) >= 0 ? hi_pl[a] : lo_pl[a]) - y[a], vel, tface);
         }
-        const float hcap = fminf(hF, hmaxF);
-        const float hfF = 1.25f * fmaxf(tfc, 0.0f) + tinyF;
-        if ((float)room > 1.001f * hcap) {
-          capped = false;
-          hs = (R)hcap;
-          hsF = hcap;
-        } else {  // near the maximum length: the cap in FP64
-          capped = room <= (R)hcap;
-          hs = capped ? room : (R)hcap;
-          hsF = (float)hs;
-        }
-        if (hfF < hsF) {
-          hsF = hfF;
-          hs = (R)hfF;
-          capped = false;
-        }
+        hs = wide_step(h, E->h_max, room, tface, tiny, &capped);
       } else {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -1630,21 +1668,22 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
       const R w1 = hh * R(DD1), w3 = hh * R(DD3), w4 = hh * R(DD4), w5 = hh * R(DD5), w6 = hh * R(DD6),
               w7 = hh * R(DD7);
       R err = 0;
-      float errf = 0.0f;
       bool finite = true;
       if constexpr (F64) {
-        // the error estimate in FP64, its norm and the step controller in FP32:
-        // they only size the next step, and their divisions, comparisons and
-        // power were a third of a step's FP64 instructions
 #pragma unroll
         for (int i = 0; i < NC; ++i) {
-          const float hc = hcf[i % 3];
-          const float e =
-              fabsf((float)fma(e7, k7[i], fma(e6, k6[i], fma(e5, k5[i], fma(e4, k4[i], fma(e3, k3[i], e1 * k1[i])))))) * hc;
+          const R hc = hh3[i % 3];
+          const R e =
+              fabs(fma(e7, k7[i], fma(e6, k6[i], fma(e5, k5[i], fma(e4, k4[i], fma(e3, k3[i], e1 * k1[i])))))) * hc;
           if ((__double2hiint(t[i]) & 0x7ff00000) == 0x7ff00000) finite = false;
-          const float base = i < 3 ? fmaf((float)ic[i], hc, orgf[i]) : 0.0f;
-          const float m = fmaxf(fabsf(fmaf((float)y[i], hc, base)), fabsf(fmaf((float)t[i], hc, base)));
-          errf = fmaxf(errf, __fdividef(e, fmaf(tolrF, m, tolaF)));
+          R size;
+          if (i < 3) {
+            const R base = fma(R(ic[i]), hc, R(E->F.org[i]));
+            size = max_bits(fabs(fma(y[i], hc, base)), fabs(fma(t[i], hc, base)));
+          } else {  // deviations, in domain units
+            size = max_bits(fabs(y[i]), fabs(t[i])) * hc;
+          }
+          err = max_bits(err, err_ratio<false>(e, size, P.tol_abs, P.tol_rel));
         }
       } else {
 #pragma unroll
@@ -1666,23 +1705,22 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
           err = fmax(err, cdiv(e, P.tol_abs + P.tol_rel * fmax(ya, yb)));
         }
       }
+      R hnext = R(0);
+      if constexpr (F64) hnext = next_step(hs, err);
       if (!finite) {
         status = QSL_LINE_NONFINITE;
-      } else if (F64 ? errf > 1.0f : err > R(1)) {
+      } else if (F64 ? gt_bits(err, 1.0) : err > R(1)) {
         c_rej += 1;
         if constexpr (F64) {
-          hF = hsF * fmaxf(0.2f, 0.9f * __powf(errf, -0.25f));
-          if (hF < (float)E->h_min) status = QSL_LINE_STALL;
+          h = hnext;
+          if (gt_bits(E->h_min, h)) status = QSL_LINE_STALL;
         } else {
           h = hs * fmax(R(0.2), R(0.9) * cpow(err, R(-0.25)));
           if (h < E->h_min) status = QSL_LINE_STALL;
         }
       } else {
         c_acc += 1;
-        R hnext = R(0);
-        float hnextF = 0.0f;
-        if constexpr (F64) hnextF = hsF * ((errf == 0.0f) ? 5.0f : fminf(5.0f, 0.9f * __powf(errf, -0.2f)));
-        else hnext = hs * ((err == R(0)) ? R(5) : fmin(R(5), R(0.9) * cpow(err, R(-0.2))));
+        if constexpr (!F64) hnext = hs * ((err == R(0)) ? R(5) : fmin(R(5), R(0.9) * cpow(err, R(-0.2))));
         // First plane crossed within the step, on the dense output (4th-order
         // continuous extension): for every plane the step ends beyond, the
         // first sign change of dense(t) - plane over t = 1/4, 1/2, 3/4, 1
@@ -1778,8 +1816,7 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
           R t1 = hs - muc, t2 = mu + t1;
           muc = (t2 - mu) - t1;
           mu = t2;
-          if constexpr (F64) hF = hnextF;
-          else h = hnext;
+          h = hnext;
           zc = 0;
           if (capped) status = QSL_LINE_MAXLEN;
         } else {
@@ -1816,7 +1853,7 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
             lface = 2 * ax_c + up_c;
           } else {
             // enter the neighbouring cell
-            zc = (F64 ? (float)dl < tinyF : dl < tiny) ? zc + 1 : 0;
+            zc = (F64 ? gt_bits(tiny, dl) : dl < tiny) ? zc + 1 : 0;
             int na = sel3(ax_c, ic[0], ic[1], ic[2]) + (up_c ? 1 : -1);
             if (zc > 3 || na < 0 || na > sel3(ax_c, E->F.n[0], E->F.n[1], E->F.n[2]) - 2) {
               // grazing a face back and forth: stay in this cell for one step
@@ -1831,7 +1868,7 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
               else y[2] = up_c ? R(0) : R(1);
               kvalid = false;
             }
-            if constexpr (F64) hF = fmaxf(hnextF, hsF);
+            if constexpr (F64) h = max_bits(hnext, hs);
             else h = fmax(hnext, hs);
           }
         }
@@ -2606,8 +2643,7 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
   bool lo_dom = false, hi_dom = false, raw = false;
   int ic[3] = {0, 0, 0};
   R mu = 0, muc = 0, sgn = 1, max_len = 0;
-  float h = 0, h_max = 0, h_min = 0, tiny = 0, hcf = 0, orgf = 0;
-  const float tola = (float)P.tol_abs, tolr = (float)P.tol_rel;
+  R h = 0, h_max = 0, h_min = 0, tiny = 0, orgc = 0;
   int ilo = 0, ihi = 0;
   int steps = 0, zc = 0;
   unsigned long long c_stage = 0, c_acc = 0, c_rej = 0, c_land = 0, c_lines = 0;
@@ -2642,12 +2678,11 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
             for (int a = 0; a < 3; ++a) ih[a] = E->F.inv_h[a];
             ihc = sel3(c, ih[0], ih[1], ih[2]);
             hhc = R(1) / ihc;
-            hcf = (float)hhc;
-            orgf = (float)sel3(c, E->F.org[0], E->F.org[1], E->F.org[2]);
+            orgc = sel3(c, E->F.org[0], E->F.org[1], E->F.org[2]);
             max_len = E->max_len;
-            h_max = (float)E->h_max;
-            h_min = (float)E->h_min;
-            tiny = 1e-4f * h_max;
+            h_max = E->h_max;
+            h_min = E->h_min;
+            tiny = R(1e-4) * h_max;
             ilo = (int)floor(sel3(c, E->lo[0], E->lo[1], E->lo[2]));
             ihi = (int)ceil(sel3(c, E->hi[0], E->hi[1], E->hi[2])) - 1;
             kvalid = false;
@@ -2670,7 +2705,7 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
             zc = 0;
             int lface;
             const int status = wide_start(E, xd, sgn, c, j, ihc, ic, &y, &lface);
-            h = (float)E->h_init;
+            h = E->h_init;
             if (status != ST_RUNNING) {
               write_end_wide(P, E, unit, c, j, writer, y, ic, hhc, R(0), lface, status, 0);
               active = false;
@@ -2727,17 +2762,14 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
       }
       // step: controller size, capped a little beyond the first plane along k1
       const R r_lo = lo_pl - y, r_hi = hi_pl - y;  // position lanes
-      const float vel = (float)(sgn * k1);
-      float tf = 1e30f;
-      if (vel != 0.0f) tf = __fdividef((float)(vel > 0.0f ? r_hi : r_lo), vel);
-      const float tf0 = __shfl_sync(W.gm, tf, W.pos(0)), tf1 = __shfl_sync(W.gm, tf, W.pos(1)),
-                  tf2 = __shfl_sync(W.gm, tf, W.pos(2));
-      const float tface = fminf(fminf(tf0, tf1), tf2);
+      const R vel = __hiloint2double(__double2hiint(k1) ^ (int)((unit & 1) << 31), __double2loint(k1));
+      const R tf = plane_time(__double2hiint(vel) >= 0 ? r_hi : r_lo, vel, R(1e30));
+      const R tf0 = gsh(W.gm, tf, W.pos(0)), tf1 = gsh(W.gm, tf, W.pos(1)), tf2 = gsh(W.gm, tf, W.pos(2));
+      const R tface = min_bits(min_bits(tf0, tf1), tf2);
       {
         // ask L1 for the vertices of the cell beyond that plane
-        const int pa = tf0 <= tface ? 0 : (tf1 <= tface ? 1 : 2);
-        const float v0 = __shfl_sync(W.gm, vel, W.pos(pa));
-        const int d = v0 > 0.0f ? 1 : -1;
+        const int pa = !gt_bits(tf0, tface) ? 0 : (!gt_bits(tf1, tface) ? 1 : 2);
+        const int d = __shfl_sync(W.gm, __double2hiint(vel), W.pos(pa)) >= 0 ? 1 : -1;
         int q[3] = {ic[0], ic[1], ic[2]};
         if (pa == 0) q[0] = min(max(q[0] + d, 0), E->F.n[0] - 2);
         else if (pa == 1) q[1] = min(max(q[1] + d, 0), E->F.n[1] - 2);
@@ -2746,22 +2778,8 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
         prefetch_l1(E->F.v + ((size_t)(q[2] + ((l >> 2) & 1)) * n01 + (size_t)(q[1] + ((l >> 1) & 1)) * n0 +
                               (size_t)(q[0] + (l & 1))));
       }
-      float hsF = fminf(h, h_max);
-      R hs;
-      bool capped = false;
-      if ((float)room > 1.001f * hsF) {
-        hs = (R)hsF;
-      } else {  // near the maximum length: the cap in FP64
-        capped = room <= (R)hsF;
-        hs = capped ? room : (R)hsF;
-        hsF = (float)hs;
-      }
-      const float hf = 1.25f * fmaxf(tface, 0.0f) + tiny;
-      if (hf < hsF) {
-        hsF = hf;
-        hs = (R)hf;
-        capped = false;
-      }
+      bool capped;
+      const R hs = wide_step(h, h_max, room, tface, tiny, &capped);
       const R hh = sgn * hs;
       // stages on K_i = hh k_i
       const R K1 = hh * k1;
@@ -2778,28 +2796,25 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
       const R K7 = hh * k7;
       c_stage += lead ? 6 : 0;
       steps += 1;
-      float err;
+      R err;
       {
-        const float e = fabsf((float)fma(R(DE7), K7, fma(R(DE6), K6, fma(R(DE5), K5, fma(R(DE4), K4,
-                              fma(R(DE3), K3, R(DE1) * K1)))))) * hcf;
-        const float base = j == 0 ? fmaf((float)sel3(c, ic[0], ic[1], ic[2]), hcf, orgf) : 0.0f;
-        const float m = fmaxf(fabsf(fmaf((float)y, hcf, base)), fabsf(fmaf((float)t, hcf, base)));
-        err = __fdividef(e, fmaf(tolr, m, tola));
-        const int r0 = W.pos(c);
-        err = fmaxf(fmaxf(__shfl_sync(W.gm, err, r0), __shfl_sync(W.gm, err, r0 + 1)), __shfl_sync(W.gm, err, r0 + 2));
-        err = fmaxf(fmaxf(__shfl_sync(W.gm, err, W.pos(0)), __shfl_sync(W.gm, err, W.pos(1))),
-                    __shfl_sync(W.gm, err, W.pos(2)));
+        const R e = fabs(fma(R(DE7), K7, fma(R(DE6), K6, fma(R(DE5), K5, fma(R(DE4), K4, fma(R(DE3), K3, R(DE1) * K1)))))) * hhc;
+        const R base = j == 0 ? fma(R(sel3(c, ic[0], ic[1], ic[2])), hhc, orgc) : R(0);
+        const R size = max_bits(fabs(fma(y, hhc, base)), fabs(fma(t, hhc, base)));
+        err = j == 3 ? R(0) : err_ratio<true>(e, size, P.tol_abs, P.tol_rel);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) err = max_bits(err, __shfl_xor_sync(W.gm, err, o));
       }
+      const R hnext = next_step(hs, err);
       const bool bad = __any_sync(W.gm, (__double2hiint(t) & 0x7ff00000) == 0x7ff00000);
       if (bad) {
         status = QSL_LINE_NONFINITE;
-      } else if (err > 1.0f) {
+      } else if (gt_bits(err, R(1))) {
         c_rej += lead;
-        h = hsF * fmaxf(0.2f, 0.9f * __powf(err, -0.25f));
-        if (h < h_min) status = QSL_LINE_STALL;
+        h = hnext;
+        if (gt_bits(h_min, h)) status = QSL_LINE_STALL;
       } else {
         c_acc += lead;
-        const float hnext = hsF * ((err == 0.0f) ? 5.0f : fminf(5.0f, 0.9f * __powf(err, -0.2f)));
         const R c4 = fma(R(DD7), K7, fma(R(DD6), K6, fma(R(DD5), K5, fma(R(DD4), K4, fma(R(DD3), K3, R(DD1) * K1)))));
         const R bspl = K1 - dy;
         const R c3 = (dy - K7) - bspl;
@@ -2843,7 +2858,7 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
             lface = 2 * ax_c + up_c;
           } else {
             // enter the neighbouring cell
-            zc = ((float)dl < tiny) ? zc + 1 : 0;
+            zc = gt_bits(tiny, dl) ? zc + 1 : 0;
             const int na = sel3(ax_c, ic[0], ic[1], ic[2]) + (up_c ? 1 : -1);
             if (zc > 3 || na < 0 || na > sel3(ax_c, E->F.n[0], E->F.n[1], E->F.n[2]) - 2) {
               // grazing a face back and forth: stay in this cell for one step
@@ -2855,7 +2870,7 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
               if (j == 0 && c == ax_c) y = up_c ? R(0) : R(1);
               kvalid = false;
             }
-            h = fmaxf(hnext, hsF);
+            h = max_bits(hnext, hs);
           }
         }
       }
