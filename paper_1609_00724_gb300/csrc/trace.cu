@@ -476,7 +476,7 @@ struct Cont {
   int64_t unit;
   double h;
   int ic[3];
-  int zc;
+  int zc, kvalid, pad;
 };
 
 template <class R>
@@ -1107,6 +1107,47 @@ __device__ __forceinline__ double quot(double a, double b) {
   return fma(fma(-b, q, a), x, q);
 }
 
+// Arithmetic that cell_kernel_f64 (one lane per line) and cell_wide_kernel
+// (sixteen) share. A line passes from the one to the other when its warp runs
+// short of lines, which depends on the scheduling, so both form every result
+// with the same operations in the same order: a call's results are then a
+// function of its inputs, and the same for every number of lanes. Products that
+// could be contracted into a later sum are rounded by __dmul_rn.
+// The sums over the stage derivatives, to be scaled by the step.
+__device__ __forceinline__ double dp_s3(double k1, double k2) { return fma(DA32, k2, DA31 * k1); }
+__device__ __forceinline__ double dp_s4(double k1, double k2, double k3) { return fma(DA43, k3, fma(DA42, k2, DA41 * k1)); }
+__device__ __forceinline__ double dp_s5(double k1, double k2, double k3, double k4) {
+  return fma(DA54, k4, fma(DA53, k3, fma(DA52, k2, DA51 * k1)));
+}
+__device__ __forceinline__ double dp_s6(double k1, double k2, double k3, double k4, double k5) {
+  return fma(DA65, k5, fma(DA64, k4, fma(DA63, k3, fma(DA62, k2, DA61 * k1))));
+}
+__device__ __forceinline__ double dp_b(double k1, double k3, double k4, double k5, double k6) {
+  return fma(DB6, k6, fma(DB5, k5, fma(DB4, k4, fma(DB3, k3, DB1 * k1))));
+}
+__device__ __forceinline__ double dp_e(double k1, double k3, double k4, double k5, double k6, double k7) {
+  return fma(DE7, k7, fma(DE6, k6, fma(DE5, k5, fma(DE4, k4, fma(DE3, k3, DE1 * k1)))));
+}
+__device__ __forceinline__ double dp_d(double k1, double k3, double k4, double k5, double k6, double k7) {
+  return fma(DD7, k7, fma(DD6, k6, fma(DD5, k5, fma(DD4, k4, fma(DD3, k3, DD1 * k1)))));
+}
+// Continuous extension of a component over the step hh with the increment dy:
+// th (dy + (1 - th) (bspl + th (c3 + (1 - th) c4))), d the sum of dp_d.
+struct Dense {
+  double bspl, c3, c4;
+};
+__device__ __forceinline__ Dense dense_of(double hh, double k1, double k7, double d, double dy) {
+  Dense D;
+  D.c4 = __dmul_rn(hh, d);
+  D.bspl = fma(hh, k1, -dy);
+  D.c3 = fma(-hh, k7, dy) - D.bspl;
+  return D;
+}
+__device__ __forceinline__ double dense_at(double th, const Dense& D, double dy, double y) {
+  const double s1 = 1.0 - th;
+  return fma(th, fma(s1, fma(th, fma(s1, D.c4, D.c3), D.bspl), dy), y);
+}
+
 // The step of the FP64 cell-wise tracers: the controller's h, at most h_max and
 // the room left, or a little beyond the first plane along the derivative (tface
 // >= 0, the time to it) where that comes first. capped: it ends at the maximum
@@ -1308,13 +1349,26 @@ __device__ __forceinline__ void cell_rhs_poly(const typename C4<R>::type* __rest
           k[3 + 3 * v2 + i] = fma(d[i][0], y[3 + 3 * v2], fma(d[i][1], y[4 + 3 * v2], d[i][2] * y[5 + 3 * v2]));
     }
   } else {
-    const R rm = rcp_norm(val[0] * val[0] + val[1] * val[1] + val[2] * val[2]);
+    R rm;
+    if constexpr (sizeof(R) == 8) rm = rcp_norm(fma(val[0], val[0], fma(val[1], val[1], val[2] * val[2])));
+    else rm = rcp_norm(val[0] * val[0] + val[1] * val[1] + val[2] * val[2]);
     R b[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) b[c] = val[c] * rm;
 #pragma unroll
     for (int c = 0; c < 3; ++c) k[c] = b[c] * ih[c];
-    if (NC == 9) {
+    if constexpr (NC == 9 && sizeof(R) == 8) {  // wide_rhs's form
+#pragma unroll
+      for (int v2 = 0; v2 < 2; ++v2) {
+        R g[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+          g[i] = fma(d[i][0], y[3 + 3 * v2], fma(d[i][1], y[4 + 3 * v2], d[i][2] * y[5 + 3 * v2]));
+        const R bs = (__dmul_rn(b[0], g[0]) + __dmul_rn(b[1], g[1])) + __dmul_rn(b[2], g[2]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) k[3 + 3 * v2 + i] = (ih[i] * rm) * fma(-b[i], bs, g[i]);
+      }
+    } else if (NC == 9) {
       R g[3][3];
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
@@ -1524,6 +1578,7 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
             k.unit = unit;
             k.h = h;
             k.zc = zc;
+            k.kvalid = kvalid;
             active = false;
           }
         }
@@ -1630,41 +1685,62 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
         }
       }
       R hh = sgn * hs;
-      // stage combinations with the step folded into the coefficients; each
-      // stage's newest term is the last FMA
-      const R c21 = hh * R(DA21), c31 = hh * R(DA31), c32 = hh * R(DA32), c41 = hh * R(DA41), c42 = hh * R(DA42),
-              c43 = hh * R(DA43), c51 = hh * R(DA51), c52 = hh * R(DA52), c53 = hh * R(DA53), c54 = hh * R(DA54),
-              c61 = hh * R(DA61), c62 = hh * R(DA62), c63 = hh * R(DA63), c64 = hh * R(DA64), c65 = hh * R(DA65);
-      const R b1 = hh * R(DB1), b3 = hh * R(DB3), b4 = hh * R(DB4), b5 = hh * R(DB5), b6 = hh * R(DB6);
-      R k2[NC], k3[NC], k4[NC], k5[NC], k6[NC], k7[NC], t[NC];
+      R k2[NC], k3[NC], k4[NC], k5[NC], k6[NC], k7[NC], t[NC], dy[NC];
+      if constexpr (F64) {
 #pragma unroll
-      for (int i = 0; i < NC; ++i) t[i] = fma(c21, k1[i], y[i]);
-      cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k2);
+        for (int i = 0; i < NC; ++i) t[i] = fma(hh, R(DA21) * k1[i], y[i]);
+        cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k2);
 #pragma unroll
-      for (int i = 0; i < NC; ++i) t[i] = fma(c32, k2[i], fma(c31, k1[i], y[i]));
-      cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k3);
+        for (int i = 0; i < NC; ++i) t[i] = fma(hh, dp_s3(k1[i], k2[i]), y[i]);
+        cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k3);
 #pragma unroll
-      for (int i = 0; i < NC; ++i) t[i] = fma(c43, k3[i], fma(c42, k2[i], fma(c41, k1[i], y[i])));
-      cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k4);
+        for (int i = 0; i < NC; ++i) t[i] = fma(hh, dp_s4(k1[i], k2[i], k3[i]), y[i]);
+        cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k4);
 #pragma unroll
-      for (int i = 0; i < NC; ++i) t[i] = fma(c54, k4[i], fma(c53, k3[i], fma(c52, k2[i], fma(c51, k1[i], y[i]))));
-      cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k5);
+        for (int i = 0; i < NC; ++i) t[i] = fma(hh, dp_s5(k1[i], k2[i], k3[i], k4[i]), y[i]);
+        cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k5);
 #pragma unroll
-      for (int i = 0; i < NC; ++i)
-        t[i] = fma(c65, k5[i], fma(c64, k4[i], fma(c63, k3[i], fma(c62, k2[i], fma(c61, k1[i], y[i])))));
-      cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k6);
-      R dy[NC];
+        for (int i = 0; i < NC; ++i) t[i] = fma(hh, dp_s6(k1[i], k2[i], k3[i], k4[i], k5[i]), y[i]);
+        cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k6);
 #pragma unroll
-      for (int i = 0; i < NC; ++i) {
-        dy[i] = fma(b6, k6[i], fma(b5, k5[i], fma(b4, k4[i], fma(b3, k3[i], b1 * k1[i]))));
-        t[i] = y[i] + dy[i];
+        for (int i = 0; i < NC; ++i) {
+          dy[i] = __dmul_rn(hh, dp_b(k1[i], k3[i], k4[i], k5[i], k6[i]));
+          t[i] = y[i] + dy[i];
+        }
+        cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k7);
+      } else {
+        // stage combinations with the step folded into the coefficients; each
+        // stage's newest term is the last FMA
+        const R c21 = hh * R(DA21), c31 = hh * R(DA31), c32 = hh * R(DA32), c41 = hh * R(DA41), c42 = hh * R(DA42),
+                c43 = hh * R(DA43), c51 = hh * R(DA51), c52 = hh * R(DA52), c53 = hh * R(DA53), c54 = hh * R(DA54),
+                c61 = hh * R(DA61), c62 = hh * R(DA62), c63 = hh * R(DA63), c64 = hh * R(DA64), c65 = hh * R(DA65);
+        const R b1 = hh * R(DB1), b3 = hh * R(DB3), b4 = hh * R(DB4), b5 = hh * R(DB5), b6 = hh * R(DB6);
+#pragma unroll
+        for (int i = 0; i < NC; ++i) t[i] = fma(c21, k1[i], y[i]);
+        cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k2);
+#pragma unroll
+        for (int i = 0; i < NC; ++i) t[i] = fma(c32, k2[i], fma(c31, k1[i], y[i]));
+        cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k3);
+#pragma unroll
+        for (int i = 0; i < NC; ++i) t[i] = fma(c43, k3[i], fma(c42, k2[i], fma(c41, k1[i], y[i])));
+        cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k4);
+#pragma unroll
+        for (int i = 0; i < NC; ++i) t[i] = fma(c54, k4[i], fma(c53, k3[i], fma(c52, k2[i], fma(c51, k1[i], y[i]))));
+        cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k5);
+#pragma unroll
+        for (int i = 0; i < NC; ++i)
+          t[i] = fma(c65, k5[i], fma(c64, k4[i], fma(c63, k3[i], fma(c62, k2[i], fma(c61, k1[i], y[i])))));
+        cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k6);
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+          dy[i] = fma(b6, k6[i], fma(b5, k5[i], fma(b4, k4[i], fma(b3, k3[i], b1 * k1[i]))));
+          t[i] = y[i] + dy[i];
+        }
+        cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k7);
       }
-      cell_rhs_poly<R, NC>(cs, st, E->F.raw, ih, t, k7);
       c_stage += 6;
       steps += 1;
-      // the error estimate's and the continuous extension's weights, scaled by the step
-      const R e1 = hh * R(DE1), e3 = hh * R(DE3), e4 = hh * R(DE4), e5 = hh * R(DE5), e6 = hh * R(DE6),
-              e7 = hh * R(DE7);
+      // the continuous extension's weights (FP32), scaled by the step
       const R w1 = hh * R(DD1), w3 = hh * R(DD3), w4 = hh * R(DD4), w5 = hh * R(DD5), w6 = hh * R(DD6),
               w7 = hh * R(DD7);
       R err = 0;
@@ -1673,8 +1749,7 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
 #pragma unroll
         for (int i = 0; i < NC; ++i) {
           const R hc = hh3[i % 3];
-          const R e =
-              fabs(fma(e7, k7[i], fma(e6, k6[i], fma(e5, k5[i], fma(e4, k4[i], fma(e3, k3[i], e1 * k1[i])))))) * hc;
+          const R e = fabs(dp_e(k1[i], k3[i], k4[i], k5[i], k6[i], k7[i])) * (hs * hc);
           if ((__double2hiint(t[i]) & 0x7ff00000) == 0x7ff00000) finite = false;
           R size;
           if (i < 3) {
@@ -1686,6 +1761,8 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
           err = max_bits(err, err_ratio<false>(e, size, P.tol_abs, P.tol_rel));
         }
       } else {
+        const R e1 = hh * R(DE1), e3 = hh * R(DE3), e4 = hh * R(DE4), e5 = hh * R(DE5), e6 = hh * R(DE6),
+                e7 = hh * R(DE7);
 #pragma unroll
         for (int i = 0; i < NC; ++i) {
           R e = fabs(fma(e7, k7[i], fma(e6, k6[i], fma(e5, k5[i], fma(e4, k4[i], fma(e3, k3[i], e1 * k1[i]))))));
@@ -1753,14 +1830,16 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
           R sg = up ? R(1) : R(-1);  // sg * f > 0 beyond the plane
           R k1a = a == 0 ? k1[0] : (a == 1 ? k1[1] : k1[2]);
           R k7a = a == 0 ? k7[0] : (a == 1 ? k7[1] : k7[2]);
-          R c4 = fma(w7, k7a, fma(w6, sel3(a, k6[0], k6[1], k6[2]), fma(w5, sel3(a, k5[0], k5[1], k5[2]),
-                 fma(w4, sel3(a, k4[0], k4[1], k4[2]), fma(w3, sel3(a, k3[0], k3[1], k3[2]), w1 * k1a)))));
-          R bspl = hh * k1a - dya;
-          R c3 = dya - hh * k7a - bspl;
+          const R k3a = sel3(a, k3[0], k3[1], k3[2]), k4a = sel3(a, k4[0], k4[1], k4[2]),
+                  k5a = sel3(a, k5[0], k5[1], k5[2]), k6a = sel3(a, k6[0], k6[1], k6[2]);
           R t;
-          if constexpr (sizeof(R) == 8) {
-            t = cross_root(r, dya, bspl, c3, c4, up);
+          if constexpr (F64) {
+            const Dense D = dense_of(hh, k1a, k7a, dp_d(k1a, k3a, k4a, k5a, k6a, k7a), dya);
+            t = cross_root(r, dya, D.bspl, D.c3, D.c4, up);
           } else {
+            R c4 = fma(w7, k7a, fma(w6, k6a, fma(w5, k5a, fma(w4, k4a, fma(w3, k3a, w1 * k1a)))));
+            R bspl = hh * k1a - dya;
+            R c3 = dya - hh * k7a - bspl;
             // The offset along the axis is t * P(t) with the cubic
             // P(t) = dya + (1 - t) (bspl + t (c3 + (1 - t) c4)). A step that
             // starts on the plane (r = 0: a seed on a domain face, or the face
@@ -1822,28 +1901,24 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
         } else {
           // advance to the plane on the dense output and snap onto it
           if constexpr (F64) {
-            // y_at's increment as one sum over the stages (its weights formed
-            // once, 7 FP64 instructions per component against 17)
-            const R s1 = R(1) - th, st_ = s1 * th;
-            const R ad = th * fma(R(2), st_, th), d4 = th * (s1 * st_);
-            const R g1 = fma(d4, w1, hh * (th * (s1 * s1))), g7 = fma(d4, w7, -(hh * (th * st_)));
-            const R g3 = d4 * w3, g4 = d4 * w4, g5 = d4 * w5, g6 = d4 * w6;
 #pragma unroll
             for (int i = 0; i < NC; ++i)
-              y[i] = fma(ad, dy[i], fma(g7, k7[i], fma(g6, k6[i], fma(g5, k5[i], fma(g4, k4[i], fma(g3, k3[i],
-                     fma(g1, k1[i], y[i])))))));
+              y[i] = dense_at(th, dense_of(hh, k1[i], k7[i], dp_d(k1[i], k3[i], k4[i], k5[i], k6[i], k7[i]), dy[i]),
+                              dy[i], y[i]);
           } else {
 #pragma unroll
-          for (int i = 0; i < NC; ++i)
-            y[i] += y_at<R>(th, dy[i], hh * k1[i], hh * k7[i],
-                            fma(w7, k7[i], fma(w6, k6[i], fma(w5, k5[i], fma(w4, k4[i], fma(w3, k3[i], w1 * k1[i]))))));
+            for (int i = 0; i < NC; ++i)
+              y[i] += y_at<R>(th, dy[i], hh * k1[i], hh * k7[i],
+                              fma(w7, k7[i], fma(w6, k6[i], fma(w5, k5[i], fma(w4, k4[i], fma(w3, k3[i], w1 * k1[i]))))));
           }
           bool dom = up_c ? sel3(ax_c, hi_dom[0], hi_dom[1], hi_dom[2]) : sel3(ax_c, lo_dom[0], lo_dom[1], lo_dom[2]);
           R target = up_c ? sel3(ax_c, hi_pl[0], hi_pl[1], hi_pl[2]) : sel3(ax_c, lo_pl[0], lo_pl[1], lo_pl[2]);
           if (ax_c == 0) y[0] = target;
           else if (ax_c == 1) y[1] = target;
           else y[2] = target;
-          R dl = th * hs;
+          R dl;
+          if constexpr (F64) dl = __dmul_rn(th, hs);
+          else dl = th * hs;
           R t1 = dl - muc, t2 = mu + t1;
           muc = (t2 - mu) - t1;
           mu = t2;
@@ -1859,6 +1934,7 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
               // grazing a face back and forth: stay in this cell for one step
               // (the cell's polynomial continued across the face)
               zc = 0;
+              if constexpr (F64) kvalid = false;  // the derivative at the new point
             } else {
               if (ax_c == 0) ic[0] = na;
               else if (ax_c == 1) ic[1] = na;
@@ -2499,22 +2575,25 @@ __device__ __forceinline__ void write_stats(const TraceParams<R>& P, int lane, u
 __device__ __forceinline__ double gsh(unsigned gm, double v, int src) { return __shfl_sync(gm, v, src); }
 
 struct WideLane {
-  unsigned gm;       // the group's lanes
-  int gb;            // its first lane
-  int c, j;          // axis and role of the lane
-  int s_src, t_src;  // lanes holding the lane's two bilinear coordinates
-  int p1_src;        // lane of the second factor of the product sum
+  unsigned gm;            // the group's lanes
+  int gb;                 // its first lane
+  int c, j;               // axis and role of the lane
+  int s_src, t_src;       // lanes holding the lane's two bilinear coordinates
+  int p0_src, p1_src;     // lanes of the first two factors of the product sum
   __device__ __forceinline__ int pos(int a) const { return gb + 4 * a; }  // position lane of axis a
 };
 
 // Stage derivative of the lane's component at the stage state t (co: the
-// lane's bilinear coefficients).
+// lane's bilinear coefficients). CELL: cell_wide_kernel's roles, whose j = 3
+// holds the lower z face, so that a value is cell_rhs_poly's sum.
+template <bool CELL>
 __device__ __forceinline__ double wide_rhs(const WideLane& W, const double* co, bool raw, double ihc, double t) {
   const double s = gsh(W.gm, t, W.s_src), w = gsh(W.gm, t, W.t_src);
   double z0 = gsh(W.gm, t, W.pos(0) + W.j), z1 = gsh(W.gm, t, W.pos(1) + W.j), z2 = gsh(W.gm, t, W.pos(2) + W.j);
   const double q = fma(fma(co[3], s, co[2]), w, fma(co[1], s, co[0]));
-  const double p0 = gsh(W.gm, q, W.pos(W.c)), p1 = gsh(W.gm, q, W.p1_src), p2 = gsh(W.gm, q, W.pos(W.c) + 2);
-  if (W.j == 0) {  // value = u d0 + (value on the lower x face)
+  const double p0 = gsh(W.gm, q, W.p0_src), p1 = gsh(W.gm, q, W.p1_src), p2 = gsh(W.gm, q, W.pos(W.c) + 2);
+  if (W.j == 0) {  // value = (derivative along x or z) x coordinate + (value on the lower x or z face)
+    if (CELL) z0 = z2;
     z1 = 1.0;
     z2 = 0.0;
   }
@@ -2525,8 +2604,8 @@ __device__ __forceinline__ double wide_rhs(const WideLane& W, const double* co, 
   const double v0 = gsh(W.gm, val, W.pos(0)), v1 = gsh(W.gm, val, W.pos(1)), v2 = gsh(W.gm, val, W.pos(2));
   const double rm = rcp_norm(fma(v0, v0, fma(v1, v1, v2 * v2)));
   const double b = val * rm;
-  const double bg = b * g;
-  const double bs = gsh(W.gm, bg, W.pos(0) + W.j) + gsh(W.gm, bg, W.pos(1) + W.j) + gsh(W.gm, bg, W.pos(2) + W.j);
+  const double bg = __dmul_rn(b, g);
+  const double bs = (gsh(W.gm, bg, W.pos(0) + W.j) + gsh(W.gm, bg, W.pos(1) + W.j)) + gsh(W.gm, bg, W.pos(2) + W.j);
   return W.j == 0 ? b * ihc : (ihc * rm) * fma(-b, bs, g);
 }
 
@@ -2598,7 +2677,8 @@ __device__ __forceinline__ int wide_start(const Item<double>* E, const double* x
   return status;
 }
 
-// The lane roles of a 16-lane group.
+// The lane roles of a 16-lane group (CELL: see wide_rhs).
+template <bool CELL>
 __device__ __forceinline__ WideLane wide_lane(int lane) {
   const int l = lane & 15;
   WideLane W;
@@ -2606,8 +2686,9 @@ __device__ __forceinline__ WideLane wide_lane(int lane) {
   W.gm = 0xffffu << W.gb;
   W.c = min(l >> 2, 2);
   W.j = l & 3;
-  W.s_src = (W.j == 0 || W.j == 3) ? W.pos(1) : W.pos(0);
-  W.t_src = W.j == 2 ? W.pos(1) : W.pos(2);
+  W.s_src = (W.j == 0 || (!CELL && W.j == 3)) ? W.pos(1) : W.pos(0);
+  W.t_src = (W.j == 2 || (CELL && W.j == 3)) ? W.pos(1) : W.pos(2);
+  W.p0_src = W.pos(W.c) + (CELL && W.j == 0 ? 2 : 0);
   W.p1_src = W.pos(W.c) + (W.j == 0 ? 3 : 1);
   return W;
 }
@@ -2617,7 +2698,7 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int l = lane & 15;
-  const WideLane W = wide_lane(lane);
+  const WideLane W = wide_lane<true>(lane);
   const int c = W.c, j = W.j;
   const bool lead = l == 0, writer = l < 12 && j < 3;
   int64_t total = P.n_units;
@@ -2636,14 +2717,14 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
   const bool usable = total > warps_total || W.gb == 0;
   const Item<R>* E = &P.item0;
 
-  bool active = false, exhausted = false, kvalid = false;
+  bool active = false, exhausted = false, kvalid = false, counted = false;
   int64_t unit = 0;
   R y = 0, k1 = 0, co[4] = {0, 0, 0, 0};
   R lo_pl = 0, hi_pl = 0, ihc = 1, hhc = 1;
   bool lo_dom = false, hi_dom = false, raw = false;
   int ic[3] = {0, 0, 0};
   R mu = 0, muc = 0, sgn = 1, max_len = 0;
-  R h = 0, h_max = 0, h_min = 0, tiny = 0, orgc = 0;
+  R h = 0, h_max = 0, h_min = 0, tiny = 0, orgc = 0, base = 0;
   int ilo = 0, ihi = 0;
   int steps = 0, zc = 0;
   unsigned long long c_stage = 0, c_acc = 0, c_rej = 0, c_land = 0, c_lines = 0;
@@ -2685,7 +2766,7 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
             tiny = R(1e-4) * h_max;
             ilo = (int)floor(sel3(c, E->lo[0], E->lo[1], E->lo[2]));
             ihi = (int)ceil(sel3(c, E->hi[0], E->hi[1], E->hi[2])) - 1;
-            kvalid = false;
+            kvalid = counted = false;
             if (k) {
               // a line that cell_kernel_f64 handed over: its state from the
               // continuation and end records
@@ -2695,6 +2776,7 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
               muc = k->muc;
               steps = e.steps;
               zc = k->zc;
+              counted = k->kvalid != 0;
               h = k->h;
 #pragma unroll
               for (int a = 0; a < 3; ++a) ic[a] = k->ic[a];
@@ -2732,16 +2814,16 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
     if (status == ST_RUNNING && !gt_bits(room, 0.0)) status = QSL_LINE_MAXLEN;
     if (status == ST_RUNNING) {
       if (!kvalid) {
-        // the lane's bilinear coefficients from the 8 corners of component c:
-        // differences along the lane's own axis (j = 3: the lower x face)
+        // the lane's four of the eight polynomial coefficients of component c
+        // (trilinear_coeffs): those with u for j = 0, with v, with w, and the
+        // lower z face for j = 3
         const size_t sy = 4 * (size_t)E->F.n[0], sz = sy * (size_t)E->F.n[1];
         const R* p = reinterpret_cast<const R*>(E->F.v) + (size_t)ic[2] * sz + (size_t)ic[1] * sy +
                      4 * (size_t)ic[0] + c;
-        const size_t oj = j == 1 ? sy : (j == 2 ? sz : 4);
-        const size_t os = (j == 0 || j == 3) ? sy : 4, ot = j == 2 ? sy : sz;
-        const R l00 = __ldg(p), l10 = __ldg(p + os), l01 = __ldg(p + ot), l11 = __ldg(p + os + ot);
-        const R h00 = __ldg(p + oj), h10 = __ldg(p + oj + os), h01 = __ldg(p + oj + ot), h11 = __ldg(p + oj + os + ot);
+        const R v0 = __ldg(p), v1 = __ldg(p + 4), v2 = __ldg(p + sy), v3 = __ldg(p + sy + 4);
+        const R v4 = __ldg(p + sz), v5 = __ldg(p + sz + 4), v6 = __ldg(p + sz + sy), v7 = __ldg(p + sz + sy + 4);
         const int icc = sel3(c, ic[0], ic[1], ic[2]);
+        base = j == 0 ? fma(R(icc), hhc, orgc) : R(0);
         lo_dom = icc <= ilo;
         hi_dom = icc >= ihi;
         lo_pl = R(0);
@@ -2750,14 +2832,18 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
         if (hi_dom) hi_pl = sel3(c, E->hi[0], E->hi[1], E->hi[2]) - R(icc);
         const R sc = raw ? R(1) : ihc;
         const bool low = j == 3;
-        const R d00 = (low ? l00 : h00 - l00) * sc, d10 = (low ? l10 : h10 - l10) * sc;
-        const R d01 = (low ? l01 : h01 - l01) * sc, d11 = (low ? l11 : h11 - l11) * sc;
-        co[0] = d00;
-        co[1] = d10 - d00;
-        co[2] = d01 - d00;
-        co[3] = (d11 - d10) - (d01 - d00);
-        k1 = wide_rhs(W, co, raw, ihc, y);
-        c_stage += lead;
+        const R d0 = (j == 0 ? v1 : (j == 1 ? v2 : v4)) - v0;
+        const R d1 = (j == 2 ? v5 : (low ? v1 : v3)) - (low ? v0 : v1), e1 = (j == 2 ? v4 : v2) - v0;
+        const R d2 = (j == 0 ? v5 : (low ? v2 : v6)) - (j == 0 ? v1 : (low ? v0 : v2)), e2 = v4 - v0;
+        const R d3 = ((low ? v3 : v7) - (low ? v1 : v6)) - ((low ? v2 : v5) - (low ? v0 : v4)),
+                e3 = (v3 - v2) - (v1 - v0);
+        co[0] = (low ? v0 : d0) * sc;
+        co[1] = (low ? d1 : d1 - e1) * sc;
+        co[2] = (low ? d2 : d2 - e2) * sc;
+        co[3] = (low ? d3 : d3 - e3) * sc;
+        k1 = wide_rhs<true>(W, co, raw, ihc, y);
+        c_stage += lead && !counted;
+        counted = false;
         kvalid = true;
       }
       // step: controller size, capped a little beyond the first plane along k1
@@ -2781,25 +2867,19 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
       bool capped;
       const R hs = wide_step(h, h_max, room, tface, tiny, &capped);
       const R hh = sgn * hs;
-      // stages on K_i = hh k_i
-      const R K1 = hh * k1;
-      const R K2 = hh * wide_rhs(W, co, raw, ihc, fma(R(DA21), K1, y));
-      const R K3 = hh * wide_rhs(W, co, raw, ihc, fma(R(DA32), K2, fma(R(DA31), K1, y)));
-      const R K4 = hh * wide_rhs(W, co, raw, ihc, fma(R(DA43), K3, fma(R(DA42), K2, fma(R(DA41), K1, y))));
-      const R K5 = hh * wide_rhs(W, co, raw, ihc,
-                                 fma(R(DA54), K4, fma(R(DA53), K3, fma(R(DA52), K2, fma(R(DA51), K1, y)))));
-      const R K6 = hh * wide_rhs(W, co, raw, ihc,
-                                 fma(R(DA65), K5, fma(R(DA64), K4, fma(R(DA63), K3, fma(R(DA62), K2, fma(R(DA61), K1, y))))));
-      const R dy = fma(R(DB6), K6, fma(R(DB5), K5, fma(R(DB4), K4, fma(R(DB3), K3, R(DB1) * K1))));
+      const R k2 = wide_rhs<true>(W, co, raw, ihc, fma(hh, R(DA21) * k1, y));
+      const R k3 = wide_rhs<true>(W, co, raw, ihc, fma(hh, dp_s3(k1, k2), y));
+      const R k4 = wide_rhs<true>(W, co, raw, ihc, fma(hh, dp_s4(k1, k2, k3), y));
+      const R k5 = wide_rhs<true>(W, co, raw, ihc, fma(hh, dp_s5(k1, k2, k3, k4), y));
+      const R k6 = wide_rhs<true>(W, co, raw, ihc, fma(hh, dp_s6(k1, k2, k3, k4, k5), y));
+      const R dy = __dmul_rn(hh, dp_b(k1, k3, k4, k5, k6));
       const R t = y + dy;
-      const R k7 = wide_rhs(W, co, raw, ihc, t);
-      const R K7 = hh * k7;
+      const R k7 = wide_rhs<true>(W, co, raw, ihc, t);
       c_stage += lead ? 6 : 0;
       steps += 1;
       R err;
       {
-        const R e = fabs(fma(R(DE7), K7, fma(R(DE6), K6, fma(R(DE5), K5, fma(R(DE4), K4, fma(R(DE3), K3, R(DE1) * K1)))))) * hhc;
-        const R base = j == 0 ? fma(R(sel3(c, ic[0], ic[1], ic[2])), hhc, orgc) : R(0);
+        const R e = fabs(dp_e(k1, k3, k4, k5, k6, k7)) * (hs * hhc);
         const R size = max_bits(fabs(fma(y, hhc, base)), fabs(fma(t, hhc, base)));
         err = j == 3 ? R(0) : err_ratio<true>(e, size, P.tol_abs, P.tol_rel);
 #pragma unroll
@@ -2815,21 +2895,23 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
         if (gt_bits(h_min, h)) status = QSL_LINE_STALL;
       } else {
         c_acc += lead;
-        const R c4 = fma(R(DD7), K7, fma(R(DD6), K6, fma(R(DD5), K5, fma(R(DD4), K4, fma(R(DD3), K3, R(DD1) * K1)))));
-        const R bspl = K1 - dy;
-        const R c3 = (dy - K7) - bspl;
         // the plane of the lane's axis that the step ends beyond (at most one)
         const R band = R(16) * eps_of<R>();
         const bool o_lo = gt_bits(r_lo - dy, lo_dom ? R(0) : band), o_hi = gt_bits(dy - r_hi, hi_dom ? R(0) : band);
-        R thc = R(2);
-        if (j == 0 && (o_lo || o_hi)) thc = cross_root(o_lo ? r_lo : r_hi, dy, bspl, c3, c4, o_lo ? 0 : 1);
-        // earliest crossing over the axes; ties go to the lower plane id
-        const R q0 = gsh(W.gm, thc, W.pos(0)), q1 = gsh(W.gm, thc, W.pos(1)), q2 = gsh(W.gm, thc, W.pos(2));
+        const bool out = j == 0 && (o_lo || o_hi);
         R th = R(2);
+        Dense D{};
         int ax_c = -1;
-        if (gt_bits(th, q0)) { th = q0; ax_c = 0; }
-        if (gt_bits(th, q1)) { th = q1; ax_c = 1; }
-        if (gt_bits(th, q2)) { th = q2; ax_c = 2; }
+        if (__any_sync(W.gm, out)) {
+          D = dense_of(hh, k1, k7, dp_d(k1, k3, k4, k5, k6, k7), dy);
+          R thc = R(2);
+          if (out) thc = cross_root(o_lo ? r_lo : r_hi, dy, D.bspl, D.c3, D.c4, o_lo ? 0 : 1);
+          // earliest crossing over the axes; ties go to the lower plane id
+          const R q0 = gsh(W.gm, thc, W.pos(0)), q1 = gsh(W.gm, thc, W.pos(1)), q2 = gsh(W.gm, thc, W.pos(2));
+          if (gt_bits(th, q0)) { th = q0; ax_c = 0; }
+          if (gt_bits(th, q1)) { th = q1; ax_c = 1; }
+          if (gt_bits(th, q2)) { th = q2; ax_c = 2; }
+        }
         if (ax_c < 0) {
           // the step stays in the cell: accept it; k7 is the next k1
           y = t;
@@ -2842,13 +2924,12 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
           if (capped) status = QSL_LINE_MAXLEN;
         } else {
           // advance to the plane on the dense output and snap onto it
-          const R s1 = R(1) - th;
-          y += th * fma(s1, fma(th, fma(s1, c4, c3), bspl), dy);
+          y = dense_at(th, D, dy, y);
           const int flags = (o_lo ? 0 : 1) | ((o_lo ? lo_dom : hi_dom) ? 2 : 0);
           const int fl = __shfl_sync(W.gm, flags, W.pos(ax_c));
           const int up_c = fl & 1;
           if (j == 0 && c == ax_c) y = up_c ? hi_pl : lo_pl;
-          const R dl = th * hs;
+          const R dl = __dmul_rn(th, hs);
           R t1 = dl - muc, t2 = mu + t1;
           muc = (t2 - mu) - t1;
           mu = t2;
@@ -2863,6 +2944,7 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
             if (zc > 3 || na < 0 || na > sel3(ax_c, E->F.n[0], E->F.n[1], E->F.n[2]) - 2) {
               // grazing a face back and forth: stay in this cell for one step
               zc = 0;
+              kvalid = false;
             } else {
               if (ax_c == 0) ic[0] = na;
               else if (ax_c == 1) ic[1] = na;
@@ -2951,7 +3033,7 @@ __device__ __forceinline__ double ck_wide_rhs(const WideLane& W, const FieldView
     C.co[2] = d01 - d00;
     C.co[3] = (d11 - d10) - C.co[2];
   }
-  const double k = wide_rhs(W, C.co, raw, ihc, t);
+  const double k = wide_rhs<false>(W, C.co, raw, ihc, t);
   return raw ? k : k * ihc;
 }
 
@@ -2967,7 +3049,7 @@ __global__ void __launch_bounds__(256) ck_wide_kernel(const __grid_constant__ Tr
   typedef double R;
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, l = lane & 15;
-  const WideLane W = wide_lane(lane);
+  const WideLane W = wide_lane<false>(lane);
   const int c = W.c, j = W.j;
   const bool lead = l == 0, writer = l < 12 && j < 3;
   int64_t total = P.n_units;
