@@ -362,6 +362,17 @@ int qsl_cnn_loss_grad(qsl_cnn* cnn, const float* x, const float* y, int n, int h
 /* One Adam update (bias-corrected) of the FP32 master from `grad`; refreshes
  * the BF16 weights. */
 int qsl_cnn_adam_step(qsl_cnn* cnn, const float* grad, float lr, float beta1, float beta2, float eps, void* stream);
+/* Every wait of the passes' kernels on the tensor core is bounded (a second).
+ * One that runs out leaves NaN in the outputs that depend on it: in prob where
+ * the rest of a tile is missing, in the gradients of the layers concerned. This
+ * check runs a forward and a loss/gradient pass (pos_weight 1) in which the waits
+ * of the kernels in the set `kernels` run out at once. */
+#define QSL_CNN_FORWARD 1 /* the forward pass                          */
+#define QSL_CNN_DGRAD 2   /* the data gradients                        */
+#define QSL_CNN_WGRAD2 4  /* layer 2's weight and bias gradients       */
+#define QSL_CNN_WGRAD13 8 /* layers 1 and 3's weight, 1's bias gradients */
+int qsl_check_cnn_waits(qsl_cnn* cnn, const float* x, const float* y, int n, int h, int w, float* prob, float* loss,
+                        float* grad, int kernels, void* stream);
 void qsl_cnn_free(qsl_cnn* cnn);
 int qsl_cnn_nparams(void);
 /* Network input (device, NCHW X[nz][2][ny][nx]) of the nz z-slices of a

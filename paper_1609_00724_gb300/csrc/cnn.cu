@@ -48,7 +48,7 @@ struct alignas(16) TileSmem {
   float w3[9 * 32];                         // [tap][channel]
   uint32_t tmem;
   int failed;
-  uint64_t bar[3];
+  uint64_t bar[3], drained;
 };
 static_assert(sizeof(TileSmem) <= 113 * 1024, "two blocks per SM");
 
@@ -116,10 +116,10 @@ __device__ __forceinline__ void conv32_issue(TileSmem& S, uint32_t tmem, int t) 
 
 // Waits for the MMA tile of the warp's row (warp / 4) and reads its sums; the
 // first four warps then let tile 2 be issued into the columns they have read.
-__device__ __forceinline__ bool conv32_read(TileSmem& S, uint32_t tmem, int warp, uint32_t phase, float* v) {
+__device__ __forceinline__ bool conv32_read(TileSmem& S, uint32_t tmem, int warp, uint32_t phase, uint32_t wait_ns, float* v) {
   const int t = warp >> 2;
   const uint32_t tq = tmem + ((uint32_t)(warp & 3) << 21) + (t & 1) * 128;
-  const bool ok = umma::bar_wait(&S.bar[t], phase);
+  const bool ok = umma::bar_wait(&S.bar[t], phase, wait_ns);
   umma::fence_after();
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -135,7 +135,7 @@ __device__ __forceinline__ bool conv32_read(TileSmem& S, uint32_t tmem, int warp
   if (t == 0) {
     umma::fence_before();
     asm volatile("bar.sync 1, 128;" ::: "memory");
-    if (warp == 0 && umma::elect()) {
+    if (warp == 0 && ok && umma::elect()) {
       umma::fence_after();
       conv32_issue(S, tmem, 2);
     }
@@ -175,6 +175,7 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
 struct TileGrid {
   int n, H, W, tx, ty;  // images, tiles along x and y
   int64_t tiles;
+  uint32_t wait_ns;     // limit of a wait
 };
 __device__ __forceinline__ void tile_of(const TileGrid& G, int64_t t, int w, int h, int* n, int* oy, int* ox) {
   *ox = (int)(t % G.tx) * w;
@@ -227,13 +228,14 @@ struct alignas(16) FwdSmem {
   float z[2][3][SPAD];                      // layer 3's sums over the rows, per tap column
   uint32_t tmem;
   // layer 1's sums ready [2], input row written, planes written [2], layer 2's sums ready [2] and read [2]
-  uint64_t l1[2], xw, aw[2], l2[2], rd[2];
+  uint64_t l1[2], xw, aw[2], l2[2], rd[2], drained;
 };
 static_assert(sizeof(FwdSmem) <= 113 * 1024, "two blocks per SM");
 
 struct FwdGrid {
   int H, W, P, nseg, zw, h, tx, ty;  // segment columns, segments per row step, output columns and rows of a task, tasks along x, y
   int64_t tasks, groups;             // groups of nseg tasks
+  uint32_t wait_ns;                  // limit of a wait
 };
 
 __global__ void __launch_bounds__(FWD_THREADS, 2)
@@ -263,6 +265,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
       umma::bar_init(&S.rd[i], 4);
     }
     umma::bar_init(&S.xw, 4);
+    umma::bar_init(&S.drained);
     umma::bar_init_fence();
   }
   if (warp == 0) umma::tmem_alloc(&S.tmem, 256);
@@ -315,7 +318,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
 #pragma unroll 1
       for (int r = 0; r < rows; ++r, ++g) {
         const int b = g & 1;
-        ok = ok && umma::bar_wait(&S.l1[b], g >> 1 & 1);
+        ok = ok && umma::bar_wait(&S.l1[b], g >> 1 & 1, G.wait_ns);
         umma::fence_after();
         if (r + 1 < rows) {  // the slot of row r is free
           put(r + 3, r + 4);
@@ -332,7 +335,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
 #pragma unroll
           for (int c = 0; c < 16; ++c) v[c] = in ? fmaxf(v[c], 0.0f) : 0.0f;
           // the planes are free once the MMAs of two rows ago are done
-          if (h == 0 && g >= 2) ok = ok && umma::bar_wait(&S.l2[b], (g >> 1) - 1 & 1);
+          if (h == 0 && g >= 2) ok = ok && umma::bar_wait(&S.l2[b], (g >> 1) - 1 & 1, G.wait_ns);
           store_half<ROW>(S.a[b], p, h, v);
         }
         umma::fence_smem();
@@ -360,7 +363,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
 #pragma unroll 1
       for (int r = 0; r < rows; ++r, ++g) {
         const int b = g & 1;
-        ok = ok && umma::bar_wait(&S.l2[b], g >> 1 & 1);
+        ok = ok && umma::bar_wait(&S.l2[b], g >> 1 & 1, G.wait_ns);
         umma::fence_after();
         // layer 2's row that this row completes
         const int gy = y0 - 3 + r, gx = ox - 1 + lc;
@@ -398,7 +401,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
         // layer 3's row that this row completes
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          S.z[b][k][p] = za[k] + (dot[6 + k].x + dot[6 + k].y);
+          // a wait that ran out leaves the outputs marked as missing, the neighbours' too
+          S.z[b][k][p] = ok ? za[k] + (dot[6 + k].x + dot[6 + k].y) : __int_as_float(0x7fc00000);
           za[k] = zb[k] + (dot[3 + k].x + dot[3 + k].y);
           zb[k] = dot[k].x + dot[k].y;
         }
@@ -406,8 +410,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
         const int zy = y0 + r - 4, zx = ox + lc;
         if (live && r >= 4 && zy < G.H && lc < G.zw && zx < G.W) {
           const float z = S.b3 + ((S.z[b][0][p] + S.z[b][1][p + 1]) + S.z[b][2][p + 2]);
-          // a wait that ran out leaves the output marked as missing
-          out[n * plane + (size_t)zy * G.W + zx] = !ok ? __int_as_float(0x7fc00000) : 1.0f / (1.0f + expf(-z));
+          out[n * plane + (size_t)zy * G.W + zx] = 1.0f / (1.0f + expf(-z));
         }
       }
     }
@@ -417,7 +420,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
     uint32_t xn = 0;
     // layer 1's row r of the task, row number gl of the block
     auto layer1 = [&](int r, uint32_t gl) {
-      ok = ok && umma::bar_wait(&S.xw, xn & 1);
+      ok = ok && umma::bar_wait(&S.xw, xn & 1, G.wait_ns);
       ++xn;
       umma::fence_after();
       if (ok && umma::elect()) {
@@ -438,8 +441,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
       for (int r = 0; r < rows; ++r, ++g) {
         if (r + 1 < rows) layer1(r + 1, g + 1);
         const int b = g & 1;
-        ok = ok && umma::bar_wait(&S.aw[b], g >> 1 & 1);
-        if (g >= 2) ok = ok && umma::bar_wait(&S.rd[b], (g >> 1) - 1 & 1);
+        ok = ok && umma::bar_wait(&S.aw[b], g >> 1 & 1, G.wait_ns);
+        if (g >= 2) ok = ok && umma::bar_wait(&S.rd[b], (g >> 1) - 1 & 1, G.wait_ns);
         umma::fence_after();
         if (ok && umma::elect()) {
           const uint64_t a = umma::desc_k(umma::smem_addr(S.a[b]), ROW);
@@ -457,6 +460,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
         __syncwarp();
       }
     }
+    umma::drain(&S.drained);  // another warp may have given up on the last ones
   }
   umma::fence_before();
   __syncthreads();
@@ -552,6 +556,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
   if (tid == 0) {
     S.failed = 0;
     for (int i = 0; i < 3; ++i) umma::bar_init(&S.bar[i]);
+    umma::bar_init(&S.drained);
     umma::bar_init_fence();
   }
   if (warp == 0) umma::tmem_alloc(&S.tmem, 256);
@@ -609,7 +614,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
     const int gy = oy + warp, gx = ox + lane;
     const bool in = lane < DW && gy < G.H && gx < G.W;
     float v[32];
-    bool ok = conv32_read(S, tmem, warp, phase, v);
+    bool ok = conv32_read(S, tmem, warp, phase, G.wait_ns, v);
     if (in) {
       const size_t o = (size_t)n * 32 * plane + (size_t)gy * G.W + gx;
 #pragma unroll
@@ -622,7 +627,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
           d1[o + (h + c) * plane] = !ok ? __int_as_float(0x7fc00000) : m[c] > 0.0f ? v[h + c] : 0.0f;
       }
     }
-    for (int t = 0; t < M2 / 128; ++t) ok = ok && umma::bar_wait(&S.bar[t], phase);
+    for (int t = 0; t < M2 / 128; ++t) ok = ok && umma::bar_wait(&S.bar[t], phase, G.wait_ns);
     if (!ok) S.failed = 1;
     umma::fence_before();
     __syncthreads();
@@ -630,6 +635,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
     if (S.failed) break;
   }
   __syncthreads();
+  if (warp == 0 && S.failed) umma::drain(&S.drained);
   if (warp == 0) umma::tmem_free(tmem, 256);
 }
 
@@ -643,7 +649,8 @@ constexpr int WG_THREADS = 512;
 constexpr int WG_K = 256;                   // pixels of a tile, at most
 struct WgradGrid {
   int n, H, W, sw, tr, tx, ty;
-  uint32_t inv;  // 2^16 / (sw + 2), rounded up
+  uint32_t inv;      // 2^16 / (sw + 2), rounded up
+  uint32_t wait_ns;  // limit of a wait
   int64_t tiles;
 };
 constexpr int WG_X = 392;                   // input pixels of a tile: 256 + 2 * pitch + 3 at most, pitch <= 64
@@ -686,7 +693,7 @@ struct alignas(16) WgradSmem {
   unsigned char x[XP * WG_X * 16];          // layer 2: 12 planes of X, ones, zeros; layers 1, 3: one chunk
   uint32_t tmem;
   int failed;
-  uint64_t full[2], empty[2];
+  uint64_t full[2], empty[2], drained;
 };
 static_assert(sizeof(WgradSmem<14>) <= 227 * 1024 && sizeof(WgradSmem<1>) <= 227 * 1024, "one block per SM");
 
@@ -717,6 +724,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
       umma::bar_init(&S.full[i]);
       umma::bar_init(&S.empty[i], 12);
     }
+    umma::bar_init(&S.drained);
     umma::bar_init_fence();
   }
   if (warp == 0) umma::tmem_alloc(&S.tmem, 512);
@@ -750,9 +758,9 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
 #pragma unroll 1
         for (int ch = 0; ch < chains; ++ch, ++stage) {
           // both buffers start empty
-          if (stage >= 2) ok = umma::bar_wait(&S.empty[stage & 1], (stage >> 1) - 1 & 1) && ok;
+          if (stage >= 2) ok = ok && umma::bar_wait(&S.empty[stage & 1], (stage >> 1) - 1 & 1, G.wait_ns);
           umma::fence_after();
-          if (umma::elect()) {
+          if (ok && umma::elect()) {
             const int k0 = ch * kstep, k1 = min(klen, k0 + kstep);
 #pragma unroll 1
             for (int tap = 2 * g; tap < 2 * g + 2 && tap < 9; ++tap) {
@@ -766,13 +774,13 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
           __syncwarp();
         }
       // the tile's planes are free once its last MMA is done
-      ok = umma::bar_wait(&S.full[(stage - 1) & 1], (stage - 1) >> 1 & 1) && ok;
+      ok = ok && umma::bar_wait(&S.full[(stage - 1) & 1], (stage - 1) >> 1 & 1, G.wait_ns);
     } else if (piece < 3) {
 #pragma unroll
       for (int g = 0; g < 5; ++g)
 #pragma unroll 1
         for (int ch = 0; ch < chains; ++ch, ++stage) {
-          ok = umma::bar_wait(&S.full[stage & 1], stage >> 1 & 1) && ok;
+          ok = ok && umma::bar_wait(&S.full[stage & 1], stage >> 1 & 1, G.wait_ns);
           umma::fence_after();
           const uint32_t col = tq + (stage & 1) * 256 + i0;
           // row 32 piece + o, column 32 piece' + i
@@ -792,14 +800,15 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
             bias += v[0];
           }
           umma::fence_before();
-          if (lane == 0) umma::bar_arrive(&S.empty[stage & 1]);
           __syncwarp();
+          if (lane == 0 && ok) umma::bar_arrive(&S.empty[stage & 1]);
         }
     }
     if (!ok) S.failed = 1;
     __syncthreads();
     if (S.failed) break;
   }
+  if (S.failed && warp == 3) umma::drain(&S.drained);
   // the pieces of D are added in shared memory, in turn, then once per block in global memory
   float* sum = reinterpret_cast<float*>(S.x);
   const float bad = S.failed ? __int_as_float(0x7fc00000) : 0.0f;
@@ -849,6 +858,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
   if (tid == 0) {
     S.failed = 0;
     umma::bar_init(&S.full[0]);
+    umma::bar_init(&S.drained);
     umma::bar_init_fence();
   }
   if (warp == 0) umma::tmem_alloc(&S.tmem, 512);
@@ -923,7 +933,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     }
     __syncwarp();
     fetch(tile + gridDim.x);
-    if (!umma::bar_wait(&S.full[0], phase)) S.failed = 1;
+    if (!umma::bar_wait(&S.full[0], phase, G.wait_ns)) S.failed = 1;
     umma::fence_after();
     if (piece < 3) {
 #pragma unroll
@@ -944,6 +954,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     umma::fence_after();
     if (S.failed) break;
   }
+  if (S.failed && warp == 3) umma::drain(&S.drained);
   // sums over the pieces of X, then over those of D in shared memory, then one atomic per block
   float* sum = reinterpret_cast<float*>(S.d);  // [32][19]: 18 weights and the bias of a channel
   const float bad = S.failed ? __int_as_float(0x7fc00000) : 0.0f;
@@ -1046,8 +1057,9 @@ int launch_tiles(K kern, int threads, size_t smem, int per_sm, int gy, int64_t t
   return QSL_OK;
 }
 
-TileGrid tile_grid(int n, int H, int W, int w, int h) {
+TileGrid tile_grid(int n, int H, int W, int w, int h, uint32_t wait_ns) {
   TileGrid G;
+  G.wait_ns = wait_ns;
   G.n = n;
   G.H = H;
   G.W = W;
@@ -1072,8 +1084,9 @@ int launch_conv(const float* x, const __nv_bfloat16* w, const float* b, float* y
 // Segment width (the one that wastes least of a row), equal output columns per
 // task, and the rows per task that let the blocks, two per SM, finish soonest
 // (a task computes four rows more than it yields).
-FwdGrid fwd_grid(int n, int H, int W, int slots) {
+FwdGrid fwd_grid(int n, int H, int W, int slots, uint32_t wait_ns) {
   FwdGrid G;
+  G.wait_ns = wait_ns;
   G.H = H;
   G.W = W;
   int64_t best = INT64_MAX;
@@ -1103,8 +1116,9 @@ FwdGrid fwd_grid(int n, int H, int W, int slots) {
 }
 
 // Strips of equal width, at most 62 columns, and as many rows as 256 pixels hold.
-WgradGrid wgrad_grid(int n, int H, int W) {
+WgradGrid wgrad_grid(int n, int H, int W, uint32_t wait_ns) {
   WgradGrid G;
+  G.wait_ns = wait_ns;
   G.n = n;
   G.H = H;
   G.W = W;
@@ -1220,6 +1234,52 @@ __global__ void dilate_kernel(const uint8_t* __restrict__ in, int nz, int ny, in
   }
 }
 
+// Limit of a kernel's waits: WAIT_NS, or none at all for a kernel of the set
+// `kernels` (qsl_check_cnn_waits; 0 in the passes).
+uint32_t wait_of(int kernels, int kernel) { return kernels & kernel ? 0 : umma::WAIT_NS; }
+
+int forward_pass(qsl_cnn* c, const float* x, int n, int H, int W, float* prob, int kernels, cudaStream_t s) {
+  int dev = 0, sms = 0;
+  QSL_CHECK_CUDA(cudaGetDevice(&dev));
+  QSL_CHECK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const FwdGrid G = fwd_grid(n, H, W, 2 * sms, wait_of(kernels, QSL_CNN_FORWARD));
+  // setmaxnreg.inc waits for registers of the launch: 128 x 72 + 128 x 120 + 32 x n <= 288 x n
+  cudaFuncAttributes at;
+  QSL_CHECK_CUDA(cudaFuncGetAttributes(&at, forward_kernel));
+  if (at.numRegs < 96) {
+    qsl::set_error("the forward kernel was built with %d registers, its split needs 96", at.numRegs);
+    return QSL_ECUDA;
+  }
+  return launch_tiles(forward_kernel, FWD_THREADS, sizeof(FwdSmem), 2, 1, G.groups, s, x, c->wb, c->w, prob, G);
+}
+
+int loss_grad_pass(qsl_cnn* c, const float* x, const float* y, int n, int H, int W, float pos_weight, float* loss,
+                   float* grad, int kernels, cudaStream_t s) {
+  size_t P = (size_t)n * H * W;
+  int rc = ensure_act(c, P, s);
+  if (rc) return rc;
+  float *a1 = c->act, *a2 = a1 + P * 32, *d2 = a2 + P * 32, *d1 = d2 + P * 32, *z = d1 + P * 32, *dz = z + P;
+  QSL_CHECK_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), s));
+  QSL_CHECK_CUDA(cudaMemsetAsync(grad, 0, NPAR * sizeof(float), s));
+  const TileGrid GD = tile_grid(n, H, W, DW, DH, wait_of(kernels, QSL_CNN_DGRAD));
+  if ((rc = launch_conv<C1, C2, true>(x, c->wb + OFF_W1, c->w + OFF_B1, a1, n, H, W, s))) return rc;
+  if ((rc = launch_conv<C2, C2, true>(a1, c->wb + OFF_W2, c->w + OFF_B2, a2, n, H, W, s))) return rc;
+  if ((rc = launch_conv<C2, 1, false>(a2, c->wb + OFF_W3, c->w + OFF_B3, z, n, H, W, s)))
+    return rc;
+  bce_kernel<<<(int)std::min<size_t>((P + BCE_THREADS - 1) / BCE_THREADS, 1024), BCE_THREADS, 0, s>>>(z, y, (int64_t)P, pos_weight, dz, loss,
+                                                                          grad + OFF_B3);
+  qsl::count_launch();
+  QSL_CHECK_CUDA(cudaGetLastError());
+  if ((rc = launch_tiles(dgrad_kernel, TILE_THREADS, sizeof(TileSmem), 2, 1, GD.tiles, s, dz, c->wb, a1, a2, d1, d2, GD)))
+    return rc;
+  WgradGrid GW = wgrad_grid(n, H, W, wait_of(kernels, QSL_CNN_WGRAD2));
+  if ((rc = launch_tiles(wgrad32_kernel, WG_THREADS, sizeof(WgradSmem<14>), 1, 1, GW.tiles, s, a1, d2, grad + OFF_W2,
+                         grad + OFF_B2, GW)))
+    return rc;
+  GW.wait_ns = wait_of(kernels, QSL_CNN_WGRAD13);
+  return launch_tiles(wgrad_io_kernel, WG_THREADS, sizeof(WgradSmem<1>), 1, 2, GW.tiles, s, x, d1, dz, a2, grad, GW);
+}
+
 }  // namespace
 
 extern "C" {
@@ -1294,47 +1354,30 @@ int qsl_cnn_params(const qsl_cnn* c, float* params) {
 }
 
 int qsl_cnn_forward(qsl_cnn* c, const float* x, int n, int H, int W, float* prob, void* stream_) {
-  cudaStream_t s = (cudaStream_t)stream_;
   if (!c || !x || !prob || !dims_ok(n, H, W)) {
     qsl::set_error("bad CNN forward arguments");
     return QSL_EINVAL;
   }
-  int dev = 0, sms = 0;
-  QSL_CHECK_CUDA(cudaGetDevice(&dev));
-  QSL_CHECK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const FwdGrid G = fwd_grid(n, H, W, 2 * sms);
-  return launch_tiles(forward_kernel, FWD_THREADS, sizeof(FwdSmem), 2, 1, G.groups, s, x, c->wb, c->w, prob, G);
+  return forward_pass(c, x, n, H, W, prob, 0, (cudaStream_t)stream_);
 }
 
 int qsl_cnn_loss_grad(qsl_cnn* c, const float* x, const float* y, int n, int H, int W, float pos_weight, float* loss,
                       float* grad, void* stream_) {
-  cudaStream_t s = (cudaStream_t)stream_;
   if (!c || !x || !y || !loss || !grad || !dims_ok(n, H, W) || !(pos_weight > 0)) {
     qsl::set_error("bad CNN loss/gradient arguments");
     return QSL_EINVAL;
   }
-  size_t P = (size_t)n * H * W;
-  int rc = ensure_act(c, P, s);
-  if (rc) return rc;
-  float *a1 = c->act, *a2 = a1 + P * 32, *d2 = a2 + P * 32, *d1 = d2 + P * 32, *z = d1 + P * 32, *dz = z + P;
-  QSL_CHECK_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), s));
-  QSL_CHECK_CUDA(cudaMemsetAsync(grad, 0, NPAR * sizeof(float), s));
-  const TileGrid GD = tile_grid(n, H, W, DW, DH);
-  if ((rc = launch_conv<C1, C2, true>(x, c->wb + OFF_W1, c->w + OFF_B1, a1, n, H, W, s))) return rc;
-  if ((rc = launch_conv<C2, C2, true>(a1, c->wb + OFF_W2, c->w + OFF_B2, a2, n, H, W, s))) return rc;
-  if ((rc = launch_conv<C2, 1, false>(a2, c->wb + OFF_W3, c->w + OFF_B3, z, n, H, W, s)))
-    return rc;
-  bce_kernel<<<(int)std::min<size_t>((P + BCE_THREADS - 1) / BCE_THREADS, 1024), BCE_THREADS, 0, s>>>(z, y, (int64_t)P, pos_weight, dz, loss,
-                                                                          grad + OFF_B3);
-  qsl::count_launch();
-  QSL_CHECK_CUDA(cudaGetLastError());
-  if ((rc = launch_tiles(dgrad_kernel, TILE_THREADS, sizeof(TileSmem), 2, 1, GD.tiles, s, dz, c->wb, a1, a2, d1, d2, GD)))
-    return rc;
-  const WgradGrid GW = wgrad_grid(n, H, W);
-  if ((rc = launch_tiles(wgrad32_kernel, WG_THREADS, sizeof(WgradSmem<14>), 1, 1, GW.tiles, s, a1, d2, grad + OFF_W2,
-                         grad + OFF_B2, GW)))
-    return rc;
-  return launch_tiles(wgrad_io_kernel, WG_THREADS, sizeof(WgradSmem<1>), 1, 2, GW.tiles, s, x, d1, dz, a2, grad, GW);
+  return loss_grad_pass(c, x, y, n, H, W, pos_weight, loss, grad, 0, (cudaStream_t)stream_);
+}
+
+int qsl_check_cnn_waits(qsl_cnn* c, const float* x, const float* y, int n, int H, int W, float* prob, float* loss,
+                        float* grad, int kernels, void* stream_) {
+  if (!c || !x || !y || !prob || !loss || !grad || !dims_ok(n, H, W)) {
+    qsl::set_error("bad CNN check arguments");
+    return QSL_EINVAL;
+  }
+  const int rc = forward_pass(c, x, n, H, W, prob, kernels, (cudaStream_t)stream_);
+  return rc ? rc : loss_grad_pass(c, x, y, n, H, W, 1.0f, loss, grad, kernels, (cudaStream_t)stream_);
 }
 
 int qsl_cnn_adam_step(qsl_cnn* c, const float* grad, float lr, float beta1, float beta2, float eps, void* stream_) {

@@ -105,21 +105,45 @@ __device__ __forceinline__ void bar_arrive(uint64_t* bar) {
 }
 __device__ __forceinline__ void bar_init_fence() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 
-// Waits for a barrier phase, for at most about a second; false if it did not
-// complete. Whole warps call it.
-__device__ __forceinline__ bool bar_wait(uint64_t* bar, uint32_t phase) {
+constexpr uint32_t WAIT_NS = 1000000000;  // limit of a wait: a second
+__device__ __forceinline__ unsigned long long clock_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+__device__ __forceinline__ bool bar_try(uint32_t bar, uint32_t phase) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(done)
+      : "r"(bar), "r"(phase)
+      : "memory");
+  return __all_sync(0xffffffffu, done);
+}
+// Waits for a barrier phase, for `limit` ns of the global timer (read every 16
+// attempts); false if it did not complete, and at once for a limit of 0. Whole
+// warps call it.
+__device__ __forceinline__ bool bar_wait(uint64_t* bar, uint32_t phase, uint32_t limit) {
+  if (limit == 0) return false;
   const uint32_t a = smem_addr(bar);
+  unsigned long long t0 = 0;
 #pragma unroll 1
-  for (int i = 0; i < (1 << 22); ++i) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(a), "r"(phase)
-        : "memory");
-    if (__all_sync(0xffffffffu, done)) return true;
+  for (;;) {
+#pragma unroll 1
+    for (int i = 0; i < 16; ++i)
+      if (bar_try(a, phase)) return true;
+    const unsigned long long t = __shfl_sync(0xffffffffu, clock_ns(), 0);
+    if (t0 == 0) t0 = t;
+    else if (t - t0 > limit) return false;
   }
-  return false;
+}
+// After a wait that ran out: the warp that issued MMAs waits for them all, so
+// that their operands and accumulators may be written and freed. `bar` is a
+// barrier of its own, in its first phase.
+__device__ __forceinline__ void drain(uint64_t* bar) {
+  if (elect()) commit(bar);
+  __syncwarp();
+  bar_wait(bar, 0, WAIT_NS);
 }
 
 // x as a sum of three BF16 values (exact: 24 significant bits in pieces of 8,

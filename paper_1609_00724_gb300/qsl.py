@@ -140,6 +140,7 @@ def lib():
     L.qsl_cnn_params.argtypes = [vp, vp]
     L.qsl_cnn_forward.argtypes = [vp, vp, i32, i32, i32, vp, vp]
     L.qsl_cnn_loss_grad.argtypes = [vp, vp, vp, i32, i32, i32, C.c_float, vp, vp, vp]
+    L.qsl_check_cnn_waits.argtypes = [vp, vp, vp, i32, i32, i32, vp, vp, vp, i32, vp]
     L.qsl_cnn_adam_step.argtypes = [vp, vp, C.c_float, C.c_float, C.c_float, C.c_float, vp]
     L.qsl_cnn_free.argtypes = [vp]
     L.qsl_cnn_features.argtypes = [vp, vp, i32, i32, i32, vp, vp]
@@ -301,6 +302,7 @@ def qsl_autotune(field, seeds, opts, stream=None):
 
 
 QSL_CNN_NPARAMS = 32 * 2 * 9 + 32 + 32 * 32 * 9 + 32 + 32 * 9 + 1
+QSL_CNN_FORWARD, QSL_CNN_DGRAD, QSL_CNN_WGRAD2, QSL_CNN_WGRAD13 = 1, 2, 4, 8
 
 
 def qsl_cnn_features(S, Q, X, stream=None):
@@ -345,6 +347,11 @@ class Cnn:
         n, c, h, w = x.shape
         _check(lib().qsl_cnn_loss_grad(self.handle, _ptr(x), _ptr(y), n, h, w, C.c_float(pos_weight), _ptr(loss),
                                        _ptr(grad), _stream(stream)))
+
+    def check_waits(self, x, y, prob, loss, grad, kernels, stream=None):
+        n, c, h, w = x.shape
+        _check(lib().qsl_check_cnn_waits(self.handle, _ptr(x), _ptr(y), n, h, w, _ptr(prob), _ptr(loss), _ptr(grad),
+                                         kernels, _stream(stream)))
 
     def adam(self, grad, lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8, stream=None):
         _check(lib().qsl_cnn_adam_step(self.handle, _ptr(grad), C.c_float(lr), C.c_float(beta1), C.c_float(beta2),
@@ -492,5 +499,5 @@ EXPORTS = ["qsl_opts_default", "qsl_load_field", "qsl_free_field", "qsl_trace_se
            "qsl_q_volume_3d", "qsl_fledge", "qsl_refine", "qsl_hilbert_encode", "qsl_hilbert_decode", "qsl_convert",
            "qsl_last_error", "qsl_last_stats", "qsl_trace_seeds_noalloc", "qsl_kernel_launches", "qsl_q_map_batch",
            "qsl_plan_q_map_batch", "qsl_plan_launch", "qsl_plan_stats", "qsl_plan_free", "qsl_autotune",
-           "qsl_cnn_create", "qsl_cnn_params", "qsl_cnn_forward", "qsl_cnn_loss_grad", "qsl_cnn_adam_step",
+           "qsl_cnn_create", "qsl_cnn_params", "qsl_cnn_forward", "qsl_cnn_loss_grad", "qsl_check_cnn_waits", "qsl_cnn_adam_step",
            "qsl_cnn_free", "qsl_cnn_nparams", "qsl_last_refine_stats", "qsl_trim_pool", "qsl_set_geometry"]
