@@ -546,7 +546,8 @@ __global__ void __launch_bounds__(CONV_THREADS) conv3x3_kernel(const float* __re
 // and a2; 32 x 64 x 64 pixels: 41 us.
 __global__ void __launch_bounds__(TILE_THREADS, 2)
     dgrad_kernel(const float* __restrict__ dz, const __nv_bfloat16* __restrict__ wb, const float* __restrict__ a1,
-                 const float* __restrict__ a2, float* __restrict__ d1, float* __restrict__ d2, const TileGrid G) {
+                 const float* __restrict__ a2, float* __restrict__ d1, float* __restrict__ d2, float* __restrict__ grad,
+                 const TileGrid G) {
   extern __shared__ __align__(16) unsigned char smem[];
   TileSmem& S = *reinterpret_cast<TileSmem*>(smem);
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -635,6 +636,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
     if (S.failed) break;
   }
   __syncthreads();
+  // the tiles that a block leaves out keep an earlier pass's d1 and d2: the
+  // gradients formed from them (layers 1 and 2) are marked as missing
+  if (S.failed)
+    for (int i = tid; i < OFF_W3; i += TILE_THREADS) atomicAdd(&grad[i], __int_as_float(0x7fc00000));
   if (warp == 0 && S.failed) umma::drain(&S.drained);
   if (warp == 0) umma::tmem_free(tmem, 256);
 }
@@ -1270,7 +1275,7 @@ int loss_grad_pass(qsl_cnn* c, const float* x, const float* y, int n, int H, int
                                                                           grad + OFF_B3);
   qsl::count_launch();
   QSL_CHECK_CUDA(cudaGetLastError());
-  if ((rc = launch_tiles(dgrad_kernel, TILE_THREADS, sizeof(TileSmem), 2, 1, GD.tiles, s, dz, c->wb, a1, a2, d1, d2, GD)))
+  if ((rc = launch_tiles(dgrad_kernel, TILE_THREADS, sizeof(TileSmem), 2, 1, GD.tiles, s, dz, c->wb, a1, a2, d1, d2, grad, GD)))
     return rc;
   WgradGrid GW = wgrad_grid(n, H, W, wait_of(kernels, QSL_CNN_WGRAD2));
   if ((rc = launch_tiles(wgrad32_kernel, WG_THREADS, sizeof(WgradSmem<14>), 1, 1, GW.tiles, s, a1, d2, grad + OFF_W2,

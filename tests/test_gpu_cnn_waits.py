@@ -66,3 +66,15 @@ def test_waits_that_run_out(setup, kernels, bad):
     assert np.array_equal(net.forward(x).cpu().numpy(), prob0)
     net.loss_grad(x, y, 1.0, loss, grad)
     _check(_blocks(grad), grad0, ())
+
+
+def test_missing_data_gradients_reach_both_layers(setup):
+    """The data gradients' kernel stops at its first tile: layer 2's gradients,
+    formed from buffers that still hold an earlier pass's values, are NaN like
+    layer 1's."""
+    qsl, net, x, other, y, (_, _, grad0) = setup
+    prob, loss = torch.zeros_like(y), torch.zeros(1, device="cuda")
+    grad = torch.zeros(qsl.QSL_CNN_NPARAMS, device="cuda")
+    net.loss_grad(other, y, 1.0, loss, grad)
+    net.check_waits(x, y, prob, loss, grad, qsl.QSL_CNN_DGRAD)
+    _check(_blocks(grad), grad0, ("w1", "b1", "w2", "b2"))
