@@ -352,7 +352,7 @@ typedef struct qsl_cnn qsl_cnn;
 int qsl_cnn_create(const float* params, qsl_cnn** out);
 /* Copies the FP32 master parameters to host memory. */
 int qsl_cnn_params(const qsl_cnn* cnn, float* params);
-/* prob[n][h][w] = sigmoid(logit) for x[n][2][h][w]. */
+/* prob[n][h][w] = sigmoid(logit) for x[n][2][h][w]; prob may overlap x. */
 int qsl_cnn_forward(qsl_cnn* cnn, const float* x, int n, int h, int w, float* prob, void* stream);
 /* Mean binary cross-entropy over pixels, pos_weight * y * softplus(-z) +
  * (1 - y) * softplus(z), and its gradient w.r.t. the parameters (device,

@@ -1145,15 +1145,13 @@ struct qsl_cnn {
   float* m = nullptr;            // Adam moments
   float* v = nullptr;
   int64_t steps = 0;
-  float* act = nullptr;          // activations of the largest batch seen
+  float* act = nullptr;          // activations of the largest batch seen (floats)
   size_t act_cap = 0;
 };
 
 namespace {
 
-int ensure_act(qsl_cnn* c, size_t pixels, cudaStream_t s) {
-  // a1, a2, d2, d1 (32 channels each), z, dz (1)
-  size_t need = pixels * (4 * 32 + 2);
+int ensure_act(qsl_cnn* c, size_t need, cudaStream_t s) {
   if (need <= c->act_cap) return QSL_OK;
   if (c->act) QSL_CHECK_CUDA(cudaFreeAsync(c->act, s));
   c->act = nullptr;
@@ -1261,7 +1259,7 @@ int forward_pass(qsl_cnn* c, const float* x, int n, int H, int W, float* prob, i
 int loss_grad_pass(qsl_cnn* c, const float* x, const float* y, int n, int H, int W, float pos_weight, float* loss,
                    float* grad, int kernels, cudaStream_t s) {
   size_t P = (size_t)n * H * W;
-  int rc = ensure_act(c, P, s);
+  int rc = ensure_act(c, P * (4 * 32 + 2), s);  // a1, a2, d2, d1 (32 channels each), z, dz
   if (rc) return rc;
   float *a1 = c->act, *a2 = a1 + P * 32, *d2 = a2 + P * 32, *d1 = d2 + P * 32, *z = d1 + P * 32, *dz = z + P;
   QSL_CHECK_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), s));
@@ -1363,7 +1361,16 @@ int qsl_cnn_forward(qsl_cnn* c, const float* x, int n, int H, int W, float* prob
     qsl::set_error("bad CNN forward arguments");
     return QSL_EINVAL;
   }
-  return forward_pass(c, x, n, H, W, prob, 0, (cudaStream_t)stream_);
+  cudaStream_t s = (cudaStream_t)stream_;
+  // prob may lie over x: blocks read and write at different times, so the pass
+  // then writes beside it
+  const size_t P = (size_t)n * H * W;
+  const uintptr_t xa = (uintptr_t)x, pa = (uintptr_t)prob;
+  if (pa >= xa + 2 * P * sizeof(float) || xa >= pa + P * sizeof(float)) return forward_pass(c, x, n, H, W, prob, 0, s);
+  int rc = ensure_act(c, P, s);
+  if (rc || (rc = forward_pass(c, x, n, H, W, c->act, 0, s))) return rc;
+  QSL_CHECK_CUDA(cudaMemcpyAsync(prob, c->act, P * sizeof(float), cudaMemcpyDeviceToDevice, s));
+  return QSL_OK;
 }
 
 int qsl_cnn_loss_grad(qsl_cnn* c, const float* x, const float* y, int n, int H, int W, float pos_weight, float* loss,
