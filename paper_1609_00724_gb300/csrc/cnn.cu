@@ -1104,7 +1104,7 @@ FwdGrid fwd_grid(int n, int H, int W, int slots, uint32_t wait_ns) {
     }
   }
   G.nseg = SP / G.P;
-  G.zw = (W + G.tx - 1) / G.tx;
+  G.zw = (int)(((int64_t)W + G.tx - 1) / G.tx);
   int64_t time = INT64_MAX;
   for (int ty = 1; ty <= std::min(H, 1024); ++ty) {
     const int h = (int)(((int64_t)H + ty - 1) / ty);
@@ -1112,7 +1112,7 @@ FwdGrid fwd_grid(int n, int H, int W, int slots, uint32_t wait_ns) {
     if (t < time) {
       time = t;
       G.h = h;
-      G.ty = (H + h - 1) / h;
+      G.ty = (int)(((int64_t)H + h - 1) / h);
     }
   }
   G.tasks = (int64_t)n * G.tx * G.ty;
@@ -1357,8 +1357,11 @@ int qsl_cnn_params(const qsl_cnn* c, float* params) {
 }
 
 int qsl_cnn_forward(qsl_cnn* c, const float* x, int n, int H, int W, float* prob, void* stream_) {
-  if (!c || !x || !prob || !dims_ok(n, H, W)) {
-    qsl::set_error("bad CNN forward arguments");
+  // a task may hang over the image by its rows (H / 1000 at these heights) or 128
+  // columns: coordinates stay 32-bit
+  constexpr int MAX_SIDE = INT32_MAX - (1 << 22);
+  if (!c || !x || !prob || !dims_ok(n, H, W) || H > MAX_SIDE || W > MAX_SIDE) {
+    qsl::set_error("bad CNN forward arguments (n h w at most 2^31, h and w at most 2^31 - 2^22 - 1)");
     return QSL_EINVAL;
   }
   cudaStream_t s = (cudaStream_t)stream_;

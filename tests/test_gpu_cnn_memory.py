@@ -24,3 +24,13 @@ def test_output_over_the_input(n, h, w, at):
     want = net.forward(x.clone().view(n, 2, h, w))
     got = net.forward(x.view(n, 2, h, w), x[at:at + n * h * w].view(n, h, w))
     assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("h,w", [(1, 2**31 - 1), (2**31 - 1, 1), (1, 2**31 - 2**22), (2**31 - 2**22, 1), (2**16, 2**16)])
+def test_sides_beyond_32_bit_coordinates_are_refused(h, w):
+    """Refused before anything is launched (the buffers here are small)."""
+    qsl, net = _net()
+    x = torch.zeros(64, device="cuda")
+    L = qsl.lib()
+    assert L.qsl_cnn_forward(net.handle, x.data_ptr(), 1, h, w, x.data_ptr(), None) == qsl.QSL_EINVAL
+    assert b"CNN forward" in L.qsl_last_error()
