@@ -494,12 +494,13 @@ struct TraceParams {
   long long max_steps;
   int euler;
   int refill_min;
-  unsigned long long timeout_ns;  // per-warp watchdog, 0 = none
+  unsigned long long timeout_ns;  // watchdog, counted by each warp; 0 = none
   int* timeout_flag;
   Cont* cont;                      // FP64 cell-wise launches: handed-over lines
   unsigned long long* cont_count;
   int handoff;                     // cell_kernel_f64: hand over a warp's lines at or below this many, 0 = never
   int cont_in;                     // cell_wide_kernel: trace the handed-over lines
+  unsigned long long* t0;          // with both: when the launch began, for the watchdog
   int64_t few;                     // ck_wide_kernel traces launches of at most this many units, trace_kernel the others
 };
 
@@ -1441,6 +1442,7 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
   int iter = 0;
   bool timed_out = false;
   const unsigned long long t_start = P.timeout_ns ? globaltimer() : 0ull;
+  if (F64 && P.timeout_ns && P.handoff > 0 && lane == 0) atomicCAS(P.t0, 0ull, t_start);
 
   for (;;) {
     if (!exhausted) {
@@ -2730,7 +2732,8 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
   unsigned long long c_stage = 0, c_acc = 0, c_rej = 0, c_land = 0, c_lines = 0;
   int iter = 0;
   bool timed_out = false;
-  const unsigned long long t_start = P.timeout_ns ? globaltimer() : 0ull;
+  // handed-over lines keep the clock of the launch that they began in
+  const unsigned long long t_start = !P.timeout_ns ? 0ull : (P.cont_in ? *P.t0 : globaltimer());
 
   for (;;) {
     if (!exhausted) {
@@ -4447,8 +4450,8 @@ size_t cont_offset(size_t n_units) {
   return (256 + sizeof(EndRec<R>) * (n_units ? n_units : 1) + 15) / 16 * 16;
 }
 
-// Scratch of one tracing launch: queue head, watchdog flag, continuation count
-// and queue head of the handed-over lines (32 bytes at offset 0), one end
+// Scratch of one tracing launch: queue head, watchdog flag, continuation count,
+// queue head of the handed-over lines and start time (40 bytes at offset 0), one end
 // record per unit from offset 256 and, FP64, the continuation records. `scratch` is
 // either caller-provided (no-allocation entry point, captured plans) or
 // allocated here.
@@ -4466,7 +4469,7 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
     QSL_CHECK_CUDA(qsl::alloc_async((void**)&scratch, scratch_bytes(sizeof(R) == 8 ? QSL_FP64 : QSL_FP32_MIXED, n_units), stream));
   unsigned long long* head = reinterpret_cast<unsigned long long*>(scratch);
   EndRec<R>* ends = reinterpret_cast<EndRec<R>*>(reinterpret_cast<unsigned char*>(scratch) + 256);
-  QSL_CHECK_CUDA(cudaMemsetAsync(head, 0, 32, stream));
+  QSL_CHECK_CUDA(cudaMemsetAsync(head, 0, 40, stream));
   TraceParams<R> P;
   P.item0 = item0;
   P.items = items_dev;
@@ -4487,6 +4490,7 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
   P.cont_count = head + 2;
   P.handoff = 0;
   P.cont_in = 0;
+  P.t0 = head + 4;
   P.few = -1;
   int threads = 32 * shape.warps_per_block;
   // persistent kernel: never launch more blocks than can be resident at once

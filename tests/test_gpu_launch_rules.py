@@ -1,0 +1,82 @@
+"""What a launch reports and does when the library chooses for the caller: the
+refill threshold (automatic, 1, 4, 8: the same bits), the resident blocks that a
+caller allows, the watchdog's one clock per launch."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1609_00724_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+U, V = (2.0, 0.0, 0.0), (0.0, 2.0, 0.0)
+
+
+@pytest.fixture(scope="module")
+def qsl():
+    from paper_1609_00724_gb300 import qsl as q
+    q.lib()
+    return q
+
+
+def _field(qsl, n, seed=5, mode=0):
+    gf = inputs.charge_field(inputs.random_charges(4, seed), n, dtype=torch.float32, device="cuda")
+    return qsl.qsl_load_field(gf.bx, gf.by, gf.bz, gf.xc, gf.yc, gf.zc, mode)
+
+
+def _map(qsl, F, m, o):
+    out = {"q": torch.empty(m * m, device="cuda"), "length": torch.empty(m * m, device="cuda"),
+           "faces": torch.empty(2 * m * m, dtype=torch.uint8, device="cuda"),
+           "status": torch.empty(m * m, dtype=torch.uint8, device="cuda")}
+    qsl.qsl_q_map_2d(F, (0, 0, 0), U, V, m, m, o, **out)
+    return out, qsl.qsl_last_stats()
+
+
+def test_handed_over_lines_keep_the_launch_clock(qsl):
+    """An FP64 cell-wise launch of 120,000 directions runs in two kernels of
+    comparable length (the second takes up the lines that the first hands over):
+    a watchdog of 40 to 80 percent of their time together stops it, whichever of
+    the two is running then."""
+    F = _field(qsl, 65, mode=1)
+    seeds = torch.as_tensor(inputs.random_seeds(60000, 43)).cuda()
+    o = qsl.qsl_opts_default(tol_abs=1e-11, tol_rel=1e-11, integrator=qsl.QSL_DOPRI5_CELL, precision=qsl.QSL_FP64)
+    for _ in range(2):
+        rec = qsl.lines_to_numpy(qsl.qsl_trace_seeds(F, seeds, o))
+        ms = qsl.qsl_last_stats()["kernel_ms"]
+    for part in (0.4, 0.5, 0.6, 0.7, 0.8):
+        o.timeout_s = part * ms * 1e-3
+        cut = qsl.lines_to_numpy(qsl.qsl_trace_seeds(F, seeds, o))
+        with pytest.raises(qsl.QslError) as e:
+            qsl.qsl_last_stats()
+        assert e.value.code == qsl.QSL_ETIMEOUT, part
+        late = (cut["status_f"] == qsl.QSL_LINE_TIMEOUT) | (cut["status_b"] == qsl.QSL_LINE_TIMEOUT)
+        assert late.any() and not late.all()
+        for k in ("q_perp", "length", "steps"):
+            assert np.array_equal(cut[k][~late], rec[k][~late], equal_nan=k != "steps"), k
+
+
+@pytest.mark.parametrize("integ,count", [(2, 4000), (0, 4000)])
+def test_watchdog_and_step_limit_with_sixteen_lanes(qsl, integ, count):
+    """Few lines in FP64 run on sixteen lanes each with either stepper: one
+    microsecond stops them after the next check (every 64 loop iterations), a step
+    limit at that many steps, and the next call runs to completion."""
+    F = _field(qsl, 65)
+    seeds = torch.as_tensor(inputs.random_seeds(count, 43)).cuda()
+    kw = dict(tol_abs=1e-9, tol_rel=1e-9, integrator=integ, precision=qsl.QSL_FP64)
+    rec = qsl.lines_to_numpy(qsl.qsl_trace_seeds(F, seeds, qsl.qsl_opts_default(**kw)))
+    qsl.qsl_last_stats()
+    cut = qsl.lines_to_numpy(qsl.qsl_trace_seeds(F, seeds, qsl.qsl_opts_default(timeout_s=1e-6, **kw)))
+    with pytest.raises(qsl.QslError) as e:
+        qsl.qsl_last_stats()
+    assert e.value.code == qsl.QSL_ETIMEOUT
+    st = np.concatenate([cut["status_f"], cut["status_b"]])
+    assert np.sum(st == qsl.QSL_LINE_TIMEOUT) > 100
+    assert np.all((st == qsl.QSL_LINE_TIMEOUT) | (st == qsl.QSL_LINE_OK))
+    few = qsl.lines_to_numpy(qsl.qsl_trace_seeds(F, seeds, qsl.qsl_opts_default(max_steps=30, **kw)))
+    qsl.qsl_last_stats()
+    st = np.concatenate([few["status_f"], few["status_b"]])
+    assert np.sum(st == qsl.QSL_LINE_MAXSTEPS) > 100
+    both = (few["status_f"] == qsl.QSL_LINE_MAXSTEPS) & (few["status_b"] == qsl.QSL_LINE_MAXSTEPS)
+    assert both.any() and np.all(few["steps"][both] == 60)
+    full = (few["status_f"] == qsl.QSL_LINE_OK) & (few["status_b"] == qsl.QSL_LINE_OK)
+    assert np.array_equal(few["steps"][full], rec["steps"][full])
