@@ -167,10 +167,9 @@ int default_shape(const qsl_opts* o, int tangent, int precision, LaunchShape* s)
     s->blocks_per_sm = w / s->warps_per_block;
     if (s->blocks_per_sm < 1) s->blocks_per_sm = 1;
   }
-  // idle lanes before a warp refills, unless asked for: 8 or, on launches of few
-  // lines, 1 (decided at the launch)
+  // idle lanes before a warp refills, unless asked for: set by the launch
   s->refill_auto = o->refill_min <= 0;
-  s->refill_min = o->refill_min > 0 ? o->refill_min : 8;
+  s->refill_min = o->refill_min > 0 ? o->refill_min : 1;
   s->line_lanes = o->line_lanes;
   return QSL_OK;
 }
@@ -399,9 +398,9 @@ int run_lines(const qsl_field* f, const SeedSource& src, int64_t S, const qsl_op
   if (rc) return rc;
   LaunchShape shape;
   default_shape(o, !o->length_only, o->precision, &shape);
-  g_last.shape = shape;
   g_last.lines = S;
   rc = trace_and_assemble(f, src, S, nullptr, cfg, o->precision, shape, out, stream, g_last.dev, &g_last.ev[0]);
+  g_last.shape = shape;
   if (rc) return rc;
   g_last.n_ev = 2;
   if (o->precision == QSL_FP32_MIXED && o->retrace_q > 0 && !o->length_only && S > 0) {

@@ -160,7 +160,7 @@ cudaError_t alloc_async(void** p, size_t bytes, cudaStream_t s);
 struct LaunchShape {
   int warps_per_block;
   int blocks_per_sm;
-  int refill_min;
+  int refill_min;  // idle lanes before a warp refills; set by the launch where refill_auto
   int line_lanes;  // cell-wise tracer: 1 or 3 lanes per line, 0 = auto
   int refill_auto; // refill_min was left to the library
 };
@@ -171,9 +171,10 @@ struct LaunchShape {
 // ev (optional): two events recorded around the tracer kernel. index
 // (optional, device): launch seed j traces seed index[j] (FP64 retrace lists).
 // scratch (optional, device): scratch_bytes(precision, 2 * n_seeds) bytes of
-// caller memory; allocated per call when null.
+// caller memory; allocated per call when null. shape.refill_min becomes the
+// threshold that the launch used.
 int trace_and_assemble(const qsl_field* f, const SeedSource& src, int64_t n_seeds, const int64_t* n_seeds_dev,
-                       const TraceConfig& cfg, int precision, const LaunchShape& shape, const LineOutputs& out,
+                       const TraceConfig& cfg, int precision, LaunchShape& shape, const LineOutputs& out,
                        cudaStream_t stream, DeviceStats* stats_dev, cudaEvent_t* ev, const int64_t* index = nullptr,
                        void* scratch = nullptr);
 size_t scratch_bytes(int precision, size_t n_units);

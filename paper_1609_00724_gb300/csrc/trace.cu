@@ -4457,7 +4457,7 @@ size_t cont_offset(size_t n_units) {
 // allocated here.
 template <class R, int NC>
 int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bool loc, const int64_t* index,
-                 int64_t n_seeds, const int64_t* n_seeds_dev, const TraceConfig& cfg, const LaunchShape& shape,
+                 int64_t n_seeds, const int64_t* n_seeds_dev, const TraceConfig& cfg, LaunchShape& shape,
                  const LineOutputs& out, cudaStream_t stream, DeviceStats* stats_dev, cudaEvent_t* ev,
                  void* scratch) {
   int dev = 0, sms = 0;
@@ -4580,8 +4580,9 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
   // 13.8, 14.2 ms; 512^2 Cash-Karp map at tol 1e-2 2.17, 1.90, 1.84, 1.83;
   // volume of 8.4 M seeds 392, 360, 361, 374. 1 and 8 on a launch of 1.4 times
   // the resident lanes: 1.18 and 1.22 ms.
-  P.refill_min = shape.refill_min > 0 ? shape.refill_min : 1;
-  if (shape.refill_auto && (coop || n_seeds_dev || 2 * n_seeds < 4 * (int64_t)blocks * threads)) P.refill_min = 1;
+  if (shape.refill_auto)
+    shape.refill_min = coop || n_seeds_dev || 2 * n_seeds < 4 * (int64_t)blocks * threads ? 1 : 8;
+  P.refill_min = shape.refill_min;
   if (ev) QSL_CHECK_CUDA(cudaEventRecord(ev[0], stream));
   if (n_seeds > 0) {
     if (ck_len) {
@@ -4668,7 +4669,7 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
 
 template <class R>
 int launch_any(const Item<R>& item0, const Item<R>* items_dev, int n_items, bool loc, const int64_t* index,
-               int64_t n_seeds, const int64_t* n_seeds_dev, const TraceConfig& cfg, const LaunchShape& shape,
+               int64_t n_seeds, const int64_t* n_seeds_dev, const TraceConfig& cfg, LaunchShape& shape,
                const LineOutputs& out, cudaStream_t stream, DeviceStats* stats_dev, cudaEvent_t* ev, void* scratch) {
   if (cfg.length_only)
     return launch_trace<R, 3>(item0, items_dev, n_items, loc, index, n_seeds, n_seeds_dev, cfg, shape, out, stream,
@@ -4680,7 +4681,7 @@ int launch_any(const Item<R>& item0, const Item<R>* items_dev, int n_items, bool
 }  // namespace
 
 int trace_and_assemble(const qsl_field* f, const SeedSource& src, int64_t n_seeds, const int64_t* n_seeds_dev,
-                       const TraceConfig& cfg, int precision, const LaunchShape& shape, const LineOutputs& out,
+                       const TraceConfig& cfg, int precision, LaunchShape& shape, const LineOutputs& out,
                        cudaStream_t stream, DeviceStats* stats_dev, cudaEvent_t* ev, const int64_t* index,
                        void* scratch) {
   bool loc = f->uniform != 0;

@@ -80,3 +80,29 @@ def test_watchdog_and_step_limit_with_sixteen_lanes(qsl, integ, count):
     assert both.any() and np.all(few["steps"][both] == 60)
     full = (few["status_f"] == qsl.QSL_LINE_OK) & (few["status_b"] == qsl.QSL_LINE_OK)
     assert np.array_equal(few["steps"][full], rec["steps"][full])
+
+
+@pytest.mark.parametrize("kw", [dict(integrator=2, tol_abs=1e-5, tol_rel=1e-5), dict(tol_abs=1e-2, tol_rel=1e-2)])
+def test_refill_threshold_is_reported_as_used(qsl, kw):
+    """900 x 900 seeds are far more than four times the resident lanes (at most 64
+    warps per SM), 60 x 60 far fewer. A line's result does not depend on when its
+    lane took it up: every threshold gives the same bits."""
+    F = _field(qsl, 33)
+    outs, used = [], []
+    for refill in (0, 1, 4, 8):
+        out, st = _map(qsl, F, 900, qsl.qsl_opts_default(refill_min=refill, retrace_q=0.0, **kw))
+        outs.append(out)
+        used.append(st["refill_min"])
+    assert used == [8, 1, 4, 8]
+    for out in outs[1:]:
+        for k in out:
+            assert torch.equal(out[k].view(torch.uint8), outs[0][k].view(torch.uint8)), k
+    o = qsl.qsl_opts_default(**kw)
+    _, st = _map(qsl, F, 60, o)
+    assert st["refill_min"] == 1
+    q = torch.empty(3600, device="cuda")
+    plan = qsl.Plan([(F, (0, 0, 0), U, V, 60, 60)], o, q=q, length=torch.empty_like(q),
+                    faces=torch.empty(7200, dtype=torch.uint8, device="cuda"),
+                    status=torch.empty(3600, dtype=torch.uint8, device="cuda"))
+    plan.launch()
+    assert plan.stats()["refill_min"] == 1
