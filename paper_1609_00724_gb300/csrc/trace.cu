@@ -16,6 +16,7 @@
 //
 // After the trace, one thread per seed reads both ends and assembles Q in
 // FP64 (Eq. finalQ and its footpoint/determinant forms).
+#include <algorithm>
 #include <cstdio>
 #include <type_traits>
 
@@ -4612,7 +4613,7 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
         TraceParams<R> Pw = P;
         Pw.head = head + 3;
         Pw.cont_in = 1;
-        launch_wide(Pw, sms * (res_w > 0 ? res_w : 1), threads, sms, stream);
+        launch_wide(Pw, sms * std::max(1, std::min(res_w, shape.blocks_per_sm)), threads, sms, stream);
         qsl::count_launch();
       }
     } else if (loc && cfg.geom == QSL_GEOM_SPHERICAL && cfg.interp_order > 1) {
@@ -4634,7 +4635,7 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
         if (n_seeds_dev || 2 * n_seeds <= P.few) {
           int res_w = 0;
           QSL_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res_w, ck_wide_kernel, threads, 0));
-          launch_ck_wide(P, sms * (res_w > 0 ? res_w : 1), threads, sms, stream);
+          launch_ck_wide(P, sms * std::max(1, std::min(res_w, shape.blocks_per_sm)), threads, sms, stream);
           qsl::count_launch();
           QSL_CHECK_CUDA(cudaGetLastError());
           one_lane = n_seeds_dev != nullptr;

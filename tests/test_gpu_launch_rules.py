@@ -106,3 +106,22 @@ def test_refill_threshold_is_reported_as_used(qsl, kw):
                     status=torch.empty(3600, dtype=torch.uint8, device="cuda"))
     plan.launch()
     assert plan.stats()["refill_min"] == 1
+
+
+@pytest.mark.parametrize("integ", [0, 2])
+def test_allowed_blocks_bound_the_sixteen_lane_kernels(qsl, integ):
+    """One resident block of one warp per SM against as many as fit: FP64 warp
+    instructions take 64 cycles of a warp and 19 of an SM, so four warps per SM and
+    more are at least twice as fast as one."""
+    F = _field(qsl, 65)
+    seeds = torch.as_tensor(inputs.random_seeds(4000, 43)).cuda()
+    ms = []
+    for blocks in (1, 0):
+        o = qsl.qsl_opts_default(tol_abs=1e-6, tol_rel=1e-6, integrator=integ, precision=qsl.QSL_FP64, warps_per_block=1,
+                                 blocks_per_sm=blocks)
+        best = np.inf
+        for _ in range(4):
+            qsl.qsl_trace_seeds(F, seeds, o)
+            best = min(best, qsl.qsl_last_stats()["kernel_ms"])
+        ms.append(best)
+    assert ms[0] > 1.6 * ms[1], ms
