@@ -4581,8 +4581,21 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
   // 13.8, 14.2 ms; 512^2 Cash-Karp map at tol 1e-2 2.17, 1.90, 1.84, 1.83;
   // volume of 8.4 M seeds 392, 360, 361, 374. 1 and 8 on a launch of 1.4 times
   // the resident lanes: 1.18 and 1.22 ms.
-  if (shape.refill_auto)
-    shape.refill_min = coop || n_seeds_dev || 2 * n_seeds < 4 * (int64_t)blocks * threads ? 1 : 8;
+  // Cash-Karp steps of the higher orders (27 and 64 vertices per stage, FP32 with
+  // the deviations) cost more than a refill, so that waiting pays only where lanes
+  // that take neighbouring seeds together share their cache lines: on fields of
+  // about 2^20 vertices (order 2) and 1.5 x 2^20 (order 3) and more. 1000^2 maps,
+  // thresholds 1 and 8, order 2: 64^3 12.3 and 14.1 ms, 88^3 16.3 and 16.3, 104^3
+  // 19.4 and 17.8, 256^3 48.7 and 32.7; order 3: 64^3 20.3 and 30.0, 112^3 36.8 and
+  // 41.0 (400^2: 8.6 and 8.5), 128^3 43.5 and 44.2 (400^2: 9.9 and 9.3), 160^3 57.1
+  // and 51.0, 256^3 97.7 and 70.6. In FP64, with Euler steps and for lengths only 8
+  // is the faster one at every size.
+  if (shape.refill_auto) {
+    const int64_t vertices = (int64_t)item0.F.n[0] * item0.F.n[1] * item0.F.n[2];
+    const bool dear = NC == 9 && sizeof(R) == 4 && cfg.integrator == QSL_RKCK54 && cfg.interp_order > 1 &&
+                      vertices < (cfg.interp_order == 2 ? 1 << 20 : 3 << 19);
+    shape.refill_min = coop || dear || n_seeds_dev || 2 * n_seeds < 4 * (int64_t)blocks * threads ? 1 : 8;
+  }
   P.refill_min = shape.refill_min;
   if (ev) QSL_CHECK_CUDA(cudaEventRecord(ev[0], stream));
   if (n_seeds > 0) {

@@ -125,3 +125,19 @@ def test_allowed_blocks_bound_the_sixteen_lane_kernels(qsl, integ):
             best = min(best, qsl.qsl_last_stats()["kernel_ms"])
         ms.append(best)
     assert ms[0] > 1.6 * ms[1], ms
+
+
+@pytest.mark.parametrize("order", [2, 3])
+def test_refill_rule_of_the_higher_orders(qsl, order):
+    """Cash-Karp with the deviations in FP32: no wait on a small field, where the
+    idle lanes cost more than the refills, 8 lanes on one that outgrows the caches."""
+    used = []
+    for n in (33, 120):
+        F, outs = _field(qsl, n), []
+        for refill in (0, 1, 8):
+            out, st = _map(qsl, F, 320, qsl.qsl_opts_default(refill_min=refill, retrace_q=0.0, interp_order=order))
+            outs.append(out)
+            used.append(st["refill_min"])
+        for k in outs[0]:
+            assert all(torch.equal(o[k].view(torch.uint8), outs[0][k].view(torch.uint8)) for o in outs[1:]), k
+    assert used == [1, 1, 8, 8, 1, 8]
