@@ -1168,15 +1168,23 @@ bool dims_ok(int n, int H, int W) { return n >= 1 && H >= 1 && W >= 1 && (int64_
 // (non-finite entries 0), channel 1 (log10 Q - 2) / 2 clamped to [-2, 3], a
 // missing Q (NaN) counted as the floor Q = 2 and an infinite one as the top
 // of the range.
-// A slice belongs to a cluster of 8 blocks that share its maximum.
-constexpr int FEAT_CLUSTER = 8, FEAT_THREADS = 512;
-__global__ void __cluster_dims__(FEAT_CLUSTER, 1, 1) __launch_bounds__(FEAT_THREADS)
+// A slice belongs to a cluster of CL blocks that share its maximum. Clusters are
+// placed at about 20 per us, a block goes over a slice at about 0.7 pixels per ns:
+// one block per slice for small slices and for many middling ones (one_block).
+// Slices x pixels, one block and 8 (and one block of the kernel before): 600 of
+// 32^2 6.2 and 32 us (6.2), 64 of 48^2 6.2 and 7.8 (6.2), 16 of 48^2 6.2 and 5.8,
+// 300 of 64^2 8.2 and 21 (10), 64 of 96^2 14 and 9.2, 300 of 128^2 35 and 29, 1,200
+// of 128^2 90 and 123, 150 of 256^2 227 and 59 (230).
+constexpr int FEAT_CLUSTER = 8;
+bool one_block(int slices, int64_t plane) { return plane <= 1024 || (plane <= 16384 && plane <= 40 * (int64_t)slices); }
+template <int CL, int THREADS>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS)
     features_kernel(const float* __restrict__ S, const float* __restrict__ Q, int64_t plane, float* __restrict__ X) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
-  __shared__ float red[FEAT_THREADS / 32], block_max;
-  const int z = blockIdx.x / FEAT_CLUSTER, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t first = (int64_t)cluster.block_rank() * FEAT_THREADS + threadIdx.x, step = FEAT_CLUSTER * FEAT_THREADS;
+  __shared__ float red[THREADS / 32], block_max;
+  const int z = blockIdx.x / CL, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t first = (int64_t)(CL > 1 ? cluster.block_rank() : 0) * THREADS + threadIdx.x, step = CL * THREADS;
   const float* s = S + (size_t)z * plane;
   const float* q = Q + (size_t)z * plane;
   float m = 0.0f;
@@ -1189,14 +1197,19 @@ __global__ void __cluster_dims__(FEAT_CLUSTER, 1, 1) __launch_bounds__(FEAT_THRE
   if (lane == 0) red[warp] = m;
   __syncthreads();
   if (warp == 0) {
-    m = lane < FEAT_THREADS / 32 ? red[lane] : 0.0f;
+    m = lane < THREADS / 32 ? red[lane] : 0.0f;
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) block_max = m;
   }
-  cluster.sync();
-  m = 0.0f;
-  for (int r = 0; r < FEAT_CLUSTER; ++r) m = fmaxf(m, *cluster.map_shared_rank(&block_max, r));
-  cluster.sync();  // no block leaves while another reads its maximum
+  if constexpr (CL > 1) {
+    cluster.sync();
+    m = 0.0f;
+    for (int r = 0; r < CL; ++r) m = fmaxf(m, *cluster.map_shared_rank(&block_max, r));
+    cluster.sync();  // no block leaves while another reads its maximum
+  } else {
+    __syncthreads();
+    m = block_max;
+  }
   const float smax = fmaxf(m, 1e-12f);
   float* x0 = X + (size_t)z * 2 * plane;
   float* x1 = x0 + plane;
@@ -1295,8 +1308,11 @@ int qsl_cnn_features(const float* S, const float* Q, int nz, int ny, int nx, flo
   const int64_t plane = (int64_t)ny * nx;
   constexpr int MAX_SLICES = 1 << 24;  // per launch
   for (int z = 0; z < nz; z += std::min(MAX_SLICES, nz - z)) {
-    features_kernel<<<std::min(MAX_SLICES, nz - z) * FEAT_CLUSTER, FEAT_THREADS, 0, (cudaStream_t)stream_>>>(
-        S + z * plane, Q + z * plane, plane, X + 2 * z * plane);
+    const int slices = std::min(MAX_SLICES, nz - z);
+    const bool one = one_block(slices, plane);
+    (one ? features_kernel<1, 256> : features_kernel<FEAT_CLUSTER, 512>)
+        <<<slices*(one ? 1 : FEAT_CLUSTER), one ? 256 : 512, 0, (cudaStream_t)stream_>>>(
+            S + z * plane, Q + z * plane, plane, X + 2 * z * plane);
     qsl::count_launch();
     QSL_CHECK_CUDA(cudaGetLastError());
   }
