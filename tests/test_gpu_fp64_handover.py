@@ -104,3 +104,29 @@ def test_maps_and_plans_repeat_bit_for_bit(qsl):
     qsl.qsl_q_map_2d(fields[0], (0, 0, 0), u, v, sizes[0], sizes[0], _opts(qsl, 1, 1e-7), **again)
     for k in again:
         assert torch.equal(again[k].view(torch.uint8), one[0][k].view(torch.uint8)), k
+
+
+@pytest.mark.parametrize("retrace_q,short", [(3.0, False), (200.0, True)])
+@pytest.mark.parametrize("integ", [0, 2])
+def test_retrace_lists_of_both_lengths(qsl, integ, retrace_q, short):
+    """FP32 maps whose FP64 retrace list is above 512 line directions per SM or below
+    it and not empty. Cell-wise: the same bits with one lane and with the library's
+    choice. Cash-Karp: the sixteen-lane kernel agrees to FP64 rounding."""
+    gf = inputs.charge_field(inputs.random_charges(4, 5), 33, dtype=torch.float32, device="cuda")
+    F = qsl.qsl_load_field(gf.bx, gf.by, gf.bz, gf.xc, gf.yc, gf.zc)
+    m, outs = 700, []
+    for lanes in (1, 0):
+        o = qsl.qsl_opts_default(integrator=integ, retrace_q=retrace_q, line_lanes=lanes)
+        if integ == 2:
+            o.tol_abs = o.tol_rel = 1e-6
+        outs.append(_map(m))
+        qsl.qsl_q_map_2d(F, (0, 0, 0), (2.0, 0.0, 0.0), (0.0, 2.0, 0.0), m, m, o, **outs[-1])
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        seeds = qsl.qsl_last_stats()["retraced"]
+        assert 0 < seeds <= 256 * sms if short else seeds > 256 * sms, seeds
+    for k in outs[0]:
+        a, b = outs[0][k], outs[1][k]
+        if integ == 2 or a.dtype == torch.uint8:
+            assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), k
+        else:
+            assert torch.allclose(a, b, rtol=1e-6, atol=0, equal_nan=True), k
