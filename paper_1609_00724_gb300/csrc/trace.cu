@@ -1095,17 +1095,15 @@ __device__ __forceinline__ bool gt_bits(double x, double thr) {
 __device__ __forceinline__ double min_bits(double x, double y) { return gt_bits(x, y) ? y : x; }  // x, y >= 0
 __device__ __forceinline__ double max_bits(double x, double y) { return gt_bits(x, y) ? x : y; }
 
-// a / b within two roundings: the hardware's approximate reciprocal (about 20
-// bits, not an FP64-pipe instruction), one Newton step and a corrected quotient,
-// 5 FP64 instructions. Where b or the quotient is near the ends of the range, and
-// for b = 0 and infinite a, the division.
+// a / b within two roundings for |b| from 2^-1022 to 2^1022: the hardware's
+// approximate reciprocal (about 20 bits, not an FP64-pipe instruction), one
+// Newton step and a corrected quotient, 5 FP64 instructions. A quotient that
+// overflows is NaN.
 __device__ __forceinline__ double quot(double a, double b) {
   double x;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(b));
   x = fma(fma(-b, x, 1.0), x, x);
   const double q = a * x;
-  const unsigned eb = (__double2hiint(b) & 0x7ff00000) - 0x01000000u, eq = __double2hiint(q) & 0x7ff00000;
-  if (eb > 0x7e000000u || eq == 0x7ff00000u) return a / b;
   return fma(fma(-b, q, a), x, q);
 }
 
@@ -1165,7 +1163,7 @@ __device__ __forceinline__ double wide_step(double h, double h_max, double room,
 // Time to the plane at the offset r along an axis with the velocity vel, `far`
 // (at least 0) when it never comes or comes later.
 __device__ __forceinline__ double plane_time(double r, double vel, double far) {
-  if (((__double2hiint(vel) & 0x7fffffff) | __double2loint(vel)) == 0) return far;
+  if ((__double2hiint(vel) & 0x7fffffff) < 0x01000000) return far;  // 0, or below 2^-1007
   const double q = quot(r, vel);
   return min_bits(far, __double2hiint(q) < 0 ? 0.0 : q);
 }
@@ -1174,9 +1172,10 @@ __device__ __forceinline__ double plane_time(double r, double vel, double far) {
 // next_step; most steps, cut at a cell face, are there.
 template <bool SKIP>
 __device__ __forceinline__ double err_ratio(double e, double size, double tol_abs, double tol_rel) {
-  const double sc = fma(tol_rel, size, tol_abs);
+  const double sc = max_bits(fma(tol_rel, size, tol_abs), 2.2250738585072014e-308);
   if (SKIP && __double2hiint(e) < __double2hiint(sc) - (13 << 20)) return 0.0;
-  return quot(e, sc);
+  const double q = quot(e, sc);
+  return __hiloint2double(__double2hiint(q) & 0x7fffffff, __double2loint(q));  // NaN: above everything for gt_bits
 }
 // Next step after a step hs with the error err (accepted up to 1): 0.9 hs times
 // err^(-1/4) and at least a fifth of it, or err^(-1/5) and at most five times.
