@@ -4440,10 +4440,12 @@ inline void launch_ck_wide(const TraceParams<float>&, int, int, int, cudaStream_
 // most handed over per launch (resident warps x kHandoff is below it).
 constexpr int kHandoff = 24;
 // Units per SM up to which the FP64 Cash-Karp launch takes sixteen lanes per
-// line. Measured on 128^3, one lane and sixteen: 32,400 seeds (426 per SM) at
-// tol 1e-2 11.9 and 7.7 ms, raw fields 14.5 and 12.7, at 1e-6 183 and 71;
-// 65,536 seeds 17.2 and 14.5, raw 20.8 and 23.7.
-constexpr int kCkWidePerSm = 512;
+// line. Measured on 128^3, one lane and sixteen: 36,100 seeds (475 per SM) at tol
+// 1e-2 10.5 and 10.4 ms (another field 12.2 and 9.6), at 1e-5 84 and 36. Raw fields
+// at tolerances where most stages are in a cell of their own (1e-3 and looser):
+// 25,200 seeds (332 per SM) 11.6 and 11.8 ms (13.2 and 10.9), 36,100 13.1 and 16.2
+// (14.8 and 14.7); at 1e-4 38,416 seeds 32.5 and 24.1, at 1e-5 127 and 78.
+constexpr int kCkWidePerSm = 512, kCkWidePerSmRaw = 352;
 constexpr size_t kContMax = 1 << 16;
 template <class R>
 size_t cont_offset(size_t n_units) {
@@ -4643,7 +4645,8 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
       // only, so both kernels are launched and one of them leaves at once.
       bool one_lane = true;
       if (sizeof(R) == 8 && NC == 9 && shape.line_lanes == 0 && !P.euler) {
-        P.few = (int64_t)kCkWidePerSm * sms;
+        const bool dear = item0.F.raw && cfg.tol_abs + cfg.tol_rel >= 1e-3;
+        P.few = (int64_t)(dear ? kCkWidePerSmRaw : kCkWidePerSm) * sms;
         if (n_seeds_dev || 2 * n_seeds <= P.few) {
           int res_w = 0;
           QSL_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res_w, ck_wide_kernel, threads, 0));

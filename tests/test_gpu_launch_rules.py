@@ -141,3 +141,17 @@ def test_refill_rule_of_the_higher_orders(qsl, order):
         for k in outs[0]:
             assert all(torch.equal(o[k].view(torch.uint8), outs[0][k].view(torch.uint8)) for o in outs[1:]), k
     assert used == [1, 1, 8, 8, 1, 8]
+
+
+def test_raw_cash_karp_maps_of_many_lines_take_one_lane(qsl):
+    """FP64 Cash-Karp on a raw field at a loose tolerance: 30,000 seeds (above 352
+    line directions per SM) run on one lane each, with the bits of line_lanes = 1;
+    20,000, and 30,000 at a tight tolerance, on sixteen (rounding apart; how far is
+    the lane tests' question)."""
+    F = _field(qsl, 33, mode=1)
+    for count, tol, same in ((30000, 1e-2, True), (20000, 1e-2, False), (30000, 1e-4, False)):
+        seeds = torch.as_tensor(inputs.random_seeds(count, 7)).cuda()
+        a, b = [qsl.lines_to_numpy(qsl.qsl_trace_seeds(F, seeds, qsl.qsl_opts_default(
+            tol_abs=tol, tol_rel=tol, precision=qsl.QSL_FP64, line_lanes=lanes))) for lanes in (1, 0)]
+        assert np.array_equal(a["face_f"], b["face_f"]) and np.array_equal(a["status_b"], b["status_b"])
+        assert np.array_equal(a["q_perp"], b["q_perp"], equal_nan=True) == same, count
