@@ -110,14 +110,18 @@ typedef struct qsl_opts {
   double retrace_q;        /* FP64 retrace threshold for QSL_FP32_MIXED; <= 0: never    */
   double domain_lo[3], domain_hi[3]; /* tracing box; lo >= hi on any axis: grid extent */
   double land_tol;         /* face landing tolerance in cells (FP32 stops at its resolution of the step) */
-  double timeout_s;        /* device watchdog per launch; <= 0: none                    */
-  int32_t line_lanes;      /* lanes per line of QSL_DOPRI5_CELL: 1 = one lane per line,
+  double timeout_s;        /* device watchdog per launch (trace, FP64 retrace); <= 0: none */
+  int32_t line_lanes;      /* lanes per line. QSL_DOPRI5_CELL: 1 = one lane per line,
                               3 = a group of three lanes (one per axis), 0 = auto (three
                               up to 512 line directions per SM, where a launch is bound
-                              by the latency of its longest lines; results agree to
-                              rounding). QSL_RKCK54 in FP64 on uniform Cartesian grids
-                              with trilinear interpolation: 1 or 3 = one lane, 0 = auto
-                              (sixteen lanes up to the same count)                       */
+                              by the latency of its longest lines; FP32 results agree to
+                              rounding). FP64 with the deviations: 3 = sixteen lanes, 0 =
+                              sixteen up to that count, above it one with the last lines
+                              of every warp on sixteen in a second kernel (results are the
+                              same bit for bit). QSL_RKCK54 in FP64 on uniform Cartesian
+                              grids with trilinear interpolation: 1 or 3 = one lane, 0 =
+                              sixteen up to that count (352 per SM for raw fields at
+                              tolerances of 1e-3 and more)                               */
   int32_t interp_order;    /* Sec. "Interpolation schemes": 1 (or 0) trilinear, 2 triquadratic
                               (Dodgson's interpolating quadratic, 27 vertices), 3 tricubic
                               (Keys cubic convolution, 64 vertices); 2 and 3 need a uniform

@@ -208,7 +208,7 @@ __device__ __forceinline__ void tile_of(const TileGrid& G, int64_t t, int w, int
 // leading pieces after the middle and last ones, the rest is FP32 addition.
 // Bound: shared memory, about 2,100 of the 2,350 cycles per row and SM (the
 // MMAs' operands half of it, layer 3's weights a quarter). 64 slices of 256 x
-// 256: 0.43 ms. Tiles of 32 x 12 pixels with N = 32 took 0.69 ms (54 MMAs of 59
+// 256: 0.42 ms. Tiles of 32 x 12 pixels with N = 32 took 0.69 ms (54 MMAs of 59
 // cycles per 128 pixels), FP32 kernels, one per layer, 5.6 ms. Eight warps on
 // layer 2's side instead of four: 0.58 against 0.51 ms at that stage (spills).
 constexpr int SP = 128, SPAD = SP + 8;      // pixels of a row step; the taps read two past them
@@ -475,8 +475,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 2)
 // had. A thread has two pixels (rows 8 apart of a 16 x 16 tile) and all output
 // channels, in pairs (fma.rn.f32x2 rounds each like fmaf); four weights per
 // shared-memory read. Bound: those reads (16 wavefronts per tap for 64 pixels)
-// and the multiply-adds alike. 32 x 64 x 64 pixels: a training step of 254 us (263
-// with the weights staged in their stored order, 32 lanes on one bank).
+// and the multiply-adds alike. 32 x 64 x 64 pixels: a training step of 259 us (9
+// more with the weights staged in their stored order, 32 lanes on one bank).
 constexpr int T = 16, TH = T + 2, CONV_THREADS = T * T / 2;
 template <int CIN, int COUT, bool RELU>
 __global__ void __launch_bounds__(CONV_THREADS) conv3x3_kernel(const float* __restrict__ x,
@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
   umma::fence_before();
   __syncthreads();
   umma::fence_after();
-  const uint32_t tmem = S.tmem, tq = tmem + ((uint32_t)(warp & 3) << 21);
+  const uint32_t tmem = S.tmem;
   uint32_t phase = 0;
   for (int64_t tile = blockIdx.x; tile < G.tiles; tile += gridDim.x, phase ^= 1) {
     int n, oy, ox;

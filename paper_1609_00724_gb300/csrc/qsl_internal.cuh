@@ -161,7 +161,7 @@ struct LaunchShape {
   int warps_per_block;
   int blocks_per_sm;
   int refill_min;  // idle lanes before a warp refills; set by the launch where refill_auto
-  int line_lanes;  // cell-wise tracer: 1 or 3 lanes per line, 0 = auto
+  int line_lanes;  // qsl_opts.line_lanes
   int refill_auto; // refill_min was left to the library
 };
 

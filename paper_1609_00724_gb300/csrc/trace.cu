@@ -1979,10 +1979,15 @@ __device__ __forceinline__ void cell_trace(const TraceParams<R>& P) {
 }
 
 // The cell-wise kernel. FP64 is bound by the FP64 pipe (19 cycles per SM and
-// warp instruction): with the controller, the plane tests and the crossing
-// search off it, about 1,000 FP64 instructions per warp step against 1,800
-// (FP64 map of 82,497 seeds on 128^3: 45.0 -> 29.6 ms, with the hand-over of
-// the last lines 20.6 ms). FP32: at most 168 registers, so three blocks of 128
+// warp instruction, 79 % busy; most of the rest waits for instructions, of which a
+// step has too many for the caches): with comparisons, divisions, powers and the
+// first search for a crossing off it, about 1,140 FP64 instructions per warp step
+// against 1,800. FP64 maps of 82,497 seeds on 128^3, two fields: 34.8 and 43.4 ms
+// before, 26.7 and 31.9, with the hand-over of the last lines 25.6 and 21.5 (raw
+// fields 48.0 and 60.0, 35.9 and 41.9, 39.2 and 35.0). FP32 norms and step sizes
+// would save 12 %, but not serve FP64's range, and arithmetic of each kernel's own
+// 4 %, but results would then depend on the scheduling (see the sums above
+// wide_step). FP32: at most 168 registers, so three blocks of 128
 // threads stay resident per SM (the allocation granularity would make 170 a
 // two-block kernel); FP64 keeps the compiler's choice (a cap would spill).
 // ITEMS: the problem comes from the launch's table; without one it is read from
@@ -2512,19 +2517,19 @@ __global__ void __launch_bounds__(256) cell_coop_kernel(const __grid_constant__ 
 // one component. Lane 4c + j of a group: axis c; j = 0 the position x_c,
 // j = 1, 2 component c of deviation j, j = 3 no state. For a stage derivative
 // it evaluates, as one bilinear polynomial (3 FMAs), d b_c / d u_j for j < 3
-// and b_c on the cell's lower x face for j = 3; three more FMAs after shuffles
+// and b_c on the cell's lower z face for j = 3; three more FMAs after shuffles
 // give value or gradient times deviation. Lanes 12..15 repeat lanes 8..11.
-// Comparisons use bit patterns; the step controller, the error norm and the
-// crossing search FP32 (cross_root), as in cell_trace. Deviations are carried
-// in cell units. One line per warp while there are warps (the first lines go
-// to one warp per SM, then to the other schedulers), else two; three lines of
-// ten lanes per warp, one more polynomial in the position lanes, measured no
-// faster (29.5 against 29.9 ms for 165 k line directions).
-// About 165 FP64 instructions per step against 865 of the three-lane kernel it
-// replaced: 7.0 against 25.6 us per step of a lone line; 64 seeds of a map on
-// 128^3 1.6 ms (6.8 ms on one lane per line).
-// End record of a group: lane (c, j) writes axis c of the end
-// point (j = 0) or of deviation j, the group's first lane the rest.
+// Comparisons use bit patterns, quotients quot, the crossing search starts in
+// FP32 (cross_root), all as in cell_trace. Deviations are carried in cell units.
+// One line per warp while there are warps (the first lines go to one warp per SM,
+// then to the other schedulers), else two; three lines of ten lanes per warp, one
+// more polynomial in the position lanes, measured no faster (29.5 against 29.9 ms
+// for 165 k line directions).
+// About 175 FP64 instructions per step against 865 of the three-lane kernel it
+// replaced: 7.4 against 23 us per step of a lone line (34 us on one lane); 64 seeds
+// of a map on 128^3 2.4 ms (7.7; on one lane 11).
+// End record of a group: lane (c, j) writes axis c of the end point (j = 0) or of
+// deviation j, the group's first lane the rest.
 __device__ __forceinline__ void write_end_wide(const TraceParams<double>& P, const Item<double>* E, int64_t unit,
                                                int c, int j, bool writer, double y, const int* ic, double hhc,
                                                double mu, int face, int status, int steps) {
@@ -2784,17 +2789,17 @@ __global__ void __launch_bounds__(256) cell_wide_kernel(const __grid_constant__ 
 #pragma unroll
               for (int a = 0; a < 3; ++a) ic[a] = k->ic[a];
             } else {
-            mu = 0;
-            muc = 0;
-            steps = 0;
-            zc = 0;
-            int lface;
-            const int status = wide_start(E, xd, sgn, c, j, ihc, ic, &y, &lface);
-            h = E->h_init;
-            if (status != ST_RUNNING) {
-              write_end_wide(P, E, unit, c, j, writer, y, ic, hhc, R(0), lface, status, 0);
-              active = false;
-            }
+              mu = 0;
+              muc = 0;
+              steps = 0;
+              zc = 0;
+              int lface;
+              const int status = wide_start(E, xd, sgn, c, j, ihc, ic, &y, &lface);
+              h = E->h_init;
+              if (status != ST_RUNNING) {
+                write_end_wide(P, E, unit, c, j, writer, y, ic, hhc, R(0), lface, status, 0);
+                active = false;
+              }
             }
           }
         }
@@ -4434,9 +4439,11 @@ inline void launch_ck_wide(const TraceParams<float>&, int, int, int, cudaStream_
 
 // A warp of cell_kernel_f64 hands its lines to cell_wide_kernel once the queue
 // is empty and at most kHandoff of them are left: on one lane each the last
-// lines take 25 us per step, on sixteen 7. Measured (FP64 map of 82,497 seeds
-// on 128^3; never, 8, 12, 16, 24, 32 lines): 29.6, 23.9, 22.2, 20.8, 20.6,
-// 20.4 ms; 196,608 seeds: 44.6, 36.4, 34.1, 33.9, 34.1, 34.0 ms. kContMax: the
+// lines take 34 us per step, on sixteen 7. Measured (FP64 maps of 82,497 seeds on
+// 128^3, ms; never, 4, 8, 12, 16, 24 lines): 31.8, 29.6, 27.4, 25.0, 23.8, 21.6, raw
+// 42.3, 41.0, 39.0, 36.6, 36.7, 34.2; the field it suits least 26.5, 25.1, 24.1,
+// 23.7, 24.4, 25.5, raw 35.4, 34.7, 33.2, 34.2, 35.5, 39.6; 197,136 seeds 49.6, 46.1,
+// 44.9, 43.0, 40.5, 38.5 and 49.7, 48.4, 47.0, 46.2, 46.1, 46.1. kContMax: the
 // most handed over per launch (resident warps x kHandoff is below it).
 constexpr int kHandoff = 24;
 // Units per SM up to which the FP64 Cash-Karp launch takes sixteen lanes per
@@ -4531,8 +4538,9 @@ int launch_trace(const Item<R>& item0, const Item<R>* items_dev, int n_items, bo
       // where the launch is bound by the latency of its longest lines rather
       // than by issue rate (measured crossover on GB300: about 640 per SM);
       // FP64 with the deviations: sixteen lanes per line up to the same count
-      // (32,000 seeds of a map on 128^3: 13.0 ms, one lane with the hand-over
-      // 13.4; 82,497 seeds 29.1 and 20.6); a device-side count is a retrace
+      // (maps on 128^3 of two fields, ms, and one lane with the hand-over: 34,200
+      // seeds 16.3 and 14.5, 17.0 and 14.3; 42,000 19.6 and 17.2, 18.3 and 17.4;
+      // 82,497 36.7 and 31.6, 25.5 and 21.6); a device-side count is a retrace
       // list, short by construction
       coop = n_seeds_dev != nullptr || 2 * n_seeds <= (int64_t)512 * sms;
     }
