@@ -4402,9 +4402,13 @@ Item<R> make_item(const qsl_field* f, const SeedSource& src, const TraceConfig& 
     it.inv_h_d[a] = f->h[a] > 0 ? 1.0 / f->h[a] : 0.0;
     it.lo_d[a] = cfg.lo[a];
     it.hi_d[a] = cfg.hi[a];
-    // the local frame measures positions in grid-index units
-    it.lo[a] = loc ? (R)((cfg.lo[a] - f->org[a]) / f->h[a]) : (R)cfg.lo[a];
-    it.hi[a] = loc ? (R)((cfg.hi[a] - f->org[a]) / f->h[a]) : (R)cfg.hi[a];
+    // the local frame measures positions in grid-index units; the grid's own edges
+    // are 0 and n - 1 exactly (the quotient may round above n - 1, for 50 vertices
+    // over a length of 2 for instance: an FP64 cell-wise line then took the last
+    // cell's face for an inner one and stayed there until its step limit)
+    it.lo[a] = !loc ? (R)cfg.lo[a] : cfg.lo[a] == f->glo[a] ? R(0) : (R)((cfg.lo[a] - f->org[a]) / f->h[a]);
+    it.hi[a] = !loc ? (R)cfg.hi[a]
+                    : cfg.hi[a] == f->ghi[a] ? R(f->n[a] - 1) : (R)((cfg.hi[a] - f->org[a]) / f->h[a]);
   }
   it.max_len = (R)cfg.max_len;
   it.h_init = (R)(cfg.h_init * cfg.cell);

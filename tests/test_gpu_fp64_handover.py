@@ -130,3 +130,17 @@ def test_retrace_lists_of_both_lengths(qsl, integ, retrace_q, short):
             assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), k
         else:
             assert torch.allclose(a, b, rtol=1e-6, atol=0, equal_nan=True), k
+
+
+@pytest.mark.parametrize("n", [50, 99])
+def test_lines_leave_through_every_face(qsl, n):
+    """Grids whose length over their spacing rounds to more than n - 1: every line
+    ends on a face within some hundred steps (one or two per cell crossed), whether
+    the domain is left to the library or given as the grid's extent."""
+    F = _field(qsl, n, 0)
+    seeds = torch.as_tensor(inputs.random_seeds(3000, n)).cuda()
+    for lanes in (1, 3):
+        for kw in ({}, {"domain_lo": (-1.0, -1.0, 0.0), "domain_hi": (1.0, 1.0, 1.0)}):
+            rec = qsl.lines_to_numpy(qsl.qsl_trace_seeds(F, seeds, _opts(qsl, lanes, 1e-6, max_steps=2000, **kw)))
+            assert np.all(rec["status_f"] == qsl.QSL_LINE_OK) and np.all(rec["status_b"] == qsl.QSL_LINE_OK)
+            assert {1, 3, 5} <= set(rec["face_f"]) | set(rec["face_b"])
